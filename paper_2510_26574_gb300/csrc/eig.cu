@@ -324,10 +324,12 @@ __global__ void k_lift_panel(const double* __restrict__ Y, int r, int ldyp, doub
     }
 }
 
+// The plane cutter reads F element by element, so any layout goes to the tensor
+// cores; only the per-tile slicing variant loads F itself by TMA.
 static bool oz_lift_enabled(const double* F, int64_t ldf, int64_t N) {
     const char* e = getenv("KEVD_LIFT");
     if (e && e[0] == 'f') return false;                       // KEVD_LIFT=fp64: the FP64-pipe GEMM
-    return N < ((int64_t)1 << 31) && ozgemm_layout_ok(F, ldf);
+    return N < ((int64_t)1 << 31) && (!(e && e[0] == 's') || ozgemm_layout_ok(F, ldf));
 }
 
 // Row maxima of |F(i, :r)| (F column-major, FP64 or FP32) as doubles; the FP64
@@ -455,7 +457,7 @@ static char lift_mode() {
 }
 
 // U = diag(1/rowdiv) F Y with FP64 F: the FP64-accurate tensor-core product
-// (ozgemm.cu) when F's layout allows, else the FP64-pipe GEMM.
+// from planes, or the FP64-pipe GEMM under KEVD_LIFT=fp64.
 static cudaError_t lift_fp64(int64_t N, int k, int r, const double* F, int64_t ldf, const double* Y, double* U,
                              const double* rowdiv, const EigWs& w, cudaStream_t s) {
     if (!oz_lift_enabled(F, ldf, N)) {

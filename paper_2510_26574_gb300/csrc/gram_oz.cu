@@ -21,19 +21,19 @@
 // levels 4 and 5 would not do: the tensor core truncates each addend to the
 // accumulator's ulp, a bias that reaches ~2^-48 of the total over a chunk.
 //
-// Accumulation.  After every 256-row chunk the drain turns levels 0-4 into one
-// integer I_0 2^24 + I_1 2^16 + I_2 2^8 + I_3 + floor(I_4 / 2^8) (I_g = L_g
-// 2^(8 g), exact FP32-to-integer conversions) added to an INT64 running sum,
-// and the rest of level 4 (I_4 mod 2^8, times 2^-32) and level 5 into an FP32
-// running sum.  The column scales 2^(E_u + E_v - 12) and the conversion to
-// FP64 are applied once per CTA, and the partials of row splits and slabs are
-// added in FP64.
+// Accumulation.  After every 256-row chunk the drain adds levels 0-4 (exact integers)
+// to an INT64 running sum in units of 2^-32 and level 5 to an FP32 one.  The column
+// scales 2^(E_u + E_v - 12) and the conversion to FP64 are applied once per CTA, and
+// the partials of row splits and slabs are added in FP64.
+//
+// Seven digits (T below 2^54, 28 pairs with s + t <= 6, levels 5 and 6 in the seventh
+// accumulator) serve the layouts of F that are not 16-byte aligned (oz_gram_digits).
 //
 // Layout.  The rows are taken in slabs sized so that the digit planes of one
 // slab stay within a fixed budget.  k_oz_planes cuts a slab once: for each of
-// U, wa F (and wc F) six planes of rank_pad columns x S rows of BF16, a
+// U, wa F (and wc F) D planes of rank_pad columns x S rows of BF16, a
 // column's rows contiguous, so that a TMA box of 32 rows x 128 (or 64) columns
-// x 6 planes with the 64-byte swizzle lands as six K-major MMA operands of two
+// x D planes with the 64-byte swizzle lands as D K-major MMA operands of two
 // 16-row quarters (64-byte rows: half as many L2 requests per byte as 32-byte
 // rows).  Every tile of the Gram reads those planes instead of cutting
 // FP64 data itself (the cutting, not the MMAs, bounded the rate when each CTA
@@ -41,42 +41,55 @@
 //
 // Per CTA of k_gram_oz: one tile of M = 128 columns of the I block by N = 64
 // columns of the J block, for one Gram and one range of rows of the slab:
-//   * lane 0 of warp 0 keeps a three-stage ring of 32-row stages filled (two
-//     TMA loads per stage: 48 KB of U planes, 24 KB of V planes);
-//   * lane 0 of warp 1 issues the 21 UMMAs of each quarter, frees a stage by a
-//     commit, and at the end of each 256-row chunk commits to the drain and
-//     waits for it before the next chunk overwrites the accumulators;
+//   * lane 0 of warp 0 keeps a ring of 32-row stages filled (two TMA loads per stage:
+//     48 KB of U planes, 24 KB of V planes, three stages; 56 + 28 KB, two, with
+//     seven digits);
+//   * warp 1 issues the UMMAs (oz_mma.cuh: planes of U kept in the collector buffer,
+//     the last stage of a chunk accumulator by accumulator), frees a stage by a
+//     commit, and waits for the drain before the next chunk overwrites the
+//     accumulators;
 //   * warps 2-17 drain (TMEM lane quarter w % 4, tile columns [16 h, 16 h + 16)
 //     with h = (w - 2) / 4) and finally add the tile's FP64 partial.
+// Bound: shared memory, 102 KB of operand reads and TMA writes per quarter = 800
+// cycles, beside 735 of MMA issue.  Measured at N = 262,144, rank 1,101: both Grams
+// 11.8 ms (17.9 ms with one reading of U's plane per MMA and the drain after the last
+// MMA of a chunk).  At N = 60,001, rank 401 (odd: seven digits) 0.71 ms, against
+// 25.9 ms on the FP64 pipe.
 // Every wait is bounded (about one second); on a timeout the CTA sets bit 2 of
 // flags, waits (bounded) for its own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "common.cuh"
 #include "gram_tc.cuh"
+#include "oz_mma.cuh"
 #include "tc_ptx.cuh"
 
 namespace kevd {
 
 constexpr int kOzQ = 16;          // rows per quarter (one MMA K step)
 constexpr int kOzSQ = 2;          // quarters per stage (one 64-byte swizzled row of K)
-constexpr int kOzStages = 3;      // stages in flight
-constexpr int kOzChunk = 16;      // quarters per exact chunk: 256 rows
-constexpr int kOzDigits = 6;
+constexpr int kOzChunkSt = 8;     // stages per exact chunk: 256 rows
 constexpr int kOzDrainWarps = 16;
 constexpr int kOzThreads = (2 + kOzDrainWarps) * 32;
 constexpr int kOzM = 128, kOzN = 64;
 constexpr uint32_t kOzPlaneU = kOzM * 64;               // one digit plane of a stage: 128 columns x 64 bytes
 constexpr uint32_t kOzPlaneV = kOzN * 64;               // 4 KB
-constexpr uint32_t kOzStageU = kOzDigits * kOzPlaneU;   // 48 KB
-constexpr uint32_t kOzStage = kOzStageU + kOzDigits * kOzPlaneV;   // 72 KB
 constexpr uint32_t kOzCols = 512;                       // TMEM: 7 accumulators x 64 columns (allocation: 512)
-constexpr size_t kOzSmem = (size_t)kOzStages * kOzStage + 1024;
 constexpr size_t kOzPlaneBudget = (size_t)6 << 30;      // bytes of digit planes per slab
-static_assert(kOzSmem <= 227 * 1024, "shared memory");
+
+// Per digit count D: one stage (72 KB at six digits, 84 KB at seven) and the ring depth.
+template <int D>
+struct OzGramCfg {
+    static constexpr uint32_t kStageU = D * kOzPlaneU;
+    static constexpr uint32_t kStage = kStageU + D * kOzPlaneV;
+    static constexpr int kStages = D == 6 ? 3 : 2;
+    static constexpr size_t kSmem = (size_t)kStages * kStage + 1024;
+    static_assert(kSmem <= 227 * 1024, "shared memory");
+};
 
 // Tile t -> (I, J) over I-blocks of 128 columns and J-blocks of 64 columns
 // with J >= 2 I (the tiles holding some entry a <= c).
@@ -98,46 +111,14 @@ int oz_ntiles(int rank) {
     return n;
 }
 
-// The six digit planes of 2 consecutive values of one column: p_s = d_s 2^(-8 s)
-// as BF16, packed two rows per 32-bit word (plane s in w[s]).  sh0 = 1029 + E, so
-// that T = round(x 2^(46 - E)), |T| < 2^46.  The balanced digits are the bytes of
-// T + 0x808080808080 minus 128 (T + C lies in [0, 2^48), and T = sum (b - 128)
-// 256^j exactly); BF16 of d 2^(-8 s) comes from the magic M_s = 1.5 * 2^(23 - 8 s),
-// whose ulp is 2^(-8 s): float(bits(M_s) + d) - M_s = d 2^(-8 s), at most 8
-// significant bits, so the upper half of the word is the exact BF16.
-static __device__ __forceinline__ void oz_digits2(double x0, double x1, int sh0, uint32_t (&w)[kOzDigits]) {
-    unsigned long long U[2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const double x = u ? x1 : x0;
-        const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-        const int e = (int)((b >> 52) & 0x7FF);
-        const int sh = sh0 - e;                                   // >= 7 since |x| < 2^E
-        long long T = 0;
-        if (e != 0 && e != 0x7FF && sh >= 1 && sh < 62) {
-            const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-            T = (long long)(((m >> (sh - 1)) + 1) >> 1);          // round half up on |x| 2^(46 - E)
-            T = T < 0x3FFFFFFFFFFFll ? T : 0x3FFFFFFFFFFFll;      // |x| rounding up to 2^E
-            if ((long long)b < 0) T = -T;
-        }
-        U[u] = (unsigned long long)(T + 0x808080808080ll);
-    }
-#pragma unroll
-    for (int s = 0; s < kOzDigits; ++s) {
-        const int bi = kOzDigits - 1 - s;                         // plane 0 is the most significant byte
-        const float Ms = 1.5f * __int_as_float((150 - 8 * s) << 23);
-        const uint32_t mb = __float_as_uint(Ms) - 128u;
-        const float f0 = __fsub_rn(__uint_as_float(mb + (uint32_t)((U[0] >> (8 * bi)) & 255u)), Ms);
-        const float f1 = __fsub_rn(__uint_as_float(mb + (uint32_t)((U[1] >> (8 * bi)) & 255u)), Ms);
-        w[s] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
-    }
-}
-
-// Digit planes of the slab of rows [row0, row0 + rows) (rows a multiple of 16;
+// D-digit planes of the slab of rows [row0, row0 + rows) (rows a multiple of 16;
 // zero past N and past rank): set 0 from F, set 1 from wa F, set 2 from wc F
 // (when wc is given).  Plane (set, s) is rank_pad x S BF16 pairs, word
-// ((set 6 + s) rank_pad + c) S / 2 + i / 2 holding rows i, i + 1 of column c.
-// Block: 8 warps = 8 columns; a warp takes 64 rows per step (a lane two).
+// ((set D + s) rank_pad + c) S / 2 + i / 2 holding rows i, i + 1 of column c.
+// Block: 8 warps = 8 columns; a warp takes 64 rows per step (a lane two, as one
+// 16-byte vector when the column is 16-byte aligned, else as two 8-byte loads:
+// any F and ldf are cut, so the FP64-pipe kernel is not needed for odd ones).
+template <int D>
 __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F, int64_t ldf, int64_t N, int rank,
                                                    int rank_pad, int64_t row0, int rows, int S,
                                                    const double* __restrict__ wa, const double* __restrict__ wc,
@@ -148,24 +129,23 @@ __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F,
     const bool on = c < rank;
     const size_t plane = (size_t)rank_pad * (S / 2);
     const int sets = wc ? 3 : 2;
-    int sh[3];
+    int E[3];
 #pragma unroll
-    for (int z = 0; z < 3; ++z) {
-        const int e = (on && z < sets) ? Ecol[z * rank + c] : -900;
-        sh[z] = e > -900 ? 1029 + e : 4096;
-    }
+    for (int z = 0; z < 3; ++z) E[z] = (on && z < sets) ? Ecol[z * rank + c] : -900;
     const double* col = F + (int64_t)c * ldf;
+    const bool vec = (reinterpret_cast<uintptr_t>(col) & 15) == 0;   // row0 is even
     for (int it = 0; it < 8; ++it) {
         const int il = blockIdx.y * 512 + it * 64 + 2 * lane;
         if (il >= rows) break;
         const int64_t i = row0 + il;
         double x0 = 0.0, x1 = 0.0;
-        if (on && i + 1 < N) {
+        if (on && vec && i + 1 < N) {
             const double2 v = *reinterpret_cast<const double2*>(col + i);
             x0 = v.x;
             x1 = v.y;
         } else if (on && i < N) {
             x0 = col[i];
+            if (i + 1 < N) x1 = col[i + 1];
         }
         const size_t at = (size_t)c * (S / 2) + (il >> 1);
 #pragma unroll
@@ -177,27 +157,29 @@ __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F,
                 y0 = i < N ? __dmul_rn(w[i], x0) : 0.0;
                 y1 = i + 1 < N ? __dmul_rn(w[i + 1], x1) : 0.0;
             }
-            uint32_t wd[kOzDigits];
-            oz_digits2(y0, y1, sh[z], wd);
+            uint32_t wd[D];
+            oz_planes2<D>(oz_T_f64<D>(y0, E[z]), oz_T_f64<D>(y1, E[z]), wd);
 #pragma unroll
-            for (int s = 0; s < kOzDigits; ++s) P[(size_t)(z * kOzDigits + s) * plane + at] = wd[s];
+            for (int s = 0; s < D; ++s) P[(size_t)(z * D + s) * plane + at] = wd[s];
         }
     }
 }
 
-__device__ __forceinline__ int oz_acc(int lv, int s) { return lv < 4 ? lv : lv == 4 ? (s <= 2 ? 4 : 5) : 6; }
-
 // One tile (I, J) of Gram blockIdx.z over rows [blockIdx.y per, + per) of the
 // slab's planes (rows of the slab: `rows`); the FP64 result is stored into
 // (accumulate = 0) or added to (accumulate = 1) its partial in gpart.
+template <int D>
 __global__ void __launch_bounds__(kOzThreads, 1)
     k_gram_oz(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmVA,
               const __grid_constant__ CUtensorMap tmVC, const int* __restrict__ Ecol, int rank, int rows, int nbi,
               int nbj, int per, double* __restrict__ gpart, int ntiles, int accumulate, int* __restrict__ flags) {
+    using Cfg = OzGramCfg<D>;
+    constexpr int S = Cfg::kStages;
+    constexpr int NA = kOzAccs<D>;
     constexpr uint32_t kIdesc = idesc_bf16(kOzM, kOzN);
     extern __shared__ uint8_t smem_raw[];
-    // full[6], empty[6], acc_full, acc_empty
-    __shared__ __align__(8) uint64_t bars[2 * kOzStages + 2];
+    // full[S], empty[S], acc_full[NA], acc_empty[NA]
+    __shared__ __align__(8) uint64_t bars[2 * S + 2 * NA];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int s_fail;
 
@@ -207,24 +189,26 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const int r0 = blockIdx.y * per, r1 = min(r0 + per, rows);
     const int nq = r0 < r1 ? (r1 - r0 + kOzQ - 1) / kOzQ : 0;
     const int nst = (nq + kOzSQ - 1) / kOzSQ;                     // stages (the last may hold one quarter)
-    const int nchunk = (nq + kOzChunk - 1) / kOzChunk;
+    const int nchunk = (nst + kOzChunkSt - 1) / kOzChunkSt;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(&bars[0]);
-    auto full = [&](int q) { return bar0 + 8u * (q % kOzStages); };
-    auto empty = [&](int q) { return bar0 + 8u * (kOzStages + q % kOzStages); };
-    const uint32_t acc_full = bar0 + 8u * (2 * kOzStages);
-    const uint32_t acc_empty = bar0 + 8u * (2 * kOzStages + 1);
+    auto full = [&](int q) { return bar0 + 8u * (q % S); };
+    auto empty = [&](int q) { return bar0 + 8u * (S + q % S); };
+    auto acc_full = [&](int a) { return bar0 + 8u * (2 * S + a); };
+    auto acc_empty = [&](int a) { return bar0 + 8u * (2 * S + NA + a); };
 
     if (tid == 0) {
-        for (int q = 0; q < kOzStages; ++q) {
+        for (int q = 0; q < S; ++q) {
             mbar_init(full(q), 1);
             mbar_init(empty(q), 1);
         }
-        mbar_init(acc_full, 1);
-        mbar_init(acc_empty, kOzDrainWarps);
+        for (int a = 0; a < NA; ++a) {
+            mbar_init(acc_full(a), 1);
+            mbar_init(acc_empty(a), kOzDrainWarps);
+        }
         s_fail = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
@@ -238,7 +222,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
     const CUtensorMap* tmV = gram ? &tmVC : &tmVA;
 
     if (wid == 0) {
@@ -248,64 +232,60 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmV)) : "memory");
             int q = 0;                                             // stage index
             for (; q < nst; ++q) {
-                if (q >= kOzStages &&
-                    !mbar_wait_or_fail(empty(q), (uint32_t)(q / kOzStages - 1) & 1, &s_fail))
-                    break;
-                const uint32_t dst = base + (uint32_t)(q % kOzStages) * kOzStage;
-                mbar_expect_tx(full(q), kOzStage);
+                if (q >= S && !mbar_wait_or_fail(empty(q), (uint32_t)(q / S - 1) & 1, &s_fail)) break;
+                const uint32_t dst = base + (uint32_t)(q % S) * Cfg::kStage;
+                mbar_expect_tx(full(q), Cfg::kStage);
                 tma_load_3d(dst, &tmU, r0 + q * kOzSQ * kOzQ, I * kOzM, 0, full(q));
-                tma_load_3d(dst + kOzStageU, tmV, r0 + q * kOzSQ * kOzQ, J * kOzN, 0, full(q));
+                tma_load_3d(dst + Cfg::kStageU, tmV, r0 + q * kOzSQ * kOzQ, J * kOzN, 0, full(q));
             }
             if (q < nst) {
                 s_fail = 1;
                 atomicOr(flags, 4);
             }
             // before the CTA ends: the copies of the last stages have landed
-            for (int j = std::max(0, q - kOzStages); j < q; ++j) mbar_wait(full(j), (uint32_t)(j / kOzStages) & 1);
+            for (int j = std::max(0, q - S); j < q; ++j) mbar_wait(full(j), (uint32_t)(j / S) & 1);
         }
     } else if (wid == 1) {
-        // ---- MMA issuer ----
-        if (lane == 0) {
-            int last = -1;
-            bool ok = true;
-            for (int g = 0; g < nst && ok; ++g) {                  // stage g: quarters 2 g, 2 g + 1
-                if (!mbar_wait_or_fail(full(g), (uint32_t)(g / kOzStages) & 1, &s_fail)) {
-                    ok = false;
-                    break;
-                }
-                tc_fence_after();
-                const uint32_t su = base + (uint32_t)(g % kOzStages) * kOzStage, sv = su + kOzStageU;
-                for (int sub = 0; sub < kOzSQ; ++sub) {
-                    const int q = g * kOzSQ + sub;
-                    if (q >= nq) break;
-                    const bool first = (q % kOzChunk) == 0;
-                    if (first && q > 0 &&
-                        !mbar_wait_or_fail(acc_empty, (uint32_t)(q / kOzChunk - 1) & 1, &s_fail)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint32_t ko = 32u * sub;                    // second K step of the 64-byte row
+        // ---- MMA issuer: the whole warp walks the stages, one elected lane issues ----
+        int last = -1;
+        bool ok = true;
+        for (int g = 0; g < nst && ok; ++g) {                      // stage g: quarters 2 g, 2 g + 1
+            const int cst = g % kOzChunkSt, c = g / kOzChunkSt;
+            const bool first = cst == 0, end = cst == kOzChunkSt - 1 || g == nst - 1;
+            bool w = mbar_wait_or_fail(full(g), (uint32_t)(g / S) & 1, &s_fail);
+            if (first && c > 0)                                    // the drain has read the previous chunk
+                for (int a = 0; a < NA && w; ++a) w = mbar_wait_or_fail(acc_empty(a), (uint32_t)(c - 1) & 1, &s_fail);
+            ok = __all_sync(0xffffffffu, w);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t du = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage);
+            const uint64_t dv = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage + Cfg::kStageU);
+            const int nsub = min(kOzSQ, nq - g * kOzSQ);
+            if (elect_one()) {
+                // (the second K step of the 64-byte rows is 32 bytes further: + 2 in the descriptors)
+                if (!end) {
+                    for (int sub = 0; sub < nsub; ++sub)
+                        oz_issue_planes<D, kOzN>(tmem, du + 2 * sub, dv + 2 * sub, kOzPlaneU >> 4, kOzPlaneV >> 4,
+                                                 kIdesc, first && sub == 0);
+                } else {
 #pragma unroll
-                    for (int lv = 0; lv <= 5; ++lv) {
-#pragma unroll
-                        for (int s = 0; s <= lv; ++s) {
-                            const bool lead = s == 0 || (lv == 4 && s == 3);    // first MMA into this accumulator
-                            umma_bf16(tmem + (uint32_t)kOzN * oz_acc(lv, s), sw64_desc(su + s * kOzPlaneU + ko),
-                                      sw64_desc(sv + (lv - s) * kOzPlaneV + ko), kIdesc, (first && lead) ? 0u : 1u);
-                        }
+                    for (int a = 0; a < NA; ++a) {
+                        for (int sub = 0; sub < nsub; ++sub)
+                            oz_issue_acc<D, kOzN>(a, tmem, du + 2 * sub, dv + 2 * sub, kOzPlaneU >> 4, kOzPlaneV >> 4,
+                                                  kIdesc, first && sub == 0);
+                        umma_commit(acc_full(a));
                     }
-                    if ((q % kOzChunk) == kOzChunk - 1 || q == nq - 1) umma_commit(acc_full);
                 }
                 umma_commit(empty(g));
-                last = g;
             }
-            if (!ok) {
-                s_fail = 1;
-                atomicOr(flags, 4);
-            }
-            if (last >= 0) mbar_wait(empty(last), (uint32_t)(last / kOzStages) & 1);   // own MMAs complete
+            __syncwarp();
+            last = g;
         }
+        if (!ok && lane == 0) {
+            s_fail = 1;
+            atomicOr(flags, 4);
+        }
+        if (last >= 0) mbar_wait(empty(last), (uint32_t)(last / S) & 1);   // own MMAs complete
     } else {
         // ---- drain: TMEM lane quarter wid % 4, tile columns [16 h, 16 h + 16) ----
         const int wq = wid & 3, h = (wid - 2) >> 2;
@@ -319,49 +299,22 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             Macc[e] = 0.f;
         }
         bool ok = true;
-        for (int c = 0; c < nchunk; ++c) {
-            if (!mbar_wait_sleep(acc_full, (uint32_t)c & 1, &s_fail, 256)) {
-                ok = false;
-                break;
-            }
-            __syncwarp();
-            tc_fence_after();
-            {
-                constexpr int half = 0;
-                const uint32_t col = (uint32_t)(16 * h);
-                // level g (0..3) adds L_g 2^(8 g) (an integer below 2^24, exact) at bit 24 - 8 g
+        for (int c = 0; c < nchunk && ok; ++c) {
 #pragma unroll
-                for (int g = 0; g < 4; ++g) {
-                    uint32_t r[16];
-                    tmem_ld16_async(tmem + lane_off + (uint32_t)(kOzN * g) + col, r);
-                    tmem_wait_ld16(r);
-                    const float up = __int_as_float((127 + 8 * g) << 23);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        Tacc[16 * half + e] += (long long)__float2int_rn(__uint_as_float(r[e]) * up) << (24 - 8 * g);
-                }
-                // level 4, one exact half at a time (units 2^-32): whole 2^-24 units to Tacc,
-                // the rest to Macc (the two halves' floors and residues add up to the sum's)
+            for (int a = 0; a < NA; ++a) {
+                const bool w = a == 0 ? mbar_wait_sleep(acc_full(a), (uint32_t)c & 1, &s_fail, 256)
+                                      : mbar_wait_or_fail(acc_full(a), (uint32_t)c & 1, &s_fail);
+                ok = __all_sync(0xffffffffu, w);
+                if (!ok) break;
+                tc_fence_after();
                 uint32_t r[16];
-                #pragma unroll
-                for (int hf = 4; hf <= 5; ++hf) {
-                    tmem_ld16_async(tmem + lane_off + (uint32_t)(kOzN * hf) + col, r);
-                    tmem_wait_ld16(r);
-                #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int i4 = __float2int_rn(__uint_as_float(r[e]) * 0x1p32f);
-                        Tacc[16 * half + e] += (long long)(i4 >> 8);
-                        Macc[16 * half + e] += (float)(i4 & 255) * 0x1p-32f;
-                    }
-                }
-                tmem_ld16_async(tmem + lane_off + (uint32_t)(kOzN * 6) + col, r);
+                tmem_ld16_async(tmem + lane_off + (uint32_t)(kOzN * a + 16 * h), r);
                 tmem_wait_ld16(r);
-#pragma unroll
-                for (int e = 0; e < 16; ++e) Macc[16 * half + e] += __uint_as_float(r[e]);
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(acc_empty(a));
+                oz_add_level<D>(a, r, Tacc, Macc, false);          // rows per CTA are within kOzNarrowK
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(acc_empty);
         }
         if (!ok) {
             if (lane == 0) {
@@ -369,7 +322,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                 atomicOr(flags, 4);
             }
         } else if (nq > 0) {
-            // entry (m, 32 h + e) = 2^(E_u + E_v - 36) (T + M 2^24), into this split's FP64 partial
+            // entry (m, 16 h + e) = 2^(E_u + E_v - 12) (T 2^-32 + M), into this split's FP64 partial
             const int ri = I * kOzM + m;
             const int eu = ri < rank ? Ecol[ri] : -900;
             const int Eoff = gram ? 2 * rank : rank;
@@ -383,8 +336,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     const int rj = J * kOzN + 16 * h + e + u;
                     const int ev = rj < rank ? Ecol[Eoff + rj] : -900;
                     v[u] = 0.0;
-                    if (eu > -900 && ev > -900)
-                        v[u] = ldexp(fma((double)Macc[e + u], 0x1p24, (double)Tacc[e + u]), eu + ev - 36);
+                    if (eu > -900 && ev > -900) v[u] = oz_value(Tacc[e + u], Macc[e + u], eu + ev - 12, false);
                 }
                 double2* dst = reinterpret_cast<double2*>(o + e);
                 if (accumulate) {
@@ -408,37 +360,40 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kOzCols) : "memory");
 }
 
-// |x| as an FP32 value truncated toward zero (flushed to 0 below 2^-126), by bit
-// manipulation on the integer pipe.
-__device__ __forceinline__ float oz_abs_f32_rz(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-    const int e = (int)(b >> 52) - 1023 + 127;
-    if (e <= 0) return 0.f;
-    if (e >= 255) return __uint_as_float(0x7F800000u);
-    return __uint_as_float(((uint32_t)e << 23) | (uint32_t)((b >> 29) & 0x7FFFFFu));
-}
+// Exponent mark of a column whose entries (or weighted entries) are not finite:
+// its digits are zero and its Gram entries come out as NaN (k_gram_oz_final).
+constexpr int kOzNonFinite = 4000;
 
-// |wa_i| and |wc_i| truncated to FP32, once per row (wc may be NULL).
-__global__ void k_weights_rz(const double* __restrict__ wa, const double* __restrict__ wc, int64_t N,
-                             float* __restrict__ wa_rz, float* __restrict__ wc_rz) {
+// High words (sign cleared) of wa_i and wc_i, once per row (wc may be NULL).
+__global__ void k_weights_hi(const double* __restrict__ wa, const double* __restrict__ wc, int64_t N,
+                             uint32_t* __restrict__ wa_hi, uint32_t* __restrict__ wc_hi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    wa_rz[i] = oz_abs_f32_rz(wa[i]);
-    if (wc) wc_rz[i] = oz_abs_f32_rz(wc[i]);
+    wa_hi[i] = (uint32_t)__double2hiint(wa[i]) & 0x7FFFFFFFu;
+    if (wc) wc_hi[i] = (uint32_t)__double2hiint(wc[i]) & 0x7FFFFFFFu;
 }
 
-// Column bounds of |F|, |wa F| and |wc F| for an FP64 factor, as the bits of
-// non-negative doubles atomically maxed into cmax[0..3 rank) (zeroed before).
-// Only the exponent E with max < 2^E is needed, so the products are formed in
-// FP32 from truncated copies (FP64 is the slow pipe; the weights' copies come
-// from k_weights_rz) and the maxima raised by 2^-20: never below the true
-// maximum, and the exponent one too high only when the maximum lies within 2^-20
-// of a power of two.  |F| itself is exact.  Each warp reads its column in
-// 256-row steps of four 16-byte vectors per lane when the column is 16-byte
-// aligned (eight loads in flight per lane), then the ragged end row by row.
+// log2 |x w| in units of 2^-20 (its fraction linear between powers of two), from
+// the high words xh and wh: exponents added, the 20-bit significands multiplied in
+// FP32.  Monotone up to the truncations, which take at most 4 units off, over the
+// whole FP64 range (an FP32 product would overflow for weights above 2^128).
+__device__ __forceinline__ int oz_log_key(uint32_t xh, uint32_t wh) {
+    const float mx = __uint_as_float(0x3F800000u | ((xh & 0xFFFFFu) << 3));
+    const float mw = __uint_as_float(0x3F800000u | ((wh & 0xFFFFFu) << 3));
+    const int e = (int)(xh >> 20) + (int)(wh >> 20) - 2046;
+    return (int)((__float_as_uint(__fmul_rz(mx, mw)) - 0x3F800000u) >> 3) + (min(e, 2046) << 20);
+}
+
+// Column bounds for an FP64 factor, atomically maxed into cmax[0..3 rank) (zeroed
+// before): the bits of max |F|, and the keys (oz_log_key, biased by 2^31) of max
+// |wa F| and max |wc F|, of which only the exponent is needed.  All on the integer
+// and FP32 pipes (FP64 is the slow pipe).  Each warp reads its column in 256-row
+// steps: four 16-byte vectors per lane when the column is 16-byte aligned, else
+// eight 8-byte loads (several loads in flight per lane either way), then the
+// ragged end row by row.
 __global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ F, int64_t ldf, int64_t N, int rank,
-                                                     int64_t per, const float* __restrict__ wa_rz,
-                                                     const float* __restrict__ wc_rz,
+                                                     int64_t per, const uint32_t* __restrict__ wa_hi,
+                                                     const uint32_t* __restrict__ wc_hi,
                                                      unsigned long long* __restrict__ cmax) {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -446,24 +401,24 @@ __global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ 
     const int64_t i0 = (int64_t)blockIdx.y * per, i1 = min(i0 + per, N);
     const double* col = F + (int64_t)c * ldf;
     unsigned long long mu = 0;
-    float ma = 0.f, mc = 0.f;
-    auto take = [&](double x, float a, float w) {
-        mu = max(mu, (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull);
-        const float xf = oz_abs_f32_rz(x);
-        ma = fmaxf(ma, xf * a);
-        mc = fmaxf(mc, xf * w);
+    int ma = INT_MIN, mc = INT_MIN;
+    auto take = [&](double x, uint32_t a, uint32_t w) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+        mu = max(mu, b);
+        ma = max(ma, oz_log_key((uint32_t)(b >> 32), a));
+        mc = max(mc, oz_log_key((uint32_t)(b >> 32), w));
     };
     int64_t i = i0;
     if ((reinterpret_cast<uintptr_t>(col + i0) & 15) == 0) {
         for (; i + 256 <= i1; i += 256) {
             double2 x[4];
-            float2 a[4], w[4];
+            uint2 a[4], w[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = i + 64 * u + 2 * lane;
                 x[u] = *reinterpret_cast<const double2*>(col + e);
-                a[u] = *reinterpret_cast<const float2*>(wa_rz + e);
-                w[u] = wc_rz ? *reinterpret_cast<const float2*>(wc_rz + e) : make_float2(0.f, 0.f);
+                a[u] = *reinterpret_cast<const uint2*>(wa_hi + e);
+                w[u] = wc_hi ? *reinterpret_cast<const uint2*>(wc_hi + e) : make_uint2(0, 0);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -471,38 +426,59 @@ __global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ 
                 take(x[u].y, a[u].y, w[u].y);
             }
         }
+    } else {
+        for (; i + 256 <= i1; i += 256) {
+            double x[8];
+            uint32_t a[8], w[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int64_t e = i + 32 * u + lane;
+                x[u] = col[e];
+                a[u] = wa_hi[e];
+                w[u] = wc_hi ? wc_hi[e] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) take(x[u], a[u], w[u]);
+        }
     }
-    for (i += lane; i < i1; i += 32) take(col[i], wa_rz[i], wc_rz ? wc_rz[i] : 0.f);
+    for (i += lane; i < i1; i += 32) take(col[i], wa_hi[i], wc_hi ? wc_hi[i] : 0);
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
         mu = max(mu, __shfl_xor_sync(0xffffffffu, mu, o));
-        ma = fmaxf(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-        mc = fmaxf(mc, __shfl_xor_sync(0xffffffffu, mc, o));
+        ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
+        mc = max(mc, __shfl_xor_sync(0xffffffffu, mc, o));
     }
     if (lane == 0) {
-        const double up = 1.0 + 0x1p-20;
         atomicMax(cmax + c, mu);
-        atomicMax(cmax + rank + c, (unsigned long long)__double_as_longlong((double)ma * up));
-        atomicMax(cmax + 2 * rank + c, (unsigned long long)__double_as_longlong((double)mc * up));
+        atomicMax(cmax + rank + c, (unsigned long long)((uint32_t)ma + 0x80000000u));
+        atomicMax(cmax + 2 * rank + c, (unsigned long long)((uint32_t)mc + 0x80000000u));
     }
 }
 
-// E = the smallest integer with max < 2^E (frexp); zero or negligible
-// (< 2^-900) columns get E = -900, which makes all their digits zero.
-__global__ void k_colexp_f64(const unsigned long long* __restrict__ cmax, int n, int* __restrict__ E) {
+// E = the smallest integer with max < 2^E (frexp's; for the weighted columns one
+// higher when the maximum lies within 2^-18 of a power of two).  Zero or
+// negligible (< 2^-900) columns get E = -900, which makes all their digits zero;
+// columns with infinities or NaN get kOzNonFinite.
+__global__ void k_colexp_f64(const unsigned long long* __restrict__ cmax, int rank, int* __restrict__ E) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= n) return;
-    const double mx = __longlong_as_double((long long)cmax[c]);
-    int e = -900;
-    if (mx >= 0x1p-900) frexp(mx, &e);
-    E[c] = e;
+    if (c >= 3 * rank) return;
+    int e;
+    if (c < rank) {
+        const int be = (int)(cmax[c] >> 52);
+        e = be == 0x7FF ? kOzNonFinite : be - 1022;
+    } else {
+        e = (((int)((uint32_t)cmax[c] - 0x80000000u) + 4) >> 20) + 1;
+        if (e > 1024) e = kOzNonFinite;
+    }
+    E[c] = e < -899 ? -900 : e;
 }
 
 // Sum of the split partials in a fixed order; entry (a, c) of tile (I, J) is
 // Gram entry (128 I + a, 64 J + c), written with its mirror when it lies in the
 // upper triangle (each unordered pair has exactly one such owner).
 __global__ void k_gram_oz_final(const double* __restrict__ gpart, int nsplit, int ntiles, int nbi, int nbj, int rank,
-                                int ngram, double* __restrict__ A, double* __restrict__ C) {
+                                int ngram, const int* __restrict__ Ecol, double* __restrict__ A,
+                                double* __restrict__ C) {
     int I, J;
     oz_tile_decode(blockIdx.x, nbi, nbj, I, J);
     const int gram = blockIdx.y;
@@ -515,37 +491,48 @@ __global__ void k_gram_oz_final(const double* __restrict__ gpart, int nsplit, in
         double sum = 0.0;
         for (int q = 0; q < nsplit; ++q)
             sum += gpart[(((size_t)gram * nsplit + q) * ntiles + blockIdx.x) * (kOzM * kOzN) + e];
+        if (Ecol[ra] == kOzNonFinite || Ecol[(gram + 1) * rank + rc] == kOzNonFinite)
+            sum = __longlong_as_double(0x7FF8000000000000ll);
         G[(int64_t)rc * rank + ra] = sum;
         G[(int64_t)ra * rank + rc] = sum;
     }
 }
 
-bool gram_oz_eligible(const double* F, int64_t ldf, int64_t N, int rank) {
+bool gram_oz_eligible(int64_t N, int rank) {
     if (const char* e = getenv("KEVD_GRAM")) {
         if (e[0] == 'f') return false;                          // KEVD_GRAM=fp64 / ffma: the FP64-pipe kernel
     }
-    return rank >= 1 && N >= 1 && N < ((int64_t)1 << 31) && ldf % 2 == 0 &&
-           (reinterpret_cast<uintptr_t>(F) % 16) == 0 && (uint64_t)ldf * 8 < ((uint64_t)1 << 40);
+    return rank >= 1 && N >= 1 && N < ((int64_t)1 << 31);
 }
 
 static int oz_rank_pad(int rank) { return (rank + kOzM - 1) / kOzM * kOzM; }
 
+// Digits of F's planes: six when F's columns are 16-byte aligned, seven for the
+// layouts that are not (an odd leading dimension), which the FP64-pipe kernel served
+// before: its error against 64 bits (7e-16 of the Grams' 2-norm at N = 60,001, rank 401)
+// is below six digits' (2e-14), seven digits keep it.
+static int oz_gram_digits(const double* F, int64_t ldf) {
+    return (reinterpret_cast<uintptr_t>(F) & 15) == 0 && ldf % 2 == 0 ? 6 : 7;
+}
+
 // Rows per slab: a multiple of 256 (no more than N needs) with the planes of
 // all sets within kOzPlaneBudget.
-static int64_t oz_slab_rows(int64_t N, int rank, int ngram) {
-    const size_t per_row = (size_t)(ngram + 1) * kOzDigits * oz_rank_pad(rank) * 2;
+static int64_t oz_slab_rows(int64_t N, int rank, int ngram, int D) {
+    const size_t per_row = (size_t)(ngram + 1) * D * oz_rank_pad(rank) * 2;
     int64_t S = (int64_t)(kOzPlaneBudget / per_row) / 256 * 256;
     S = std::max<int64_t>(S, 256);
     return std::min<int64_t>(S, (N + 255) / 256 * 256);
 }
 
 // Row splits per slab (the same in every slab): ntiles x ngram x nsplit CTAs
-// filling whole waves of one CTA per SM, at least 4,096 rows per split.
+// filling whole waves of one CTA per SM, at least 4,096 rows per split and at most
+// kOzNarrowK.
 static int oz_nsplit(int64_t S, int64_t nctas, int nsm) {
-    int best = 1;
+    const int lo = (int)((S + kOzNarrowK - 1) / kOzNarrowK);
+    int best = lo;
     double best_eff = -1.0;
-    for (int sp = 1; sp <= 8; ++sp) {
-        if (sp > 1 && S / sp < 4096) break;
+    for (int sp = lo; sp <= std::max(lo, 8); ++sp) {
+        if (sp > lo && S / sp < 4096) break;
         const int64_t blocks = nctas * sp;
         const double eff = (double)blocks / (double)(((blocks + nsm - 1) / nsm) * nsm);
         if (eff > best_eff + 0.02) {
@@ -558,43 +545,83 @@ static int oz_nsplit(int64_t S, int64_t nctas, int nsm) {
 
 size_t gram_oz_partial_doubles(int64_t N, int rank, int ngram, int nsm) {
     const int nt = oz_ntiles(rank);
-    const int ns = oz_nsplit(oz_slab_rows(N, rank, ngram), (int64_t)nt * ngram, nsm);
+    int ns = 1;
+    for (int D = 6; D <= 7; ++D)
+        ns = std::max(ns, oz_nsplit(oz_slab_rows(N, rank, ngram, D), (int64_t)nt * ngram, nsm));
     return (size_t)ngram * ns * nt * kOzM * kOzN;
 }
 
 size_t gram_oz_plane_bytes(int64_t N, int rank, int ngram) {
-    return (size_t)(ngram + 1) * kOzDigits * oz_rank_pad(rank) * (size_t)oz_slab_rows(N, rank, ngram) * 2;
+    size_t b = 0;
+    for (int D = 6; D <= 7; ++D)
+        b = std::max(b, (size_t)(ngram + 1) * D * oz_rank_pad(rank) * (size_t)oz_slab_rows(N, rank, ngram, D) * 2);
+    return b;
 }
 
 typedef CUresult (*EncodeTiledFnOz)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                     const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                     CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// 3-D map over one set of planes (rows S, columns rank_pad, six digits), box
-// 32 rows x `cols` columns x 6 digits with the 64-byte swizzle.
-static bool oz_plane_map(EncodeTiledFnOz enc, CUtensorMap* map, uint16_t* base, int64_t S, int rank_pad, int cols) {
-    const cuuint64_t dims[3] = {(cuuint64_t)S, (cuuint64_t)rank_pad, (cuuint64_t)kOzDigits};
+// 3-D map over one set of planes (rows S, columns rank_pad, D digits), box
+// 32 rows x `cols` columns x D digits with the 64-byte swizzle.
+static bool oz_plane_map(EncodeTiledFnOz enc, CUtensorMap* map, uint16_t* base, int64_t S, int rank_pad, int cols,
+                         int D) {
+    const cuuint64_t dims[3] = {(cuuint64_t)S, (cuuint64_t)rank_pad, (cuuint64_t)D};
     const cuuint64_t strides[2] = {(cuuint64_t)S * 2, (cuuint64_t)S * 2 * rank_pad};
-    const cuuint32_t box[3] = {(cuuint32_t)(kOzSQ * kOzQ), (cuuint32_t)cols, (cuuint32_t)kOzDigits};
+    const cuuint32_t box[3] = {(cuuint32_t)(kOzSQ * kOzQ), (cuuint32_t)cols, (cuuint32_t)D};
     const cuuint32_t estr[3] = {1, 1, 1};
     return enc(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
-                           float* wa_rz, float* wc_rz, unsigned long long* cmax, int* Ecol, double* gpart,
-                           uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s) {
+template <int D>
+static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t ldf, int64_t N, int rank,
+                                 const double* wa, const double* wc, const int* Ecol, double* gpart, uint16_t* planes,
+                                 int* flags, double* A, double* C, int nsm, cudaStream_t s) {
     cudaError_t e;
     const int ngram = wc ? 2 : 1;
+    const int rank_pad = oz_rank_pad(rank);
+    const int64_t S = oz_slab_rows(N, rank, ngram, D);
+    const size_t set = (size_t)D * rank_pad * S;                  // BF16 elements per set
+    CUtensorMap mu, mva, mvc;
+    if (!oz_plane_map(enc, &mu, planes, S, rank_pad, kOzM, D) ||
+        !oz_plane_map(enc, &mva, planes + set, S, rank_pad, kOzN, D) ||
+        !oz_plane_map(enc, &mvc, planes + (ngram == 2 ? 2 : 1) * set, S, rank_pad, kOzN, D))
+        return cudaErrorInvalidValue;
+    const int nbi = (rank + kOzM - 1) / kOzM, nbj = (rank + kOzN - 1) / kOzN;
+    const int nt = oz_ntiles(rank);
+    const int ns = oz_nsplit(S, (int64_t)nt * ngram, nsm);
+    if ((e = cudaFuncSetAttribute(k_gram_oz<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)OzGramCfg<D>::kSmem)) != cudaSuccess)
+        return e;
+    for (int64_t row0 = 0; row0 < N; row0 += S) {
+        const int rows = (int)((std::min<int64_t>(S, N - row0) + kOzQ - 1) / kOzQ * kOzQ);
+        k_oz_planes<D><<<dim3((unsigned)(rank_pad / 8), (unsigned)((rows + 511) / 512)), 256, 0, s>>>(
+            F, ldf, N, rank, rank_pad, row0, rows, (int)S, wa, wc, Ecol, reinterpret_cast<uint32_t*>(planes));
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const int per = ((rows + ns - 1) / ns + kOzQ - 1) / kOzQ * kOzQ;
+        k_gram_oz<D><<<dim3((unsigned)nt, (unsigned)ns, (unsigned)ngram), kOzThreads, OzGramCfg<D>::kSmem, s>>>(
+            mu, mva, mvc, Ecol, rank, rows, nbi, nbj, per, gpart, nt, row0 > 0 ? 1 : 0, flags);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    k_gram_oz_final<<<dim3((unsigned)nt, (unsigned)ngram), 256, 0, s>>>(gpart, ns, nt, nbi, nbj, rank, ngram, Ecol, A,
+                                                                        C);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
+                           uint32_t* wa_hi, uint32_t* wc_hi, unsigned long long* cmax, int* Ecol, double* gpart,
+                           uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s) {
+    cudaError_t e;
     if ((e = cudaMemsetAsync(cmax, 0, 3 * (size_t)rank * sizeof(unsigned long long), s)) != cudaSuccess) return e;
     {
         const int ncs = (int)std::max<int64_t>(1, std::min<int64_t>(64, N / 8192));
         const int64_t pr = ((N + ncs - 1) / ncs + 255) / 256 * 256;
-        k_weights_rz<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(wa, wc, N, wa_rz, wc ? wc_rz : nullptr);
+        k_weights_hi<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(wa, wc, N, wa_hi, wc ? wc_hi : nullptr);
         k_colmax3_f64<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(
-            F, ldf, N, rank, pr, wa_rz, wc ? wc_rz : nullptr, cmax);
-        k_colexp_f64<<<(3 * rank + 255) / 256, 256, 0, s>>>(cmax, 3 * rank, Ecol);
+            F, ldf, N, rank, pr, wa_hi, wc ? wc_hi : nullptr, cmax);
+        k_colexp_f64<<<(3 * rank + 255) / 256, 256, 0, s>>>(cmax, rank, Ecol);
     }
     static EncodeTiledFnOz enc = nullptr;
     if (!enc) {
@@ -606,31 +633,9 @@ cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, co
             return cudaErrorNotSupported;
         enc = reinterpret_cast<EncodeTiledFnOz>(p);
     }
-    const int rank_pad = oz_rank_pad(rank);
-    const int64_t S = oz_slab_rows(N, rank, ngram);
-    const size_t set = (size_t)kOzDigits * rank_pad * S;          // BF16 elements per set
-    CUtensorMap mu, mva, mvc;
-    if (!oz_plane_map(enc, &mu, planes, S, rank_pad, kOzM) || !oz_plane_map(enc, &mva, planes + set, S, rank_pad, kOzN) ||
-        !oz_plane_map(enc, &mvc, planes + (ngram == 2 ? 2 : 1) * set, S, rank_pad, kOzN))
-        return cudaErrorInvalidValue;
-    const int nbi = (rank + kOzM - 1) / kOzM, nbj = (rank + kOzN - 1) / kOzN;
-    const int nt = oz_ntiles(rank);
-    const int ns = oz_nsplit(S, (int64_t)nt * ngram, nsm);
-    if ((e = cudaFuncSetAttribute(k_gram_oz, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem)) !=
-        cudaSuccess)
-        return e;
-    for (int64_t row0 = 0; row0 < N; row0 += S) {
-        const int rows = (int)((std::min<int64_t>(S, N - row0) + kOzQ - 1) / kOzQ * kOzQ);
-        k_oz_planes<<<dim3((unsigned)(rank_pad / 8), (unsigned)((rows + 511) / 512)), 256, 0, s>>>(
-            F, ldf, N, rank, rank_pad, row0, rows, (int)S, wa, wc, Ecol, reinterpret_cast<uint32_t*>(planes));
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        const int per = ((rows + ns - 1) / ns + kOzQ - 1) / kOzQ * kOzQ;
-        k_gram_oz<<<dim3((unsigned)nt, (unsigned)ns, (unsigned)ngram), kOzThreads, kOzSmem, s>>>(
-            mu, mva, mvc, Ecol, rank, rows, nbi, nbj, per, gpart, nt, row0 > 0 ? 1 : 0, flags);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    k_gram_oz_final<<<dim3((unsigned)nt, (unsigned)ngram), 256, 0, s>>>(gpart, ns, nt, nbi, nbj, rank, ngram, A, C);
-    return cudaGetLastError();
+    return oz_gram_digits(F, ldf) == 6
+               ? gram_oz_slabs<6>(enc, F, ldf, N, rank, wa, wc, Ecol, gpart, planes, flags, A, C, nsm, s)
+               : gram_oz_slabs<7>(enc, F, ldf, N, rank, wa, wc, Ecol, gpart, planes, flags, A, C, nsm, s);
 }
 
 }  // namespace kevd

@@ -26,13 +26,13 @@ cudaError_t launch_gram_tc(const float* F, int64_t ldf, int64_t N, int rank, con
 // cmax: 3 x rank, Ecol: 3 x rank scratch; gpart: gram_oz_partial_doubles(...);
 // planes: gram_oz_plane_bytes(...) bytes, 16-byte aligned (the digit planes of
 // one slab of rows).  Writes A (and C) in full, exactly symmetric.
-bool gram_oz_eligible(const double* F, int64_t ldf, int64_t N, int rank);
+bool gram_oz_eligible(int64_t N, int rank);
 size_t gram_oz_partial_doubles(int64_t N, int rank, int ngram, int nsm);
 size_t gram_oz_plane_bytes(int64_t N, int rank, int ngram);
-// wa_rz, wc_rz: N floats of scratch each (the weights' truncated FP32 copies for
-// the column bounds; wc_rz unused when wc is NULL).
+// wa_hi, wc_hi: N words of scratch each (the weights' high words for the column
+// bounds; wc_hi unused when wc is NULL).  Any ldf and alignment of F.
 cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
-                           float* wa_rz, float* wc_rz, unsigned long long* cmax, int* Ecol, double* gpart,
+                           uint32_t* wa_hi, uint32_t* wc_hi, unsigned long long* cmax, int* Ecol, double* gpart,
                            uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s);
 
 }  // namespace kevd

@@ -28,7 +28,8 @@ struct NormWs {
     int* flags;     // bit 0: some d~ <= 0, bit 1: some q~ <= 0
     double* wa;     // N rounded up to 64: 1 / d~_i^2, zero past N
     double* wc;     // N rounded up to 64: 1 / q~_i, zero past N
-    float* waf;     // N rounded up to 64: FP32 copies of the Gram weights (FP32 path), zero past N
+    float* waf;     // N rounded up to 64: FP32 copies of the Gram weights (FP32 path), zero past N; the
+                    // FP64 path keeps their high words here while it bounds the columns
     float* wcf;
     unsigned* cmax; // 3 x rank: column maxima of |F|, |wa F|, |wc F| (tensor-core Gram, FP32 F)
     float* mag;     // 3 x rank: their grid magic numbers
@@ -702,11 +703,11 @@ static int normalize_impl(const T* Fd, int64_t ldf, int64_t N, int rank, double*
         // exactly (plain split products in the MMA's FP32 accumulation were
         // measured to bias these N-long sums), or the FFMA kernel.
         KEVD_CUDA_TRY(gram32(Fd, ldf, N, rank, w.waf, w.wcf, w.gpart, A, C, w, s));
-    } else if (gram_oz_eligible(reinterpret_cast<const double*>(Fd), ldf, N, rank)) {
+    } else if (gram_oz_eligible(N, rank)) {
         // FP64 F: digit-sliced products on the tensor cores at FP64 accuracy
         TraceScope tr(kStGram, s);
-        KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, w.wc, w.waf, w.wcf,
-                                     w.cmax64, w.ecol,
+        KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, w.wc,
+                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf), w.cmax64, w.ecol,
                                      w.gpart, w.planes, w.flags, A, C, kSMs, s));
     } else {
         const int nb = (rank + kGT - 1) / kGT, ntri = nb * (nb + 1) / 2;
@@ -785,10 +786,10 @@ static int symmetric_impl(const T* Fd, int64_t ldf, int64_t N, int rank, double*
     }
     if constexpr (std::is_same<T, float>::value) {
         KEVD_CUDA_TRY(gram32(Fd, ldf, N, rank, w.waf, nullptr, w.gpart, As, nullptr, w, s));
-    } else if (gram_oz_eligible(reinterpret_cast<const double*>(Fd), ldf, N, rank)) {
+    } else if (gram_oz_eligible(N, rank)) {
         TraceScope tr(kStGram, s);
-        KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, nullptr, w.waf, w.wcf,
-                                     w.cmax64, w.ecol, w.gpart, w.planes, w.flags, As, nullptr, kSMs, s));
+        KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, nullptr,
+                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf), w.cmax64, w.ecol, w.gpart, w.planes, w.flags, As, nullptr, kSMs, s));
     } else {
         const int nb = (rank + kGT - 1) / kGT, ntri = nb * (nb + 1) / 2;
         const int ns = gram_splits(N, ntri);

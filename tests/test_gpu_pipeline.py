@@ -139,3 +139,47 @@ def test_fp64_grams_tensor_core_and_fp64_pipe(kevd, monkeypatch, N, rank, pad, g
     As = As.cpu().numpy()
     assert np.array_equal(As, As.T)
     assert np.max(np.abs(As - As0)) < 1e-12 * np.max(np.abs(As0))
+
+
+# F views whose columns are not 16-byte aligned (odd leading dimension, or a start one
+# element in): the Grams from seven digit planes.  Rank 65 / 129 leave one column in the
+# last 64- and 128-column tile, N = 255 / 257 / 33 end inside and just past a 256-row
+# chunk and a 32-row stage, N = 70,001 needs two row splits.  Bar: the operands carry
+# 2^-55 of their column's largest entry, well inside the 1e-12 of the aligned layouts.
+@pytest.mark.parametrize("N,rank,ld,off", [(255, 65, 255, 0), (257, 129, 261, 0), (33, 16, 33, 0), (4097, 64, 4098, 1),
+                                           (70001, 130, 70001, 0)])
+def test_fp64_grams_unaligned_layouts(kevd, N, rank, ld, off):
+    g = torch.Generator().manual_seed(N)
+    F = torch.rand(rank, N, generator=g, dtype=torch.float64) * torch.logspace(0, -3, rank, dtype=torch.float64)[:, None]
+    buf = torch.full((rank * ld + off,), float("nan"), dtype=torch.float64, device="cuda")
+    Fg = buf[off:].view(rank, ld)[:, :N]
+    Fg.copy_(F)
+    dt, qt, A, C = kevd.bistoch_normalize(Fg, rank)
+    d0 = F.sum(1) @ F
+    q0 = (F @ (1 / d0)) @ F
+    for G, w in ((A, 1 / (d0 * d0)), (C, 1 / q0)):
+        G0 = (F * w) @ F.T
+        G = G.cpu()
+        assert torch.equal(G, G.T)
+        assert torch.max(torch.abs(G - G0)) < 1e-12 * torch.max(torch.abs(G0))
+
+
+def test_fp64_grams_wide_weights(kevd):
+    """Rows whose degree is 1e-25 of the others' (weights 1e50, beyond FP32's range) and an
+    infinite entry: the first is within the bar of the FP64 sums, the second never comes
+    out as a finite Gram."""
+    N, rank = 3001, 40
+    g = torch.Generator().manual_seed(5)
+    F = torch.rand(rank, N, generator=g, dtype=torch.float64)
+    F[:, 7] *= 1e-25
+    Fg = F.cuda()
+    dt, qt, A, C = kevd.bistoch_normalize(Fg, rank)
+    d0 = F.sum(1) @ F
+    A0 = (F / (d0 * d0)) @ F.T
+    assert torch.max(torch.abs(A.cpu() - A0)) < 1e-12 * torch.max(torch.abs(A0))
+    Fg[3, 11] = float("inf")
+    try:
+        _, _, A, C = kevd.bistoch_normalize(Fg, rank)
+    except kevd.KevdError:
+        return
+    assert not torch.isfinite(A).all()
