@@ -160,8 +160,8 @@ struct EigWs {
     double* ymax;   // k: max_c |Y(c, j)|
     int* ozflag;    // bit 2: a bounded wait of the tensor-core lift gave up
     uint16_t* lp;   // digit planes of one row slab of F (lift from planes, ozmm.cu); before the
-                    // lift, the planes of the r x r stage's operands (at least 14 r ldk)
-    uint16_t* yp;   // digit planes of Y^T: 7 x k x ldk
+                    // lift, the planes of the r x r stage's operands (2 r rows and 128 more)
+    uint16_t* yp;   // digit planes of Y^T: k rows
     int* fexp;      // row exponents of the slab
     int* ye;        // k: row exponents of Y^T
     int* rre;       // 3 r: row exponents of the r x r stage's planes
@@ -205,11 +205,11 @@ static EigWs carve_eig(void* base, int64_t N, int r, int k, int64_t lwork, size_
     w.Yp = c.take<double>((size_t)k * lift_ldyp(r));
     w.ymax = c.take<double>(k);
     w.ozflag = c.take<int>(4);
-    const int ldk = lift_ldk(r);
-    w.lp = c.take<uint16_t>(std::max({(size_t)3 * lift_slab(N, r, 3), (size_t)kDigits * lift_slab(N, r, kDigits),
-                                      (size_t)2 * kDigits * r}) *
-                            ldk);
-    w.yp = c.take<uint16_t>((size_t)kDigits * k * ldk);
+    const int nq = lift_ldk(r) / 16;
+    w.lp = c.take<uint16_t>(std::max({oz_tile_elems(lift_slab(N, r, 3), nq, 3),
+                                      oz_tile_elems(lift_slab(N, r, kDigits), nq, kDigits),
+                                      oz_tile_elems(r, nq, kDigits) * 2 + oz_tile_elems(128, nq, kDigits)}));
+    w.yp = c.take<uint16_t>(oz_tile_elems(k, nq, kDigits));
     w.fexp = c.take<int>((size_t)lift_slab(N, r, 3));
     w.ye = c.take<int>(k);
     w.rre = c.take<int>((size_t)3 * r);
@@ -350,55 +350,37 @@ __global__ void k_rowmax_any(const T* __restrict__ F, int64_t ldf, int64_t N, in
     }
 }
 
-// D-digit planes of rows [row0, row0 + rows) of F (column-major N x r) with one
-// exponent per row from frow: word (s S + il) ldk / 2 + c / 2 holds columns c, c + 1
-// of slab row il (zero past r), fexp[il] the row's exponent.  Block: a 32-row x
-// 64-column tile transposed through shared memory (reads coalesced down columns,
-// plane writes coalesced along rows).
+// D-digit planes (tiles of oz_tile_at, nq quarters) of rows [row0, row0 + rows) of F
+// (column-major N x r, zero past r) with one exponent per row from frow; fexp[il] is
+// slab row il's exponent.  Block: 32 rows x 8 quarters; a thread cuts the 16 columns of
+// one row's quarter, so that reads run down columns and a warp's store fills 32 rows'
+// consecutive 32 bytes of a plane.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_lift_planes(const T* __restrict__ F, int64_t ldf, int64_t N, int r, int ldk,
-                                                     int64_t row0, int rows, int S, const double* __restrict__ frow,
-                                                     uint32_t* __restrict__ P, int* __restrict__ fexp) {
-    __shared__ T tile[64][33];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int c0 = blockIdx.x * 64, il0 = blockIdx.y * 32;
+__global__ void __launch_bounds__(256) k_lift_planes(const T* __restrict__ F, int64_t ldf, int64_t N, int r, int nq,
+                                                     int64_t row0, int rows, const double* __restrict__ frow,
+                                                     uint16_t* __restrict__ P, int* __restrict__ fexp) {
+    const int il = blockIdx.y * 32 + (threadIdx.x & 31), q = blockIdx.x * 8 + (threadIdx.x >> 5);
+    if (il >= rows || q >= nq) return;
+    const int64_t i = row0 + il;
+    T x[16];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const int c = c0 + wid + 8 * j, il = il0 + lane;
-        T v = T(0);
-        if (c < r && il < rows && row0 + il < N) v = F[(int64_t)c * ldf + row0 + il];
-        tile[wid + 8 * j][lane] = v;
+    for (int e = 0; e < 16; ++e) x[e] = (i < N && 16 * q + e < r) ? F[(int64_t)(16 * q + e) * ldf + i] : T(0);
+    const int E = i < N ? exp_of(frow[i]) : -900;
+    if (q == 0) fexp[il] = E;
+    long long t[16];
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        if constexpr (std::is_same<T, double>::value) t[e] = oz_T_f64<D>(x[e], E);
+        else t[e] = oz_T_f32<D>(x[e], E);
     }
-    __syncthreads();
-    const size_t plane = (size_t)S * (ldk / 2);
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-        const int rr = wid + 8 * q, il = il0 + rr;
-        if (il >= rows) break;
-        const int E = row0 + il < N ? exp_of(frow[row0 + il]) : -900;
-        if (blockIdx.x == 0 && lane == 0) fexp[il] = E;
-        const int c = c0 + 2 * lane;
-        if (c >= ldk) continue;
-        long long T0, T1;
-        if constexpr (std::is_same<T, double>::value) {
-            T0 = oz_T_f64<D>(tile[2 * lane][rr], E);
-            T1 = oz_T_f64<D>(tile[2 * lane + 1][rr], E);
-        } else {
-            T0 = oz_T_f32<D>(tile[2 * lane][rr], E);
-            T1 = oz_T_f32<D>(tile[2 * lane + 1][rr], E);
-        }
-        uint32_t wd[D];
-        oz_planes2<D>(T0, T1, wd);
-#pragma unroll
-        for (int s2 = 0; s2 < D; ++s2) P[s2 * plane + (size_t)il * (ldk / 2) + c / 2] = wd[s2];
-    }
+    oz_store_quarter<D>(P, il, q, nq, t);
 }
 
 // D-digit planes of Y^T (row j = column j of Y, r x k column-major; zero past r)
-// and their row exponents; one block per row.
+// and their row exponents; one block per row, a thread per quarter.
 template <int D>
-__global__ void __launch_bounds__(256) k_lift_ypl(const double* __restrict__ Y, int r, int k, int ldk,
-                                                  uint32_t* __restrict__ P, int* __restrict__ ye) {
+__global__ void __launch_bounds__(256) k_lift_ypl(const double* __restrict__ Y, int r, int nq,
+                                                  uint16_t* __restrict__ P, int* __restrict__ ye) {
     const int j = blockIdx.x;
     const double* y = Y + (int64_t)j * r;
     unsigned long long mx = 0;
@@ -413,12 +395,11 @@ __global__ void __launch_bounds__(256) k_lift_ypl(const double* __restrict__ Y, 
     for (int q = 1; q < (int)(blockDim.x >> 5); ++q) mx = max(mx, red[q]);
     const int E = exp_of(__longlong_as_double((long long)mx));
     if (threadIdx.x == 0) ye[j] = E;
-    const size_t plane = (size_t)k * (ldk / 2);
-    for (int c = 2 * threadIdx.x; c < ldk; c += 2 * blockDim.x) {
-        uint32_t wd[D];
-        oz_planes2<D>(oz_T_f64<D>(c < r ? y[c] : 0.0, E), oz_T_f64<D>(c + 1 < r ? y[c + 1] : 0.0, E), wd);
+    for (int q = threadIdx.x; q < nq; q += blockDim.x) {
+        long long t[16];
 #pragma unroll
-        for (int s2 = 0; s2 < D; ++s2) P[s2 * plane + (size_t)j * (ldk / 2) + c / 2] = wd[s2];
+        for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<D>(16 * q + e < r ? y[16 * q + e] : 0.0, E);
+        oz_store_quarter<D>(P, j, q, nq, t);
     }
 }
 
@@ -428,21 +409,19 @@ __global__ void __launch_bounds__(256) k_lift_ypl(const double* __restrict__ Y, 
 template <typename T, int D>
 static cudaError_t lift_planes(int64_t N, int k, int r, const T* F, int64_t ldf, const double* Y, double* U,
                                const double* rowdiv, const EigWs& w, cudaStream_t s) {
-    const int ldk = lift_ldk(r);
+    const int nq = lift_ldk(r) / 16;
     const int64_t S = lift_slab(N, r, D);
     cudaError_t e;
     k_rowmax_any<T><<<(unsigned)((N + 255) / 256), 256, 0, s>>>(F, ldf, N, r, w.frow);
-    k_lift_ypl<D><<<k, 256, 0, s>>>(Y, r, k, ldk, reinterpret_cast<uint32_t*>(w.yp), w.ye);
-    CUtensorMap ma, mb;
-    if (!ozmm_map(&ma, w.lp, S, ldk, S * ldk, true, D) || !ozmm_map(&mb, w.yp, k, ldk, (int64_t)k * ldk, false, D))
-        return cudaErrorInvalidValue;
+    k_lift_ypl<D><<<k, 256, 0, s>>>(Y, r, nq, w.yp, w.ye);
+    const OzOperand B{w.yp, nq, w.ye, 0}, A{w.lp, nq, w.fexp, 0};
     for (int64_t row0 = 0; row0 < N; row0 += S) {
         const int rows = (int)std::min<int64_t>(S, N - row0);
-        k_lift_planes<T, D><<<dim3((unsigned)((ldk + 63) / 64), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
-            F, ldf, N, r, ldk, row0, rows, (int)S, w.frow, reinterpret_cast<uint32_t*>(w.lp), w.fexp);
+        k_lift_planes<T, D><<<dim3((unsigned)((nq + 7) / 8), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
+            F, ldf, N, r, nq, row0, rows, w.frow, w.lp, w.fexp);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        if ((e = launch_ozmm(ma, mb, w.fexp, 0, w.ye, 0, rows, k, ldk, nullptr, U + row0, N, 0, nullptr, 0, 0,
-                             w.ozflag, s, D, rowdiv ? rowdiv + row0 : nullptr)) != cudaSuccess)
+        if ((e = launch_ozmm(A, B, rows, k, 16 * nq, nullptr, U + row0, N, 0, nullptr, 0, w.ozflag, s, D,
+                             rowdiv ? rowdiv + row0 : nullptr)) != cudaSuccess)
             return e;
     }
     return cudaSuccess;
@@ -710,17 +689,17 @@ __global__ void k_unit_cols(double* __restrict__ Y, int r) {
 // Planes of the rows of the column-major rows x cols matrix A (ld lda); K = cols.
 static cudaError_t rr_row_planes(const double* A, int64_t lda, int rows, int cols, uint16_t* P, int* ex,
                                  double* rmax, cudaStream_t s) {
-    const int ldk = lift_ldk(cols);
+    const int nq = lift_ldk(cols) / 16;
     k_rowmax_any<double><<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(A, lda, rows, cols, rmax);
-    k_lift_planes<double, kDigits><<<dim3((unsigned)((ldk + 63) / 64), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
-        A, lda, rows, cols, ldk, 0, rows, rows, rmax, reinterpret_cast<uint32_t*>(P), ex);
+    k_lift_planes<double, kDigits><<<dim3((unsigned)((nq + 7) / 8), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
+        A, lda, rows, cols, nq, 0, rows, rmax, P, ex);
     return cudaGetLastError();
 }
 
 // Planes of the columns of the column-major rows x cols matrix A (ld rows): plane
 // row j holds column j; K = rows.
 static cudaError_t rr_col_planes(const double* A, int rows, int cols, uint16_t* P, int* ex, cudaStream_t s) {
-    k_lift_ypl<kDigits><<<cols, 256, 0, s>>>(A, rows, cols, lift_ldk(rows), reinterpret_cast<uint32_t*>(P), ex);
+    k_lift_ypl<kDigits><<<cols, 256, 0, s>>>(A, rows, lift_ldk(rows) / 16, P, ex);
     return cudaGetLastError();
 }
 
@@ -728,11 +707,9 @@ static cudaError_t rr_col_planes(const double* A, int rows, int cols, uint16_t* 
 // ldc), from the planes of A's m rows and B's n rows.
 static cudaError_t rr_product(const uint16_t* Pa, const int* ea, int m, const uint16_t* Pb, const int* eb, int n,
                               int K, double* C, int64_t ldc, int* flag, cudaStream_t s) {
-    const int ldk = lift_ldk(K);
-    CUtensorMap ma, mb;
-    if (!ozmm_map(&ma, Pa, m, ldk, (int64_t)m * ldk, true) || !ozmm_map(&mb, Pb, n, ldk, (int64_t)n * ldk, false))
-        return cudaErrorInvalidValue;
-    return launch_ozmm(ma, mb, ea, 0, eb, 0, m, n, ldk, nullptr, C, ldc, 0, nullptr, 0, 0, flag, s);
+    const int nq = lift_ldk(K) / 16;
+    return launch_ozmm(OzOperand{Pa, nq, ea, 0}, OzOperand{Pb, nq, eb, 0}, m, n, 16 * nq, nullptr, C, ldc, 0, nullptr,
+                       0, flag, s, kDigits, nullptr, true);
 }
 
 // M = (R C) R^T (Section 2.2's inner matrix; R upper triangular with A = R^T R,
@@ -740,7 +717,7 @@ static cudaError_t rr_product(const uint16_t* Pa, const int* ea, int m, const ui
 // product's A operand and the second's B operand.
 static cudaError_t form_inner(const double* R, const double* C, int r, const EigWs& w, cudaStream_t s) {
     uint16_t* PR = w.lp;
-    uint16_t* P1 = w.lp + (size_t)kDigits * r * lift_ldk(r);
+    uint16_t* P1 = w.lp + oz_tile_elems(r, lift_ldk(r) / 16, kDigits);
     int* eR = w.rre;
     int* e1 = w.rre + r;
     cudaError_t e;
@@ -809,7 +786,8 @@ constexpr double kRitzTol = 1e-6;
 
 // M: full symmetric r x r.  Q, Y: r x b scratch.  Output lam (k, ascending) and
 // V (r x k, same order) when *ok is set on return.  Planes: M's rows (r), Q's and
-// Y's columns (b each) at w.lp, which holds 7 ldk (r + 2b) <= 14 r ldk elements.
+// Y's columns (b each) at w.lp, which holds the tiles of 2 r + 128 rows (3 b <= r, and a
+// row block rounds each up by at most 127 rows).
 static int subspace_topk(cusolverDnHandle_t h, cublasHandle_t hb, const double* M, int r, int k, int b, double* Q,
                          double* Y, double* V, double* lam, double* ss, double* work, int lwork, int* info,
                          const EigWs& w, cudaStream_t s, bool* ok) {
@@ -820,10 +798,10 @@ static int subspace_topk(cusolverDnHandle_t h, cublasHandle_t hb, const double* 
     double* Z = theta + b;
     double* res = Z + (size_t)r * k;
     double* tau = res + k;
-    const size_t pl = (size_t)kDigits * lift_ldk(r);
+    const int nq = lift_ldk(r) / 16;
     uint16_t* Pm = w.lp;
-    uint16_t* Pq = Pm + pl * r;
-    uint16_t* Py = Pq + pl * b;
+    uint16_t* Pq = Pm + oz_tile_elems(r, nq, kDigits);
+    uint16_t* Py = Pq + oz_tile_elems(b, nq, kDigits);
     int* me = w.rre;
     int* qe = me + r;
     int* ye = qe + b;

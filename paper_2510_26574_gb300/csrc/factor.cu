@@ -74,15 +74,15 @@ static FactorWs carve_factor(void* base, int64_t N, int d, int r, int b, size_t*
         o.ldF = (int)(((int64_t)r + 15 * (int64_t)std::max(rounds_max, 1) + 15) / 16 * 16);
         o.ldR = (b + 15) / 16 * 16;
         o.ldLi = (b + 1) / 2 * 2;
-        o.Xp = c.take<uint16_t>((size_t)kDigits * N * o.ldX);
+        o.Xp = c.take<uint16_t>(oz_tile_elems(N, o.ldX / 16, kDigits));
         o.xe = c.take<int>(N);
-        o.Fp = c.take<uint16_t>((size_t)kDigits * N * o.ldF);
-        o.Rp = c.take<uint16_t>((size_t)kDigits * N * o.ldR);
+        o.Fp = c.take<uint16_t>(oz_tile_elems(N, o.ldF / 16, kDigits));
+        o.Rp = c.take<uint16_t>(oz_tile_elems(N, o.ldR / 16, kDigits));
         o.re = c.take<int>(N);
-        o.PXp = c.take<uint16_t>((size_t)kDigits * b * o.ldX);
+        o.PXp = c.take<uint16_t>(oz_tile_elems(b, o.ldX / 16, kDigits));
         o.pxe = c.take<int>(b);
-        o.PFp = c.take<uint16_t>((size_t)kDigits * b * o.ldF);
-        o.Lp = c.take<uint16_t>((size_t)kDigits * b * o.ldR);
+        o.PFp = c.take<uint16_t>(oz_tile_elems(b, o.ldF / 16, kDigits));
+        o.Lp = c.take<uint16_t>(oz_tile_elems(b, o.ldR / 16, kDigits));
         o.le = c.take<int>(b);
         o.Linv = c.take<double>((size_t)b * o.ldLi);
         o.flags = c.take<int>(4);
@@ -588,32 +588,46 @@ __global__ void __launch_bounds__(256) k_engine(FactorWs w, const double* __rest
 }
 
 // Digit planes of X (seven digits, one exponent per row from max |X(i, :)|),
-// columns d .. ldX - 1 zero.  One warp per row, a lane two columns at a time.
+// columns d .. ldX - 1 zero.  Block: 32 rows x 8 quarters of 16 columns; a thread cuts
+// one row's quarter, so that a warp's store fills 32 rows' consecutive 32 bytes of a
+// plane.
 __global__ void __launch_bounds__(256) k_xplanes(const double* __restrict__ X, int64_t N, int d, OzWs o) {
-    const int lane = threadIdx.x & 31;
-    const int64_t i = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+    __shared__ unsigned long long red[8][32];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    const int nq = o.ldX / 16;
+    const double* x = X + (i < N ? i : 0) * d;
+    double v[16];
+    unsigned long long mx = 0;
+    for (int q = wid; q < nq; q += 8) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            v[e] = i < N && 16 * q + e < d ? x[16 * q + e] : 0.0;
+            mx = max(mx, (unsigned long long)__double_as_longlong(v[e]) & 0x7FFFFFFFFFFFFFFFull);
+        }
+    }
+    red[wid][lane] = mx;
+    __syncthreads();
     if (i >= N) return;
-    const double* x = X + i * d;
-    double mx = 0.0;
-    for (int c = lane; c < d; c += 32) mx = fmax(mx, fabs(x[c]));
 #pragma unroll
-    for (int q = 16; q; q >>= 1) mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, q));
-    const int E = exp_of(mx);
-    if (lane == 0) o.xe[i] = E;
-    const size_t plane = (size_t)N * o.ldX / 2;                 // words
-    uint32_t* P = reinterpret_cast<uint32_t*>(o.Xp) + (size_t)i * (o.ldX / 2);
-    for (int c = 2 * lane; c < o.ldX; c += 64) {
-        const double x0 = c < d ? x[c] : 0.0, x1 = c + 1 < d ? x[c + 1] : 0.0;
-        uint32_t wd[kDigits];
-        digits2_e(x0, x1, E, wd);
+    for (int u = 0; u < 8; ++u) mx = max(mx, red[u][lane]);
+    const int E = exp_of(__longlong_as_double((long long)mx));
+    if (wid == 0) o.xe[i] = E;
+    for (int q = wid; q < nq; q += 8) {
+        long long t[16];
 #pragma unroll
-        for (int s = 0; s < kDigits; ++s) P[s * plane + c / 2] = wd[s];
+        for (int e = 0; e < 16; ++e) {
+            if (nq > 8) v[e] = 16 * q + e < d ? x[16 * q + e] : 0.0;    // one quarter per warp is still in v
+            t[e] = oz_T_f64<kDigits>(v[e], E);
+        }
+        oz_store_quarter<kDigits>(o.Xp, i, q, nq, t);
     }
 }
 
 // Pivot panels of the round as rows of the digit planes: row l < m of PXp is
 // row S_l of Xp (exponent pxe_l), row l of PFp is row S_l of Fp over the padded
-// rank kp; rows l >= m are zero.  One block per row l, 16-byte copies.
+// rank kp; rows l >= m are zero.  One block per row l; a thread copies the 32 bytes of
+// one quarter and plane (halves exchanged when the two rows' swizzles differ).
 __global__ void __launch_bounds__(128) k_ozpanel(FactorWs w, OzWs o, int64_t N, int b) {
     const FactorState* st = w.st;
     if (st->done || st->m == 0) return;
@@ -622,16 +636,19 @@ __global__ void __launch_bounds__(128) k_ozpanel(FactorWs w, OzWs o, int64_t N, 
     const bool on = l < st->m;
     const int64_t row = on ? w.prop[w.acc_pos[l]] : 0;
     if (threadIdx.x == 0) o.pxe[l] = on ? o.xe[row] : -900;
-    const int kp = st->kp;
-    const uint4 z = make_uint4(0, 0, 0, 0);
-    for (int s = 0; s < kDigits; ++s) {
-        const uint4* xs = reinterpret_cast<const uint4*>(o.Xp + ((size_t)s * N + row) * o.ldX);
-        uint4* xd = reinterpret_cast<uint4*>(o.PXp + ((size_t)s * b + l) * o.ldX);
-        for (int c = threadIdx.x; c < o.ldX / 8; c += blockDim.x) xd[c] = on ? xs[c] : z;
-        const uint4* fs = reinterpret_cast<const uint4*>(o.Fp + ((size_t)s * N + row) * o.ldF);
-        uint4* fd = reinterpret_cast<uint4*>(o.PFp + ((size_t)s * b + l) * o.ldF);
-        for (int c = threadIdx.x; c < kp / 8; c += blockDim.x) fd[c] = on ? fs[c] : z;
-    }
+    const int flip = ((int)(row >> 2) ^ (l >> 2)) & 1;
+    auto gather = [&](const uint16_t* src, uint16_t* dst, int nq, int nused) {
+        for (int u = threadIdx.x; u < nused * kDigits; u += blockDim.x) {
+            const int q = u / kDigits, z = u % kDigits;
+            const uint4* sp = reinterpret_cast<const uint4*>(src + oz_tile_at(row, q, z, nq, kDigits));
+            uint4* dp = reinterpret_cast<uint4*>(dst + oz_tile_at(l, q, z, nq, kDigits));
+            const uint4 zero = make_uint4(0, 0, 0, 0);
+            dp[0] = on ? sp[flip] : zero;
+            dp[1] = on ? sp[flip ^ 1] : zero;
+        }
+    };
+    gather(o.Xp, o.PXp, o.ldX / 16, o.ldX / 16);
+    gather(o.Fp, o.PFp, o.ldF / 16, st->kp / 16);
 }
 
 // L(T,T)^-1 of the round (lower triangular, m x m) and its digit planes: rows j
@@ -674,13 +691,11 @@ __global__ void __launch_bounds__(128) k_linv(FactorWs w, OzWs o, int b) {
         for (int l = 0; l < m; ++l) mx = fmax(mx, fabs(row[l]));
         const int E = exp_of(mx);
         o.le[c] = E;
-        uint32_t* P = reinterpret_cast<uint32_t*>(o.Lp) + (size_t)c * (o.ldR / 2);
-        const size_t plane = (size_t)b * o.ldR / 2;
-        for (int l = 0; l < o.ldR; l += 2) {
-            uint32_t wd[kDigits];
-            digits2_e(l < m ? row[l] : 0.0, l + 1 < m ? row[l + 1] : 0.0, E, wd);
+        for (int q = 0; q < o.ldR / 16; ++q) {
+            long long t[16];
 #pragma unroll
-            for (int s = 0; s < kDigits; ++s) P[s * plane + l / 2] = wd[s];
+            for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<kDigits>(16 * q + e < m ? row[16 * q + e] : 0.0, E);
+            oz_store_quarter<kDigits>(o.Lp, c, q, o.ldR / 16, t);
         }
     }
 }
@@ -688,62 +703,66 @@ __global__ void __launch_bounds__(128) k_linv(FactorWs w, OzWs o, int b) {
 // R = K(:, T) - F(:, :k) F(T, :k)^T from the tensor-core products: the kernel
 // values exp(-(|x_i|^2 + |x_s|^2 - 2 x_i.x_s) / eps) (1 at the pivot itself)
 // minus Df, as digit planes with one exponent per row (the row maximum over
-// the round's pivots).  Block: 32 rows x 8 warps, warp g taking the 16 pivots
-// [16 g, 16 g + 16) (16 values per thread: low register use, four blocks per SM).
-__global__ void __launch_bounds__(256, 4) k_rprep(FactorWs w, OzWs o, int64_t N, double inv_eps,
-                                                  const unsigned long long* __restrict__ tblg) {
+// the round's pivots).  Block: 32 rows x ldR / 16 warps, warp g taking the quarter of
+// 16 pivots [16 g, 16 g + 16).
+__global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, double inv_eps,
+                                               const unsigned long long* __restrict__ tblg) {
     const FactorState* st = w.st;
     if (st->done || st->m == 0) return;
     const int m = st->m, k = st->k;
     __shared__ unsigned long long red[8][32];
     __shared__ unsigned long long tbl[1024];
+    __shared__ double s_xn[128];
+    __shared__ int64_t s_row[128];
     for (int e = threadIdx.x; e < 1024; e += blockDim.x) tbl[e] = tblg[e];
-    __syncthreads();
-    const int il = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t row = (int64_t)blockIdx.x * 32 + il;
-    const int l0 = 16 * g;
-    double R[16];
-    unsigned long long mx = 0;                                 // max |R| as the bits of a non-negative double
-    const double xi = row < N ? w.xn[row] : 0.0;
-#pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        const int l = l0 + e;
-        double rv = 0.0;
-        if (row < N && l < m) {
-            const int pos = w.acc_pos[l];
-            const int64_t at = row + (int64_t)l * w.ldD;
-            double kv;
-            if (w.prop[pos] == row) {
-                kv = 1.0;
-            } else {
-                double d2 = fma(-2.0, w.Dx[at], xi + w.xnS[pos]);
-                if (__double_as_longlong(d2) < 0) d2 = 0.0;     // negative rounding residue
-                kv = kexp(-d2 * inv_eps, tbl);
-            }
-            rv = k > 0 ? kv - w.Df[at] : kv;
-        }
-        R[e] = rv;
-        mx = max(mx, (unsigned long long)__double_as_longlong(rv) & 0x7FFFFFFFFFFFFFFFull);
+    for (int l = threadIdx.x; l < m; l += blockDim.x) {
+        const int pos = w.acc_pos[l];
+        s_xn[l] = w.xnS[pos];
+        s_row[l] = w.prop[pos];
     }
-    red[g][il] = mx;
     __syncthreads();
-    if (row >= N || l0 >= o.ldR) return;
-    unsigned long long rm = red[0][il];
+    const int lane = threadIdx.x & 31, g = threadIdx.x >> 5, nq = o.ldR / 16;
+    const int l0 = 16 * g;
+    for (int64_t row0 = (int64_t)blockIdx.x * 32; row0 < N; row0 += (int64_t)gridDim.x * 32) {
+        const int64_t row = row0 + lane;
+        double R[16], df[16];
+        const bool on = row < N;
+        const double xi = on ? w.xn[row] : 0.0;
 #pragma unroll
-    for (int q = 1; q < 8; ++q) rm = max(rm, red[q][il]);
-    const int E = exp_of(__longlong_as_double((long long)rm));
-    if (g == 0) o.re[row] = E;
-    const size_t plane = (size_t)N * o.ldR / 2;
-    uint32_t* P = reinterpret_cast<uint32_t*>(o.Rp) + (size_t)row * (o.ldR / 2) + l0 / 2;
-    const int npair = min(8, (o.ldR - l0) / 2);
-#pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        if (e < npair) {
-            uint32_t wd[kDigits];
-            digits2_e(R[2 * e], R[2 * e + 1], E, wd);
-#pragma unroll
-            for (int s = 0; s < kDigits; ++s) P[s * plane + e] = wd[s];
+        for (int e = 0; e < 16; ++e) {
+            const int64_t at = row + (int64_t)(l0 + e) * w.ldD;
+            const bool in = on && l0 + e < m;
+            R[e] = in ? w.Dx[at] : 0.0;
+            df[e] = in && k > 0 ? w.Df[at] : 0.0;
         }
+        unsigned long long mx = 0;                             // max |R| as the bits of a non-negative double
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+            const int l = l0 + e;
+            double rv = 0.0;
+            if (on && l < m) {
+                double kv = 1.0;
+                if (s_row[l] != row) {
+                    double d2 = fma(-2.0, R[e], xi + s_xn[l]);
+                    if (__double_as_longlong(d2) < 0) d2 = 0.0;     // negative rounding residue
+                    kv = kexp(-d2 * inv_eps, tbl);
+                }
+                rv = kv - df[e];
+            }
+            R[e] = rv;
+            mx = max(mx, (unsigned long long)__double_as_longlong(rv) & 0x7FFFFFFFFFFFFFFFull);
+        }
+        red[g][lane] = mx;
+        __syncthreads();
+        for (int q = 0; q < nq; ++q) mx = max(mx, red[q][lane]);
+        __syncthreads();                                       // red is rewritten for the next rows
+        if (!on) continue;
+        const int E = exp_of(__longlong_as_double((long long)mx));
+        if (g == 0) o.re[row] = E;
+        long long t[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<kDigits>(R[e], E);
+        oz_store_quarter<kDigits>(o.Rp, row, g, nq, t);
     }
 }
 
@@ -956,17 +975,11 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
     const bool oz = oz_engine_for(opts, N, b, allow_oz);
     FactorWs w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b));
     if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return KEVD_EWORKSPACE;
-    // tensor maps of the digit planes: X and F (A operands), the pivot panels (B),
-    // R and L^-1 of each round
-    CUtensorMap mXp, mPX, mFp, mPF, mRp, mLp;
+    // the digit planes: X and F (A operands), the pivot panels (B), R and L^-1 of each round
     const unsigned long long* exp_tbl = nullptr;
-    if (oz && !(ozmm_map(&mXp, ow.Xp, N, ow.ldX, N * ow.ldX, true) &&
-                ozmm_map(&mPX, ow.PXp, b, ow.ldX, (int64_t)b * ow.ldX, false) &&
-                ozmm_map(&mFp, ow.Fp, N, ow.ldF, N * ow.ldF, true) &&
-                ozmm_map(&mPF, ow.PFp, b, ow.ldF, (int64_t)b * ow.ldF, false) &&
-                ozmm_map(&mRp, ow.Rp, N, ow.ldR, N * ow.ldR, true) &&
-                ozmm_map(&mLp, ow.Lp, b, ow.ldR, (int64_t)b * ow.ldR, false)))
-        return KEVD_ECUDA;
+    const OzOperand oX{ow.Xp, ow.ldX / 16, ow.xe, 0}, oPX{ow.PXp, ow.ldX / 16, ow.pxe, 0},
+        oF{ow.Fp, ow.ldF / 16, nullptr, 1}, oPF{ow.PFp, ow.ldF / 16, nullptr, 1}, oR{ow.Rp, ow.ldR / 16, ow.re, 0},
+        oL{ow.Lp, ow.ldR / 16, ow.le, 0};
 
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const double* Xd = static_cast<const double*>(X);
@@ -985,7 +998,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
             k_prepare<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(Xd, N, d, w, rho);
             if (oz) {
                 KEVD_CUDA_TRY(kexp_table(s, &exp_tbl));
-                k_xplanes<<<(unsigned)((N + 7) / 8), 256, 0, s>>>(Xd, N, d, ow);
+                k_xplanes<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(Xd, N, d, ow);
                 KEVD_CUDA_TRY(cudaMemsetAsync(ow.flags, 0, sizeof(int), s));
             }
         }
@@ -1034,17 +1047,15 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
                     // X X(S,:)^T and F(:, :k) F(S, :k)^T on the tensor cores at FP64 accuracy
                     TraceScope tp(kStProducts, s);
                     k_ozpanel<<<b, 128, 0, s>>>(w, ow, N, b);
-                    KEVD_CUDA_TRY(launch_ozmm(mXp, mPX, ow.xe, 0, ow.pxe, 0, N, b, ow.ldX, w.st, w.Dx, w.ldD, 0,
-                                              nullptr, 0, 0, ow.flags, s));
-                    KEVD_CUDA_TRY(launch_ozmm(mFp, mPF, nullptr, 1, nullptr, 1, N, b, -3, w.st, w.Df, w.ldD, 0,
-                                              nullptr, 0, 0, ow.flags, s));
+                    KEVD_CUDA_TRY(launch_ozmm(oX, oPX, N, b, ow.ldX, w.st, w.Dx, w.ldD, 0, nullptr, 0, ow.flags, s));
+                    KEVD_CUDA_TRY(launch_ozmm(oF, oPF, N, b, -3, w.st, w.Df, w.ldD, 0, nullptr, 0, ow.flags, s));
                 }
                 TraceScope tr(kStEngine, s);
                 // R = K(:, T) - F F(T,:)^T; G = R L^-T into F(:, k:k+m), on the tensor cores; rho
-                k_rprep<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(w, ow, N, inv_eps, exp_tbl);
+                k_rprep<<<(unsigned)std::min<int64_t>((N + 31) / 32, 152 * 8), 2 * ow.ldR, 0, s>>>(w, ow, N, inv_eps,
+                                                                                                   exp_tbl);
                 k_linv<<<1, 128, (size_t)b * b * sizeof(double), s>>>(w, ow, b);
-                KEVD_CUDA_TRY(launch_ozmm(mRp, mLp, ow.re, 0, ow.le, 0, N, b, -2, w.st, Fd, ldf, ldf, ow.Fp, ow.ldF,
-                                          N * ow.ldF, ow.flags, s));
+                KEVD_CUDA_TRY(launch_ozmm(oR, oL, N, b, -2, w.st, Fd, ldf, ldf, ow.Fp, ow.ldF / 16, ow.flags, s));
                 k_rho_update<<<(unsigned)((N + 63) / 64), 256, 0, s>>>(w, Fd, ldf, rho, N);
             } else {
                 TraceScope tr(kStEngine, s);

@@ -51,8 +51,8 @@ struct FactorWs {
 
 // Panels of the tensor-core products of the FP64 path (host-launched kernels only).
 // Workspace of the FP64 engine on the tensor cores (ozmm.cu): seven-digit BF16
-// planes (plane s of an R x ldk operand at s R ldk, row i at i ldk, K-major)
-// and their row exponents.
+// planes (tiles of oz_tile_at, ld / 16 quarters, rows padded to 128) and their row
+// exponents.
 struct OzWs {
     uint16_t* Xp;      // X: N x ldX, exponents xe (once per factorisation)
     int* xe;

@@ -3,15 +3,20 @@
 // error-free slicing of the operands in the manner of Ozaki, Ogita, Oishi and
 // Rump (2012), with BF16 slice products summed exactly in TMEM.
 //
+// Operands.  A = (sa F)^T (sa F) with sa = 1 / d~ and C = (sc F)^T (sc F) with
+// sc = 1 / sqrt(q~): each Gram has one scaled operand for both sides, so one set of
+// planes, and the scaling evens out the rows (with the whole weight on one side a
+// row of small degree is tiny in the one operand and huge in the other, and its
+// product is lost below their columns' largest entries).
+//
 // Slicing.  Every operand column c (over all rows) has an exponent E_c with
 // max_i |x_ic| < 2^E_c.  T = round(x 2^(46 - E_c)) is an integer below 2^46,
 // written in six balanced base-256 digits d_0 .. d_5 (d_s in [-128, 127]), so
 // x = 2^(E_c - 6) sum_s d_s 2^(-8 s) up to 2^(E_c - 47).  Digit plane s holds
-// p_s = d_s 2^(-8 s), an exact BF16 value.  The operands are U = F (the I
-// block of columns) and V = w F (the J block, w = wa or wc).
+// p_s = d_s 2^(-8 s), an exact BF16 value.  U is the I block of columns, V the J block.
 //
 // Products.  The Gram entry is 2^(E_u + E_v - 12) sum_(s,t) sum_i p_s p_t; the
-// pairs with s + t <= 5 are kept (21 MMAs per 16 rows), the rest lie below
+// pairs with s + t <= 5 and (3, 3) are kept (22 MMAs per 16 rows), the rest lie below
 // 2^-48 of the largest product.  Level g = s + t has g + 1 pairs whose
 // products are integer multiples of 2^(-8 g) below 2^14 in magnitude, so over
 // 256 rows the level-g sum is an integer multiple of 2^(-8 g) below 2^24 for
@@ -31,7 +36,7 @@
 //
 // Layout.  The rows are taken in slabs sized so that the digit planes of one
 // slab stay within a fixed budget.  k_oz_planes cuts a slab once: for each of
-// U, wa F (and wc F) D planes of rank_pad columns x S rows of BF16, a
+// sa F (and sc F) D planes of rank_pad columns x S rows of BF16, a
 // column's rows contiguous, so that a TMA box of 32 rows x 128 (or 64) columns
 // x D planes with the 64-byte swizzle lands as D K-major MMA operands of two
 // 16-row quarters (64-byte rows: half as many L2 requests per byte as 32-byte
@@ -112,26 +117,25 @@ int oz_ntiles(int rank) {
 }
 
 // D-digit planes of the slab of rows [row0, row0 + rows) (rows a multiple of 16;
-// zero past N and past rank): set 0 from F, set 1 from wa F, set 2 from wc F
-// (when wc is given).  Plane (set, s) is rank_pad x S BF16 pairs, word
-// ((set D + s) rank_pad + c) S / 2 + i / 2 holding rows i, i + 1 of column c.
-// Block: 8 warps = 8 columns; a warp takes 64 rows per step (a lane two, as one
-// 16-byte vector when the column is 16-byte aligned, else as two 8-byte loads:
-// any F and ldf are cut, so the FP64-pipe kernel is not needed for odd ones).
+// zero past N and past rank): set 0 from sa F, set 1 from sc F (when sc is given).
+// Plane (set, s) is rank_pad x S BF16 pairs, word ((set D + s) rank_pad + c) S / 2 +
+// i / 2 holding rows i, i + 1 of column c.  Block: 8 warps = 8 columns; a warp takes
+// 64 rows per step (a lane two, as one 16-byte vector when the column is 16-byte
+// aligned, else as two 8-byte loads: any F and ldf are cut).
 template <int D>
 __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F, int64_t ldf, int64_t N, int rank,
                                                    int rank_pad, int64_t row0, int rows, int S,
-                                                   const double* __restrict__ wa, const double* __restrict__ wc,
+                                                   const double* __restrict__ sa, const double* __restrict__ sc,
                                                    const int* __restrict__ Ecol, uint32_t* __restrict__ P) {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (c >= rank_pad) return;
     const bool on = c < rank;
     const size_t plane = (size_t)rank_pad * (S / 2);
-    const int sets = wc ? 3 : 2;
-    int E[3];
+    const int sets = sc ? 2 : 1;
+    int E[2];
 #pragma unroll
-    for (int z = 0; z < 3; ++z) E[z] = (on && z < sets) ? Ecol[z * rank + c] : -900;
+    for (int z = 0; z < 2; ++z) E[z] = (on && z < sets) ? Ecol[z * rank + c] : -900;
     const double* col = F + (int64_t)c * ldf;
     const bool vec = (reinterpret_cast<uintptr_t>(col) & 15) == 0;   // row0 is even
     for (int it = 0; it < 8; ++it) {
@@ -149,14 +153,11 @@ __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F,
         }
         const size_t at = (size_t)c * (S / 2) + (il >> 1);
 #pragma unroll
-        for (int z = 0; z < 3; ++z) {
+        for (int z = 0; z < 2; ++z) {
             if (z >= sets) break;
-            double y0 = x0, y1 = x1;
-            if (z > 0) {
-                const double* w = z == 1 ? wa : wc;
-                y0 = i < N ? __dmul_rn(w[i], x0) : 0.0;
-                y1 = i + 1 < N ? __dmul_rn(w[i + 1], x1) : 0.0;
-            }
+            const double* w = z == 0 ? sa : sc;
+            const double y0 = i < N ? __dmul_rn(w[i], x0) : 0.0;
+            const double y1 = i + 1 < N ? __dmul_rn(w[i + 1], x1) : 0.0;
             uint32_t wd[D];
             oz_planes2<D>(oz_T_f64<D>(y0, E[z]), oz_T_f64<D>(y1, E[z]), wd);
 #pragma unroll
@@ -170,8 +171,9 @@ __global__ void __launch_bounds__(256) k_oz_planes(const double* __restrict__ F,
 // (accumulate = 0) or added to (accumulate = 1) its partial in gpart.
 template <int D>
 __global__ void __launch_bounds__(kOzThreads, 1)
-    k_gram_oz(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmVA,
-              const __grid_constant__ CUtensorMap tmVC, const int* __restrict__ Ecol, int rank, int rows, int nbi,
+    k_gram_oz(const __grid_constant__ CUtensorMap tmUA, const __grid_constant__ CUtensorMap tmVA,
+              const __grid_constant__ CUtensorMap tmUC, const __grid_constant__ CUtensorMap tmVC,
+              const int* __restrict__ Ecol, int rank, int rows, int nbi,
               int nbj, int per, double* __restrict__ gpart, int ntiles, int accumulate, int* __restrict__ flags) {
     using Cfg = OzGramCfg<D>;
     constexpr int S = Cfg::kStages;
@@ -185,7 +187,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
 
     int I, J;
     oz_tile_decode(blockIdx.x, nbi, nbj, I, J);
-    const int gram = blockIdx.z;                                   // 0: A (wa), 1: C (wc)
+    const int gram = blockIdx.z;                                   // 0: A (sa), 1: C (sc)
     const int r0 = blockIdx.y * per, r1 = min(r0 + per, rows);
     const int nq = r0 < r1 ? (r1 - r0 + kOzQ - 1) / kOzQ : 0;
     const int nst = (nq + kOzSQ - 1) / kOzSQ;                     // stages (the last may hold one quarter)
@@ -223,19 +225,20 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const CUtensorMap* tmU = gram ? &tmUC : &tmUA;
     const CUtensorMap* tmV = gram ? &tmVC : &tmVA;
 
     if (wid == 0) {
         // ---- TMA producer ----
         if (lane == 0) {
-            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmU)) : "memory");
+            asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmU)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmV)) : "memory");
             int q = 0;                                             // stage index
             for (; q < nst; ++q) {
                 if (q >= S && !mbar_wait_or_fail(empty(q), (uint32_t)(q / S - 1) & 1, &s_fail)) break;
                 const uint32_t dst = base + (uint32_t)(q % S) * Cfg::kStage;
                 mbar_expect_tx(full(q), Cfg::kStage);
-                tma_load_3d(dst, &tmU, r0 + q * kOzSQ * kOzQ, I * kOzM, 0, full(q));
+                tma_load_3d(dst, tmU, r0 + q * kOzSQ * kOzQ, I * kOzM, 0, full(q));
                 tma_load_3d(dst + Cfg::kStageU, tmV, r0 + q * kOzSQ * kOzQ, J * kOzN, 0, full(q));
             }
             if (q < nst) {
@@ -313,7 +316,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(acc_empty(a));
-                oz_add_level<D>(a, r, Tacc, Macc, false);          // rows per CTA are within kOzNarrowK
+                oz_add_level<D>(a, r, Tacc, Macc);          // rows per CTA are within kOzNarrowK
             }
         }
         if (!ok) {
@@ -324,8 +327,8 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         } else if (nq > 0) {
             // entry (m, 16 h + e) = 2^(E_u + E_v - 12) (T 2^-32 + M), into this split's FP64 partial
             const int ri = I * kOzM + m;
-            const int eu = ri < rank ? Ecol[ri] : -900;
-            const int Eoff = gram ? 2 * rank : rank;
+            const int Eoff = gram * rank;
+            const int eu = ri < rank ? Ecol[Eoff + ri] : -900;
             double* o = gpart + (((size_t)gram * gridDim.y + blockIdx.y) * ntiles + blockIdx.x) * (kOzM * kOzN) +
                         (size_t)m * kOzN + 16 * h;
 #pragma unroll
@@ -336,7 +339,7 @@ __global__ void __launch_bounds__(kOzThreads, 1)
                     const int rj = J * kOzN + 16 * h + e + u;
                     const int ev = rj < rank ? Ecol[Eoff + rj] : -900;
                     v[u] = 0.0;
-                    if (eu > -900 && ev > -900) v[u] = oz_value(Tacc[e + u], Macc[e + u], eu + ev - 12, false);
+                    if (eu > -900 && ev > -900) v[u] = oz_value(Tacc[e + u], Macc[e + u], eu + ev - 12);
                 }
                 double2* dst = reinterpret_cast<double2*>(o + e);
                 if (accumulate) {
@@ -360,53 +363,51 @@ __global__ void __launch_bounds__(kOzThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kOzCols) : "memory");
 }
 
-// Exponent mark of a column whose entries (or weighted entries) are not finite:
-// its digits are zero and its Gram entries come out as NaN (k_gram_oz_final).
+// Exponent mark of a column whose scaled entries are not finite: its digits are zero
+// and its Gram entries come out as NaN (k_gram_oz_final).
 constexpr int kOzNonFinite = 4000;
 
-// High words (sign cleared) of wa_i and wc_i, once per row (wc may be NULL).
-__global__ void k_weights_hi(const double* __restrict__ wa, const double* __restrict__ wc, int64_t N,
-                             uint32_t* __restrict__ wa_hi, uint32_t* __restrict__ wc_hi) {
+// High words (sign cleared) of sa_i and sc_i, once per row (sc may be NULL).
+__global__ void k_weights_hi(const double* __restrict__ sa, const double* __restrict__ sc, int64_t N,
+                             uint32_t* __restrict__ sa_hi, uint32_t* __restrict__ sc_hi) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= N) return;
-    wa_hi[i] = (uint32_t)__double2hiint(wa[i]) & 0x7FFFFFFFu;
-    if (wc) wc_hi[i] = (uint32_t)__double2hiint(wc[i]) & 0x7FFFFFFFu;
+    sa_hi[i] = (uint32_t)__double2hiint(sa[i]) & 0x7FFFFFFFu;
+    if (sc) sc_hi[i] = (uint32_t)__double2hiint(sc[i]) & 0x7FFFFFFFu;
 }
 
 // log2 |x w| in units of 2^-20 (its fraction linear between powers of two), from
 // the high words xh and wh: exponents added, the 20-bit significands multiplied in
 // FP32.  Monotone up to the truncations, which take at most 4 units off, over the
 // whole FP64 range (an FP32 product would overflow for weights above 2^128).
+// Infinite and NaN factors give the largest key.
 __device__ __forceinline__ int oz_log_key(uint32_t xh, uint32_t wh) {
     const float mx = __uint_as_float(0x3F800000u | ((xh & 0xFFFFFu) << 3));
     const float mw = __uint_as_float(0x3F800000u | ((wh & 0xFFFFFu) << 3));
     const int e = (int)(xh >> 20) + (int)(wh >> 20) - 2046;
-    return (int)((__float_as_uint(__fmul_rz(mx, mw)) - 0x3F800000u) >> 3) + (min(e, 2046) << 20);
+    const int key = (int)((__float_as_uint(__fmul_rz(mx, mw)) - 0x3F800000u) >> 3) + (e << 20);
+    return max(xh, wh) >= 0x7FF00000u ? INT_MAX : key;
 }
 
-// Column bounds for an FP64 factor, atomically maxed into cmax[0..3 rank) (zeroed
-// before): the bits of max |F|, and the keys (oz_log_key, biased by 2^31) of max
-// |wa F| and max |wc F|, of which only the exponent is needed.  All on the integer
-// and FP32 pipes (FP64 is the slow pipe).  Each warp reads its column in 256-row
-// steps: four 16-byte vectors per lane when the column is 16-byte aligned, else
-// eight 8-byte loads (several loads in flight per lane either way), then the
-// ragged end row by row.
-__global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ F, int64_t ldf, int64_t N, int rank,
-                                                     int64_t per, const uint32_t* __restrict__ wa_hi,
-                                                     const uint32_t* __restrict__ wc_hi,
-                                                     unsigned long long* __restrict__ cmax) {
+// Column bounds of sa F and sc F for an FP64 factor: the keys (oz_log_key, biased by
+// 2^31) of their largest entries, atomically maxed into cmax[0..2 rank) (zeroed
+// before); only the exponents are needed.  All on the integer and FP32 pipes (FP64 is
+// the slow pipe).  Each warp reads its column in 256-row steps: four 16-byte vectors
+// per lane when the column is 16-byte aligned, else eight 8-byte loads (several loads
+// in flight per lane either way), then the ragged end row by row.
+__global__ void __launch_bounds__(256) k_colmax_f64(const double* __restrict__ F, int64_t ldf, int64_t N, int rank,
+                                                    int64_t per, const uint32_t* __restrict__ sa_hi,
+                                                    const uint32_t* __restrict__ sc_hi, uint32_t* __restrict__ cmax) {
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (c >= rank) return;
     const int64_t i0 = (int64_t)blockIdx.y * per, i1 = min(i0 + per, N);
     const double* col = F + (int64_t)c * ldf;
-    unsigned long long mu = 0;
     int ma = INT_MIN, mc = INT_MIN;
     auto take = [&](double x, uint32_t a, uint32_t w) {
-        const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
-        mu = max(mu, b);
-        ma = max(ma, oz_log_key((uint32_t)(b >> 32), a));
-        mc = max(mc, oz_log_key((uint32_t)(b >> 32), w));
+        const uint32_t xh = (uint32_t)__double2hiint(x) & 0x7FFFFFFFu;
+        ma = max(ma, oz_log_key(xh, a));
+        mc = max(mc, oz_log_key(xh, w));
     };
     int64_t i = i0;
     if ((reinterpret_cast<uintptr_t>(col + i0) & 15) == 0) {
@@ -417,8 +418,8 @@ __global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ 
             for (int u = 0; u < 4; ++u) {
                 const int64_t e = i + 64 * u + 2 * lane;
                 x[u] = *reinterpret_cast<const double2*>(col + e);
-                a[u] = *reinterpret_cast<const uint2*>(wa_hi + e);
-                w[u] = wc_hi ? *reinterpret_cast<const uint2*>(wc_hi + e) : make_uint2(0, 0);
+                a[u] = *reinterpret_cast<const uint2*>(sa_hi + e);
+                w[u] = sc_hi ? *reinterpret_cast<const uint2*>(sc_hi + e) : make_uint2(0, 0);
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -434,43 +435,31 @@ __global__ void __launch_bounds__(256) k_colmax3_f64(const double* __restrict__ 
             for (int u = 0; u < 8; ++u) {
                 const int64_t e = i + 32 * u + lane;
                 x[u] = col[e];
-                a[u] = wa_hi[e];
-                w[u] = wc_hi ? wc_hi[e] : 0;
+                a[u] = sa_hi[e];
+                w[u] = sc_hi ? sc_hi[e] : 0;
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) take(x[u], a[u], w[u]);
         }
     }
-    for (i += lane; i < i1; i += 32) take(col[i], wa_hi[i], wc_hi ? wc_hi[i] : 0);
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        mu = max(mu, __shfl_xor_sync(0xffffffffu, mu, o));
-        ma = max(ma, __shfl_xor_sync(0xffffffffu, ma, o));
-        mc = max(mc, __shfl_xor_sync(0xffffffffu, mc, o));
-    }
+    for (i += lane; i < i1; i += 32) take(col[i], sa_hi[i], sc_hi ? sc_hi[i] : 0);
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    mc = __reduce_max_sync(0xffffffffu, mc);
     if (lane == 0) {
-        atomicMax(cmax + c, mu);
-        atomicMax(cmax + rank + c, (unsigned long long)((uint32_t)ma + 0x80000000u));
-        atomicMax(cmax + 2 * rank + c, (unsigned long long)((uint32_t)mc + 0x80000000u));
+        atomicMax(cmax + c, (uint32_t)ma + 0x80000000u);
+        atomicMax(cmax + rank + c, (uint32_t)mc + 0x80000000u);
     }
 }
 
-// E = the smallest integer with max < 2^E (frexp's; for the weighted columns one
-// higher when the maximum lies within 2^-18 of a power of two).  Zero or
-// negligible (< 2^-900) columns get E = -900, which makes all their digits zero;
-// columns with infinities or NaN get kOzNonFinite.
-__global__ void k_colexp_f64(const unsigned long long* __restrict__ cmax, int rank, int* __restrict__ E) {
+// E = the smallest integer with max < 2^E (frexp's, or one higher when the maximum
+// lies within 2^-18 of a power of two).  Negligible (< 2^-900) columns get E = -900,
+// which makes all their digits zero; columns with infinities or NaN kOzNonFinite.
+__global__ void k_colexp_f64(const uint32_t* __restrict__ cmax, int n, int* __restrict__ E) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= 3 * rank) return;
-    int e;
-    if (c < rank) {
-        const int be = (int)(cmax[c] >> 52);
-        e = be == 0x7FF ? kOzNonFinite : be - 1022;
-    } else {
-        e = (((int)((uint32_t)cmax[c] - 0x80000000u) + 4) >> 20) + 1;
-        if (e > 1024) e = kOzNonFinite;
-    }
-    E[c] = e < -899 ? -900 : e;
+    if (c >= n) return;
+    const int key = (int)(cmax[c] - 0x80000000u);
+    const int e = ((min(key, INT_MAX - 4) + 4) >> 20) + 1;
+    E[c] = key == INT_MAX || e > 1024 ? kOzNonFinite : e < -899 ? -900 : e;
 }
 
 // Sum of the split partials in a fixed order; entry (a, c) of tile (I, J) is
@@ -491,7 +480,7 @@ __global__ void k_gram_oz_final(const double* __restrict__ gpart, int nsplit, in
         double sum = 0.0;
         for (int q = 0; q < nsplit; ++q)
             sum += gpart[(((size_t)gram * nsplit + q) * ntiles + blockIdx.x) * (kOzM * kOzN) + e];
-        if (Ecol[ra] == kOzNonFinite || Ecol[(gram + 1) * rank + rc] == kOzNonFinite)
+        if (Ecol[gram * rank + ra] == kOzNonFinite || Ecol[gram * rank + rc] == kOzNonFinite)
             sum = __longlong_as_double(0x7FF8000000000000ll);
         G[(int64_t)rc * rank + ra] = sum;
         G[(int64_t)ra * rank + rc] = sum;
@@ -518,7 +507,7 @@ static int oz_gram_digits(const double* F, int64_t ldf) {
 // Rows per slab: a multiple of 256 (no more than N needs) with the planes of
 // all sets within kOzPlaneBudget.
 static int64_t oz_slab_rows(int64_t N, int rank, int ngram, int D) {
-    const size_t per_row = (size_t)(ngram + 1) * D * oz_rank_pad(rank) * 2;
+    const size_t per_row = (size_t)ngram * D * oz_rank_pad(rank) * 2;
     int64_t S = (int64_t)(kOzPlaneBudget / per_row) / 256 * 256;
     S = std::max<int64_t>(S, 256);
     return std::min<int64_t>(S, (N + 255) / 256 * 256);
@@ -554,7 +543,7 @@ size_t gram_oz_partial_doubles(int64_t N, int rank, int ngram, int nsm) {
 size_t gram_oz_plane_bytes(int64_t N, int rank, int ngram) {
     size_t b = 0;
     for (int D = 6; D <= 7; ++D)
-        b = std::max(b, (size_t)(ngram + 1) * D * oz_rank_pad(rank) * (size_t)oz_slab_rows(N, rank, ngram, D) * 2);
+        b = std::max(b, (size_t)ngram * D * oz_rank_pad(rank) * (size_t)oz_slab_rows(N, rank, ngram, D) * 2);
     return b;
 }
 
@@ -577,17 +566,17 @@ static bool oz_plane_map(EncodeTiledFnOz enc, CUtensorMap* map, uint16_t* base, 
 
 template <int D>
 static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t ldf, int64_t N, int rank,
-                                 const double* wa, const double* wc, const int* Ecol, double* gpart, uint16_t* planes,
+                                 const double* sa, const double* sc, const int* Ecol, double* gpart, uint16_t* planes,
                                  int* flags, double* A, double* C, int nsm, cudaStream_t s) {
     cudaError_t e;
-    const int ngram = wc ? 2 : 1;
+    const int ngram = sc ? 2 : 1;
     const int rank_pad = oz_rank_pad(rank);
     const int64_t S = oz_slab_rows(N, rank, ngram, D);
     const size_t set = (size_t)D * rank_pad * S;                  // BF16 elements per set
-    CUtensorMap mu, mva, mvc;
-    if (!oz_plane_map(enc, &mu, planes, S, rank_pad, kOzM, D) ||
-        !oz_plane_map(enc, &mva, planes + set, S, rank_pad, kOzN, D) ||
-        !oz_plane_map(enc, &mvc, planes + (ngram == 2 ? 2 : 1) * set, S, rank_pad, kOzN, D))
+    CUtensorMap mua, mva, muc, mvc;
+    uint16_t* pc = planes + (ngram == 2 ? set : 0);
+    if (!oz_plane_map(enc, &mua, planes, S, rank_pad, kOzM, D) || !oz_plane_map(enc, &muc, pc, S, rank_pad, kOzM, D) ||
+        !oz_plane_map(enc, &mva, planes, S, rank_pad, kOzN, D) || !oz_plane_map(enc, &mvc, pc, S, rank_pad, kOzN, D))
         return cudaErrorInvalidValue;
     const int nbi = (rank + kOzM - 1) / kOzM, nbj = (rank + kOzN - 1) / kOzN;
     const int nt = oz_ntiles(rank);
@@ -598,11 +587,11 @@ static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t l
     for (int64_t row0 = 0; row0 < N; row0 += S) {
         const int rows = (int)((std::min<int64_t>(S, N - row0) + kOzQ - 1) / kOzQ * kOzQ);
         k_oz_planes<D><<<dim3((unsigned)(rank_pad / 8), (unsigned)((rows + 511) / 512)), 256, 0, s>>>(
-            F, ldf, N, rank, rank_pad, row0, rows, (int)S, wa, wc, Ecol, reinterpret_cast<uint32_t*>(planes));
+            F, ldf, N, rank, rank_pad, row0, rows, (int)S, sa, sc, Ecol, reinterpret_cast<uint32_t*>(planes));
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         const int per = ((rows + ns - 1) / ns + kOzQ - 1) / kOzQ * kOzQ;
         k_gram_oz<D><<<dim3((unsigned)nt, (unsigned)ns, (unsigned)ngram), kOzThreads, OzGramCfg<D>::kSmem, s>>>(
-            mu, mva, mvc, Ecol, rank, rows, nbi, nbj, per, gpart, nt, row0 > 0 ? 1 : 0, flags);
+            mua, mva, muc, mvc, Ecol, rank, rows, nbi, nbj, per, gpart, nt, row0 > 0 ? 1 : 0, flags);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     k_gram_oz_final<<<dim3((unsigned)nt, (unsigned)ngram), 256, 0, s>>>(gpart, ns, nt, nbi, nbj, rank, ngram, Ecol, A,
@@ -610,18 +599,18 @@ static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t l
     return cudaGetLastError();
 }
 
-cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
-                           uint32_t* wa_hi, uint32_t* wc_hi, unsigned long long* cmax, int* Ecol, double* gpart,
+cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* sa, const double* sc,
+                           uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, double* gpart,
                            uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(cmax, 0, 3 * (size_t)rank * sizeof(unsigned long long), s)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(cmax, 0, 2 * (size_t)rank * sizeof(uint32_t), s)) != cudaSuccess) return e;
     {
         const int ncs = (int)std::max<int64_t>(1, std::min<int64_t>(64, N / 8192));
         const int64_t pr = ((N + ncs - 1) / ncs + 255) / 256 * 256;
-        k_weights_hi<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(wa, wc, N, wa_hi, wc ? wc_hi : nullptr);
-        k_colmax3_f64<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(
-            F, ldf, N, rank, pr, wa_hi, wc ? wc_hi : nullptr, cmax);
-        k_colexp_f64<<<(3 * rank + 255) / 256, 256, 0, s>>>(cmax, rank, Ecol);
+        k_weights_hi<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(sa, sc, N, sa_hi, sc ? sc_hi : nullptr);
+        k_colmax_f64<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(
+            F, ldf, N, rank, pr, sa_hi, sc ? sc_hi : nullptr, cmax);
+        k_colexp_f64<<<(2 * rank + 255) / 256, 256, 0, s>>>(cmax, 2 * rank, Ecol);
     }
     static EncodeTiledFnOz enc = nullptr;
     if (!enc) {
@@ -634,8 +623,8 @@ cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, co
         enc = reinterpret_cast<EncodeTiledFnOz>(p);
     }
     return oz_gram_digits(F, ldf) == 6
-               ? gram_oz_slabs<6>(enc, F, ldf, N, rank, wa, wc, Ecol, gpart, planes, flags, A, C, nsm, s)
-               : gram_oz_slabs<7>(enc, F, ldf, N, rank, wa, wc, Ecol, gpart, planes, flags, A, C, nsm, s);
+               ? gram_oz_slabs<6>(enc, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, nsm, s)
+               : gram_oz_slabs<7>(enc, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, nsm, s);
 }
 
 }  // namespace kevd

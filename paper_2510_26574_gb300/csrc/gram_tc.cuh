@@ -21,18 +21,17 @@ cudaError_t launch_gram_tc(const float* F, int64_t ldf, int64_t N, int rank, con
                            unsigned* cmax, float* mag, float* gpart, int* flags, int nb, int ntri, int64_t per,
                            int nsplit, cudaStream_t s);
 
-// FP64 factor: weighted Grams on the tensor cores at FP64 accuracy (gram_oz.cu).
-// wa, wc: FP64 weights zero-padded to a multiple of 64 rows (wc NULL: A only);
-// cmax: 3 x rank, Ecol: 3 x rank scratch; gpart: gram_oz_partial_doubles(...);
-// planes: gram_oz_plane_bytes(...) bytes, 16-byte aligned (the digit planes of
-// one slab of rows).  Writes A (and C) in full, exactly symmetric.
+// FP64 factor: weighted Grams on the tensor cores at FP64 accuracy (gram_oz.cu),
+// A = (sa F)^T (sa F) and C = (sc F)^T (sc F).  sa, sc: N row scales (sc NULL: A
+// only); sa_hi, sc_hi: N words of scratch each; cmax, Ecol: 2 x rank scratch; gpart:
+// gram_oz_partial_doubles(...); planes: gram_oz_plane_bytes(...) bytes, 16-byte aligned
+// (the digit planes of one slab of rows).  Any ldf and alignment of F.  Writes A (and
+// C) in full, exactly symmetric.
 bool gram_oz_eligible(int64_t N, int rank);
 size_t gram_oz_partial_doubles(int64_t N, int rank, int ngram, int nsm);
 size_t gram_oz_plane_bytes(int64_t N, int rank, int ngram);
-// wa_hi, wc_hi: N words of scratch each (the weights' high words for the column
-// bounds; wc_hi unused when wc is NULL).  Any ldf and alignment of F.
-cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
-                           uint32_t* wa_hi, uint32_t* wc_hi, unsigned long long* cmax, int* Ecol, double* gpart,
+cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* sa, const double* sc,
+                           uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, double* gpart,
                            uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s);
 
 }  // namespace kevd

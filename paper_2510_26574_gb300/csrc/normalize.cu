@@ -33,8 +33,8 @@ struct NormWs {
     float* wcf;
     unsigned* cmax; // 3 x rank: column maxima of |F|, |wa F|, |wc F| (tensor-core Gram, FP32 F)
     float* mag;     // 3 x rank: their grid magic numbers
-    unsigned long long* cmax64;   // 3 x rank: the same maxima for FP64 F
-    int* ecol;      // 3 x rank: their exponents
+    uint32_t* cmax64;   // 2 x rank: keys of the column maxima of the scaled FP64 F
+    int* ecol;      // 2 x rank: their exponents
     uint16_t* planes;   // FP64 Gram: digit planes of one slab of rows
     double* gpart;  // nsplit x ntri x 2 x 64 x 64 Gram partials (128 x 128 for FP32 F)
 };
@@ -94,8 +94,8 @@ static NormWs carve_norm(void* base, int64_t N, int rank, size_t* bytes, bool fp
     w.wcf = c.take<float>(Npad);
     w.cmax = c.take<unsigned>(3 * (size_t)rank);
     w.mag = c.take<float>(3 * (size_t)rank);
-    w.cmax64 = c.take<unsigned long long>(3 * (size_t)rank);
-    w.ecol = c.take<int>(3 * (size_t)rank);
+    w.cmax64 = c.take<uint32_t>(2 * (size_t)rank);
+    w.ecol = c.take<int>(2 * (size_t)rank);
     w.gpart = c.take<double>(std::max(std::max(gp64, gp32), gpoz));
     w.planes = fp64 ? c.take<uint16_t>(std::max(gram_oz_plane_bytes(N, rank, 2), gram_oz_plane_bytes(N, rank, 1)) / 2)
                     : nullptr;
@@ -247,6 +247,16 @@ __global__ void k_gram_weights(const double* __restrict__ dtil, const double* __
     wc[i] = 1.0 / qtil[i];
     waf[i] = (float)wa[i];
     wcf[i] = (float)wc[i];
+}
+
+// Row scales of the tensor-core FP64 Grams: sa = 1/d~ (or 1/sqrt(d~) with qtil ==
+// nullptr, the symmetric form's one Gram) and sc = 1/sqrt(q~).
+__global__ void k_gram_scales(const double* __restrict__ dtil, const double* __restrict__ qtil, int64_t N,
+                              double* __restrict__ sa, double* __restrict__ sc) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= N) return;
+    sa[i] = 1.0 / (qtil ? dtil[i] : sqrt(dtil[i]));
+    if (qtil) sc[i] = 1.0 / sqrt(qtil[i]);
 }
 
 // Weighted Gram partials.  Block = one (I, J) tile and one row split; 256
@@ -693,22 +703,24 @@ static int normalize_impl(const T* Fd, int64_t ldf, int64_t N, int rank, double*
     }
     KEVD_LAUNCH_CHECK();
 
+    const bool oz = std::is_same<T, double>::value && gram_oz_eligible(N, rank);
     {
         TraceScope tr(kStGram, s);
         const int64_t Npad = (N + 63) / 64 * 64;
-        k_gram_weights<<<(unsigned)((Npad + 255) / 256), 256, 0, s>>>(dtil, qtil, N, Npad, w.wa, w.wc, w.waf, w.wcf);
+        if (oz) k_gram_scales<<<rows_blocks, 256, 0, s>>>(dtil, qtil, N, w.wa, w.wc);
+        else k_gram_weights<<<(unsigned)((Npad + 255) / 256), 256, 0, s>>>(dtil, qtil, N, Npad, w.wa, w.wc, w.waf, w.wcf);
     }
     if constexpr (std::is_same<T, float>::value) {
         // FP32 F: tensor-core slice products with the leading product summed
         // exactly (plain split products in the MMA's FP32 accumulation were
         // measured to bias these N-long sums), or the FFMA kernel.
         KEVD_CUDA_TRY(gram32(Fd, ldf, N, rank, w.waf, w.wcf, w.gpart, A, C, w, s));
-    } else if (gram_oz_eligible(N, rank)) {
+    } else if (oz) {
         // FP64 F: digit-sliced products on the tensor cores at FP64 accuracy
         TraceScope tr(kStGram, s);
         KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, w.wc,
-                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf), w.cmax64, w.ecol,
-                                     w.gpart, w.planes, w.flags, A, C, kSMs, s));
+                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf),
+                                     w.cmax64, w.ecol, w.gpart, w.planes, w.flags, A, C, kSMs, s));
     } else {
         const int nb = (rank + kGT - 1) / kGT, ntri = nb * (nb + 1) / 2;
         const int ns = gram_splits(N, ntri);
@@ -777,19 +789,22 @@ static int symmetric_impl(const T* Fd, int64_t ldf, int64_t N, int rank, double*
         if (vec) k_rowdot<T, VV><<<vrows_blocks, 256, vsm, s>>>(Fd, ldf, N, rank, w.svec, dtil, w.flags, 1);
         else k_rowdot<T, 1><<<rows_blocks, 256, vsm, s>>>(Fd, ldf, N, rank, w.svec, dtil, w.flags, 1);
     }
+    const bool oz = std::is_same<T, double>::value && gram_oz_eligible(N, rank);
     {
         TraceScope tr(kStGram, s);
         const int64_t Npad = (N + 63) / 64 * 64;
-        k_recip_pad<<<(unsigned)((Npad + 255) / 256), 256, 0, s>>>(dtil, N, Npad, w.wa);
+        if (oz) k_gram_scales<<<rows_blocks, 256, 0, s>>>(dtil, nullptr, N, w.wa, nullptr);
+        else k_recip_pad<<<(unsigned)((Npad + 255) / 256), 256, 0, s>>>(dtil, N, Npad, w.wa);
         if constexpr (std::is_same<T, float>::value)
             k_recip_f<<<(unsigned)((Npad + 255) / 256), 256, 0, s>>>(dtil, N, Npad, w.waf);
     }
     if constexpr (std::is_same<T, float>::value) {
         KEVD_CUDA_TRY(gram32(Fd, ldf, N, rank, w.waf, nullptr, w.gpart, As, nullptr, w, s));
-    } else if (gram_oz_eligible(N, rank)) {
+    } else if (oz) {
         TraceScope tr(kStGram, s);
         KEVD_CUDA_TRY(launch_gram_oz(reinterpret_cast<const double*>(Fd), ldf, N, rank, w.wa, nullptr,
-                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf), w.cmax64, w.ecol, w.gpart, w.planes, w.flags, As, nullptr, kSMs, s));
+                                     reinterpret_cast<uint32_t*>(w.waf), reinterpret_cast<uint32_t*>(w.wcf),
+                                     w.cmax64, w.ecol, w.gpart, w.planes, w.flags, As, nullptr, kSMs, s));
     } else {
         const int nb = (rank + kGT - 1) / kGT, ntri = nb * (nb + 1) / 2;
         const int ns = gram_splits(N, ntri);

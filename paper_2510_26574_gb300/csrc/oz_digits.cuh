@@ -140,4 +140,42 @@ __device__ __forceinline__ void digits2_e(double x0, double x1, int E, uint32_t 
     digits2(x0, x1, E > -900 ? 1021 + E : 4096, w);
 }
 
+// Layout of the planes of an R x 16 nq operand of k_ozmm: tiles of 128 rows x 16
+// columns (32 bytes per row, the 16-byte halves exchanged in rows 4-7 of every eight:
+// the 32-byte-swizzled K-major MMA operand), the D planes of a tile one after the
+// other, a row block's tiles along K.  One bulk copy of 4 D KB brings a tile: a tensor
+// map's box of 32-byte rows moves one row per cycle, 32 bytes per cycle and SM
+// (measured), below what the MMAs take.
+__host__ __device__ inline size_t oz_tile_elems(int64_t rows, int nq, int D) {
+    return (size_t)((rows + 127) / 128) * nq * D * 2048;
+}
+// Offset (in elements) of the 32 bytes of row i, quarter q, plane s.
+__host__ __device__ inline size_t oz_tile_at(int64_t i, int q, int s, int nq, int D) {
+    return (((size_t)(i >> 7) * nq + q) * D + s) * 2048 + (size_t)(i & 127) * 16;
+}
+
+// 32 bytes to a 32-byte aligned global address as one full-sector store.
+static __device__ __forceinline__ void stg256(void* p, const uint32_t (&w)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]),
+                 "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+                 : "memory");
+}
+
+// Cuts the 16 sliced values T (oz_T_f64 / oz_T_f32) of row i, quarter q into its D
+// planes.
+template <int D>
+static __device__ __forceinline__ void oz_store_quarter(uint16_t* P, int64_t i, int q, int nq, const long long (&T)[16]) {
+    uint16_t* dst = P + oz_tile_at(i, q, 0, nq, D);
+    const bool swap = (i & 4) != 0;
+#pragma unroll
+    for (int s = 0; s < D; ++s) {
+        uint32_t v[8], w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = oz_word<D>(T[2 * j], T[2 * j + 1], s);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = swap ? v[j ^ 4] : v[j];
+        stg256(dst + (size_t)s * 2048, w);
+    }
+}
+
 }  // namespace kevd
