@@ -49,17 +49,14 @@
 //   * lane 0 of warp 0 keeps a ring of 32-row stages filled (two TMA loads per stage:
 //     48 KB of U planes, 24 KB of V planes, three stages; 56 + 28 KB, two, with
 //     seven digits);
-//   * warp 1 issues the UMMAs (oz_mma.cuh: planes of U kept in the collector buffer,
-//     the last stage of a chunk accumulator by accumulator), frees a stage by a
-//     commit, and waits for the drain before the next chunk overwrites the
-//     accumulators;
+//   * a lane of warp 1 issues the UMMAs (oz_mma.cuh: planes of U kept in the collector
+//     buffer, the accumulators ending one after the other) and frees a stage by a commit;
 //   * warps 2-17 drain (TMEM lane quarter w % 4, tile columns [16 h, 16 h + 16)
 //     with h = (w - 2) / 4) and finally add the tile's FP64 partial.
-// Bound: shared memory, 102 KB of operand reads and TMA writes per quarter = 800
-// cycles, beside 735 of MMA issue.  Measured at N = 262,144, rank 1,101: both Grams
-// 11.8 ms (17.9 ms with one reading of U's plane per MMA and the drain after the last
-// MMA of a chunk).  At N = 60,001, rank 401 (odd: seven digits) 0.71 ms, against
-// 25.9 ms on the FP64 pipe.
+// Bound: the issue of the MMAs (oz_mma.cuh).  Measured at N = 262,144, rank 1,101: both
+// Grams 11.8 ms (17.9 ms with one reading of U's plane per MMA, level order and one
+// barrier for all accumulators).  At N = 60,001, rank 401 (odd: seven digits) 0.70 ms,
+// against 25.9 ms on the FP64 pipe.
 // Every wait is bounded (about one second); on a timeout the CTA sets bit 2 of
 // flags, waits (bounded) for its own copies and MMAs, frees TMEM and exits.
 #include <cuda.h>
@@ -77,7 +74,6 @@ namespace kevd {
 
 constexpr int kOzQ = 16;          // rows per quarter (one MMA K step)
 constexpr int kOzSQ = 2;          // quarters per stage (one 64-byte swizzled row of K)
-constexpr int kOzChunkSt = 8;     // stages per exact chunk: 256 rows
 constexpr int kOzDrainWarps = 16;
 constexpr int kOzThreads = (2 + kOzDrainWarps) * 32;
 constexpr int kOzM = 128, kOzN = 64;
@@ -191,7 +187,6 @@ __global__ void __launch_bounds__(kOzThreads, 1)
     const int r0 = blockIdx.y * per, r1 = min(r0 + per, rows);
     const int nq = r0 < r1 ? (r1 - r0 + kOzQ - 1) / kOzQ : 0;
     const int nst = (nq + kOzSQ - 1) / kOzSQ;                     // stages (the last may hold one quarter)
-    const int nchunk = (nst + kOzChunkSt - 1) / kOzChunkSt;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     const uint32_t raw = smem_u32(smem_raw);
@@ -249,51 +244,33 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             for (int j = std::max(0, q - S); j < q; ++j) mbar_wait(full(j), (uint32_t)(j / S) & 1);
         }
     } else if (wid == 1) {
-        // ---- MMA issuer: the whole warp walks the stages, one elected lane issues ----
-        int last = -1;
-        bool ok = true;
-        for (int g = 0; g < nst && ok; ++g) {                      // stage g: quarters 2 g, 2 g + 1
-            const int cst = g % kOzChunkSt, c = g / kOzChunkSt;
-            const bool first = cst == 0, end = cst == kOzChunkSt - 1 || g == nst - 1;
-            bool w = mbar_wait_or_fail(full(g), (uint32_t)(g / S) & 1, &s_fail);
-            if (first && c > 0)                                    // the drain has read the previous chunk
-                for (int a = 0; a < NA && w; ++a) w = mbar_wait_or_fail(acc_empty(a), (uint32_t)(c - 1) & 1, &s_fail);
-            ok = __all_sync(0xffffffffu, w);
-            if (!ok) break;
-            tc_fence_after();
-            const uint64_t du = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage);
-            const uint64_t dv = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage + Cfg::kStageU);
-            const int nsub = min(kOzSQ, nq - g * kOzSQ);
-            if (elect_one()) {
+        // ---- MMA issuer: one elected lane ----
+        if (elect_one()) {
+            OzIssuer<D, kOzN, false> is{tmem, kIdesc, kOzPlaneU >> 4, kOzPlaneV >> 4, acc_full(0), acc_empty(0), &s_fail};
+            int g = 0;
+            bool ok = true;
+            for (; g < nst && ok; ++g) {                           // stage g: quarters 2 g, 2 g + 1
+                ok = mbar_wait_quick(full(g), (uint32_t)(g / S) & 1, &s_fail);
+                if (!ok) break;
+                tc_fence_after();
+                const uint64_t du = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage);
+                const uint64_t dv = sw64_desc(base + (uint32_t)(g % S) * Cfg::kStage + Cfg::kStageU);
                 // (the second K step of the 64-byte rows is 32 bytes further: + 2 in the descriptors)
-                if (!end) {
-                    for (int sub = 0; sub < nsub; ++sub)
-                        oz_issue_planes<D, kOzN>(tmem, du + 2 * sub, dv + 2 * sub, kOzPlaneU >> 4, kOzPlaneV >> 4,
-                                                 kIdesc, first && sub == 0);
-                } else {
-#pragma unroll
-                    for (int a = 0; a < NA; ++a) {
-                        for (int sub = 0; sub < nsub; ++sub)
-                            oz_issue_acc<D, kOzN>(a, tmem, du + 2 * sub, dv + 2 * sub, kOzPlaneU >> 4, kOzPlaneV >> 4,
-                                                  kIdesc, first && sub == 0);
-                        umma_commit(acc_full(a));
-                    }
-                }
+                for (int sub = 0; sub < kOzSQ && ok; ++sub)
+                    if (2 * g + sub < nq) ok = is.quarter(du + 2 * sub, dv + 2 * sub, 2 * g + sub, nq);
                 umma_commit(empty(g));
             }
-            __syncwarp();
-            last = g;
+            if (!ok) {
+                s_fail = 1;
+                atomicOr(flags, 4);
+            }
+            if (g > 0) mbar_wait(empty(g - 1), (uint32_t)((g - 1) / S) & 1);   // own MMAs complete
         }
-        if (!ok && lane == 0) {
-            s_fail = 1;
-            atomicOr(flags, 4);
-        }
-        if (last >= 0) mbar_wait(empty(last), (uint32_t)(last / S) & 1);   // own MMAs complete
+        __syncwarp();
     } else {
         // ---- drain: TMEM lane quarter wid % 4, tile columns [16 h, 16 h + 16) ----
         const int wq = wid & 3, h = (wid - 2) >> 2;
         const int m = 32 * wq + lane;
-        const uint32_t lane_off = (uint32_t)(32 * wq) << 16;
         long long Tacc[16];
         float Macc[16];
 #pragma unroll
@@ -301,24 +278,9 @@ __global__ void __launch_bounds__(kOzThreads, 1)
             Tacc[e] = 0;
             Macc[e] = 0.f;
         }
-        bool ok = true;
-        for (int c = 0; c < nchunk && ok; ++c) {
-#pragma unroll
-            for (int a = 0; a < NA; ++a) {
-                const bool w = a == 0 ? mbar_wait_sleep(acc_full(a), (uint32_t)c & 1, &s_fail, 256)
-                                      : mbar_wait_or_fail(acc_full(a), (uint32_t)c & 1, &s_fail);
-                ok = __all_sync(0xffffffffu, w);
-                if (!ok) break;
-                tc_fence_after();
-                uint32_t r[16];
-                tmem_ld16_async(tmem + lane_off + (uint32_t)(kOzN * a + 16 * h), r);
-                tmem_wait_ld16(r);
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(acc_empty(a));
-                oz_add_level<D>(a, r, Tacc, Macc);          // rows per CTA are within kOzNarrowK
-            }
-        }
+        OzDrain<D, kOzN, false> dr{tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(16 * h), acc_full(0), acc_empty(0),
+                                   &s_fail};
+        const bool ok = dr.tile(nq, Tacc, Macc);                   // rows per CTA are within kOzNarrowK
         if (!ok) {
             if (lane == 0) {
                 s_fail = 1;
@@ -504,13 +466,13 @@ static int oz_gram_digits(const double* F, int64_t ldf) {
     return (reinterpret_cast<uintptr_t>(F) & 15) == 0 && ldf % 2 == 0 ? 6 : 7;
 }
 
-// Rows per slab: a multiple of 256 (no more than N needs) with the planes of
-// all sets within kOzPlaneBudget.
+// Rows per slab: a multiple of 256 with the planes of all sets within kOzPlaneBudget, the
+// rows spread evenly over the slabs (a short last slab would leave most SMs idle).
 static int64_t oz_slab_rows(int64_t N, int rank, int ngram, int D) {
     const size_t per_row = (size_t)ngram * D * oz_rank_pad(rank) * 2;
-    int64_t S = (int64_t)(kOzPlaneBudget / per_row) / 256 * 256;
-    S = std::max<int64_t>(S, 256);
-    return std::min<int64_t>(S, (N + 255) / 256 * 256);
+    const int64_t most = std::max<int64_t>(256, (int64_t)(kOzPlaneBudget / per_row) / 256 * 256);
+    const int64_t nslab = (N + most - 1) / most;
+    return ((N + nslab - 1) / nslab + 255) / 256 * 256;
 }
 
 // Row splits per slab (the same in every slab): ntiles x ngram x nsplit CTAs
@@ -520,11 +482,11 @@ static int oz_nsplit(int64_t S, int64_t nctas, int nsm) {
     const int lo = (int)((S + kOzNarrowK - 1) / kOzNarrowK);
     int best = lo;
     double best_eff = -1.0;
-    for (int sp = lo; sp <= std::max(lo, 8); ++sp) {
+    for (int sp = lo; sp <= lo + 8; ++sp) {
         if (sp > lo && S / sp < 4096) break;
         const int64_t blocks = nctas * sp;
         const double eff = (double)blocks / (double)(((blocks + nsm - 1) / nsm) * nsm);
-        if (eff > best_eff + 0.02) {
+        if (eff > best_eff + 0.01) {
             best_eff = eff;
             best = sp;
         }

@@ -162,16 +162,30 @@ static __device__ __forceinline__ void stg256(void* p, const uint32_t (&w)[8]) {
 }
 
 // Cuts the 16 sliced values T (oz_T_f64 / oz_T_f32) of row i, quarter q into its D
-// planes.
+// planes (rolled over the planes: the unrolled form costs more in instruction fetches).
 template <int D>
 static __device__ __forceinline__ void oz_store_quarter(uint16_t* P, int64_t i, int q, int nq, const long long (&T)[16]) {
     uint16_t* dst = P + oz_tile_at(i, q, 0, nq, D);
     const bool swap = (i & 4) != 0;
+    unsigned long long off = 0;
 #pragma unroll
+    for (int z = 0; z < D; ++z) off |= 0x80ull << (8 * z);
+    unsigned long long U[16];                                   // balanced digits: byte D - 1 - s is plane s's, plus 128
+#pragma unroll
+    for (int e = 0; e < 16; ++e) U[e] = ((unsigned long long)T[e] + off) << (8 * (8 - D));
+#pragma unroll 1
     for (int s = 0; s < D; ++s) {
+        const float Ms = 1.5f * __int_as_float((150 - 8 * s) << 23);
+        const uint32_t mb = __float_as_uint(Ms) - 128u;
         uint32_t v[8], w[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) v[j] = oz_word<D>(T[2 * j], T[2 * j + 1], s);
+        for (int j = 0; j < 8; ++j) {
+            const float f0 = __fsub_rn(__uint_as_float(mb + (uint32_t)(U[2 * j] >> 56)), Ms);
+            const float f1 = __fsub_rn(__uint_as_float(mb + (uint32_t)(U[2 * j + 1] >> 56)), Ms);
+            v[j] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+            U[2 * j] <<= 8;
+            U[2 * j + 1] <<= 8;
+        }
 #pragma unroll
         for (int j = 0; j < 8; ++j) w[j] = swap ? v[j ^ 4] : v[j];
         stg256(dst + (size_t)s * 2048, w);

@@ -45,7 +45,6 @@ namespace kevd {
 namespace {
 
 constexpr int kQ = 16;
-constexpr int kChunk = 16;
 constexpr int kDrainWarps = 16;
 constexpr int kThreads = (2 + kDrainWarps) * 32;
 constexpr int kM = 128;
@@ -111,19 +110,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int nj = (n + kN - 1) / kN;
     const int64_t ntile = (M + kM - 1) / kM * nj;
     const int nq = (K + kQ - 1) / kQ;
-    const int nchunk = (nq + kChunk - 1) / kChunk;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;
     const uint32_t bar0 = smem_u32(&bars[0]);
-    auto full = [&](int64_t g) { return bar0 + 8u * (uint32_t)(g % kStages); };
-    auto empty = [&](int64_t g) { return bar0 + 8u * (uint32_t)(kStages + g % kStages); };
+    auto full = [&](int st) { return bar0 + 8u * (uint32_t)st; };
+    auto empty = [&](int st) { return bar0 + 8u * (uint32_t)(kStages + st); };
     auto acc_full = [&](int a) { return bar0 + 8u * (uint32_t)(2 * kStages + a); };
     auto acc_empty = [&](int a) { return bar0 + 8u * (uint32_t)(2 * kStages + NA + a); };
 
     if (tid == 0) {
-        for (int q = 0; q < kStages; ++q) {
+        for (int q = 0; q < kStages; ++q) {   // (stage indexes and phases run by increments: no divisions in the loops)
             mbar_init(full(q), 1);
             mbar_init(empty(q), 1);
         }
@@ -147,28 +145,32 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
 
     if (wid == 0) {
-        // ---- TMA producer: quarter g = (tile iteration) nq + q ----
+        // ---- copies of the quarters into the ring ----
         if (lane == 0) {
-            int64_t g = 0;
+            int st_ = 0;
+            uint32_t ph = 1;                                       // the first pass finds the stages empty
             bool ok = true;
             for (int64_t t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
                 const uint16_t* pa = A.p + oz_tile_at((t / nj) * kM, 0, 0, A.nq, D);
                 const uint16_t* pb = B.p + oz_tile_at((t % nj) * kN, 0, 0, B.nq, D);
-                for (int q = 0; q < nq; ++q, ++g) {
-                    if (g >= kStages && !mbar_wait_or_fail(empty(g), (uint32_t)(g / kStages - 1) & 1, &s_fail)) {
-                        ok = false;
-                        break;
-                    }
-                    const uint32_t dst = base + (uint32_t)(g % kStages) * kStage;
-                    mbar_expect_tx(full(g), kStage);
-                    bulk_g2s(dst, pa + (size_t)q * D * 2048, kStageA, full(g));
-                    const uint16_t* src = pb + (size_t)q * D * 2048;
+                for (int q = 0; q < nq; ++q) {
+                    ok = mbar_wait_quick(empty(st_), ph, &s_fail);
+                    if (!ok) break;
+                    const uint32_t dst = base + (uint32_t)st_ * kStage;
+                    mbar_expect_tx(full(st_), kStage);
+                    bulk_g2s(dst, pa, kStageA, full(st_));
                     if (kN == 128) {
-                        bulk_g2s(dst + kStageA, src, D * kPlaneB, full(g));
+                        bulk_g2s(dst + kStageA, pb, D * kPlaneB, full(st_));
                     } else {
 #pragma unroll
                         for (int s = 0; s < D; ++s)
-                            bulk_g2s(dst + kStageA + s * kPlaneB, src + s * 2048, kPlaneB, full(g));
+                            bulk_g2s(dst + kStageA + s * kPlaneB, pb + s * 2048, kPlaneB, full(st_));
+                    }
+                    pa += D * 2048;
+                    pb += D * 2048;
+                    if (++st_ == kStages) {
+                        st_ = 0;
+                        ph ^= 1;
                     }
                 }
             }
@@ -176,57 +178,58 @@ __global__ void __launch_bounds__(kThreads, 1)
                 s_fail = 1;
                 atomicOr(flags, 4);
             }
-            for (int64_t j = g > kStages ? g - kStages : 0; j < g; ++j) mbar_wait(full(j), (uint32_t)(j / kStages) & 1);
+            // this CTA's copies have landed before it exits: every stage's last phase (a stage
+            // never used waits on the phase before its first, which is complete)
+            for (int j = 0; j < kStages; ++j) mbar_wait(full(j), j < st_ ? ph ^ 1 : ph);
         }
     } else if (wid == 1) {
-        // ---- MMA issuer: the whole warp walks the quarters, one elected lane issues ----
-        int64_t g = 0, c = 0, last = -1;
-        bool ok = true;
-        for (int64_t t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
-            for (int q = 0; q < nq; ++q, ++g) {
-                const bool first = (q % kChunk) == 0, end = (q % kChunk) == kChunk - 1 || q == nq - 1;
-                bool w = mbar_wait_or_fail(full(g), (uint32_t)(g / kStages) & 1, &s_fail);
-                if (first && c > 0)                            // the drain has read the previous chunk
-                    for (int a = 0; a < NA && w; ++a)
-                        w = mbar_wait_or_fail(acc_empty(a), (uint32_t)(c - 1) & 1, &s_fail);
-                ok = __all_sync(0xffffffffu, w);
-                if (!ok) break;
-                tc_fence_after();
-                const uint32_t sa = base + (uint32_t)(g % kStages) * kStage;
-                const uint64_t da = sw32_desc(sa), db = sw32_desc(sa + kStageA);
-                if (elect_one()) {
-                    if (!end) {
-                        oz_issue_planes<D, kN, STRICT>(tmem, da, db, kPlaneA >> 4, kPlaneB >> 4, kIdesc, first);
-                    } else {
-#pragma unroll
-                        for (int a = 0; a < NA; ++a) {
-                            oz_issue_acc<D, kN>(a, tmem, da, db, kPlaneA >> 4, kPlaneB >> 4, kIdesc, first);
-                            umma_commit(acc_full(a));
-                        }
+        // ---- MMA issuer: one elected lane ----
+        if (elect_one()) {
+            OzIssuer<D, kN, STRICT> is{tmem, kIdesc, kPlaneA >> 4, kPlaneB >> 4, acc_full(0), acc_empty(0), &s_fail};
+            int st_ = 0, prev = -1;
+            uint32_t ph = 0, prev_ph = 0;
+            bool ok = true;
+            for (int64_t t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+                for (int q = 0; q < nq && ok; ++q) {
+                    ok = mbar_wait_quick(full(st_), ph, &s_fail);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint32_t sa = base + (uint32_t)st_ * kStage;
+                    ok = is.quarter(sw32_desc(sa), sw32_desc(sa + kStageA), q, nq);
+                    umma_commit(empty(st_));
+                    prev = st_;
+                    prev_ph = ph;
+                    if (++st_ == kStages) {
+                        st_ = 0;
+                        ph ^= 1;
                     }
-                    umma_commit(empty(g));
                 }
-                __syncwarp();
-                last = g;
-                c += end;
             }
+            if (!ok) {
+                s_fail = 1;
+                atomicOr(flags, 4);
+            }
+            if (prev >= 0) mbar_wait(empty(prev), prev_ph);        // the last commit covers the earlier ones
         }
-        if (!ok && lane == 0) {
-            s_fail = 1;
-            atomicOr(flags, 4);
-        }
-        if (last >= 0) mbar_wait(empty(last), (uint32_t)(last / kStages) & 1);
+        __syncwarp();
     } else {
         // ---- drain and epilogue: TMEM lane quarter wid % 4, columns [16 h + 64 g, + 16) ----
         const int wq = wid & 3, h = (wid - 2) >> 2;
         const int m = 32 * wq + lane;
-        const uint32_t lane_off = (uint32_t)(32 * wq) << 16;
         const int pcols = (ncols + kQ - 1) / kQ * kQ;   // new columns' planes: zeros past ncols up to 16
-        int64_t c = 0;
+        OzDrain<D, kN, STRICT> dr{tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(16 * h), acc_full(0), acc_empty(0),
+                                  &s_fail};
         bool ok = true;
-        for (int64_t t = blockIdx.x; t < ntile && ok; t += gridDim.x) {
+        for (int64_t t = blockIdx.x; t < ntile; t += gridDim.x) {
             const int64_t i0 = (t / nj) * kM;
             const int j0 = (int)(t % nj) * kN;
+            // row and column exponents of the tile, loaded while its products run (lane 16 g + e
+            // holds column j0 + 64 g + 16 h + e's)
+            const int64_t gi = i0 + m;
+            const int cj = j0 + 64 * (lane >> 4) + 16 * h + (lane & 15);
+            const int ei = gi < M ? (ea ? ea[gi] : A.e_const) : -900;
+            const int ejl = cj < ncols ? (eb ? eb[cj] : B.e_const) : -900;
+            const double dinv = rowdiv && gi < M ? 1.0 / rowdiv[gi] : 1.0;
             long long Tacc[16 * kNH];
             float Macc[16 * kNH];
 #pragma unroll
@@ -234,60 +237,35 @@ __global__ void __launch_bounds__(kThreads, 1)
                 Tacc[e] = 0;
                 Macc[e] = 0.f;
             }
-            for (int ch = 0; ch < nchunk && ok; ++ch, ++c) {
-#pragma unroll
-                for (int a = 0; a < NA; ++a) {
-                    const bool w = a == 0 ? mbar_wait_sleep(acc_full(a), (uint32_t)c & 1, &s_fail, 64)
-                                          : mbar_wait_or_fail(acc_full(a), (uint32_t)c & 1, &s_fail);
-                    ok = __all_sync(0xffffffffu, w);
-                    if (!ok) break;
-                    tc_fence_after();
-#pragma unroll
-                    for (int half = 0; half < kNH; ++half) {
-                        uint32_t r[16];
-                        tmem_ld16_async(tmem + lane_off + (uint32_t)(kN * a + 16 * h + 64 * half), r);
-                        tmem_wait_ld16(r);
-                        if (half == kNH - 1) {                  // TMEM free for the next chunk or tile
-                            tc_fence_before();
-                            __syncwarp();
-                            if (lane == 0) mbar_arrive(acc_empty(a));
-                        }
-                        oz_add_level<D, STRICT>(a, r, Tacc + 16 * half, Macc + 16 * half);
-                    }
-                }
-            }
+            ok = dr.tile(nq, Tacc, Macc);
             if (!ok) break;
-            const int64_t gi = i0 + m;
-            if (gi < M && D == kDigits && pout) {
-                // the solve: C and the seven planes of its 16 columns (exponent 1), each
-                // plane's 32 bytes of the row as one store
-                const int ei = ea ? ea[gi] : A.e_const;
-                long long Tq[16];
+            // values four at a time (rolled, the sums moving down: see oz_mma.cuh on code size)
+            double* cp = Cout + gi + (int64_t)(j0 + 16 * h) * ldc;
+#pragma unroll 1
+            for (int u = 0; u < 4 * kNH; ++u) {
+                const int c0 = 4 * u + 48 * (u >> 2);           // 16 columns, then 16 more 64 further
+                long long Tq[4];
 #pragma unroll
-                for (int e = 0; e < 16; ++e) {
-                    const int gj = j0 + 16 * h + e;
+                for (int e = 0; e < 4; ++e) {
+                    const int ej = __shfl_sync(0xffffffffu, ejl, 4 * u + e);
                     double v = 0.0;
-                    if (gj < ncols) {
-                        const int ej = eb ? eb[gj] : B.e_const;
-                        if (ei > -900 && ej > -900) v = oz_value<STRICT>(Tacc[e], Macc[e], ei + ej - 12);
-                        Cout[gi + (int64_t)gj * ldc] = v;
-                    }
-                    Tq[e] = oz_T_f64<kDigits>(v, 1);
+                    if (ei > -900 && ej > -900)
+                        v = STRICT ? oz_value_strict(Tacc[e], Macc[e], ei + ej - 12)
+                                   : oz_value(Tacc[e], Macc[e], ei + ej - 12);
+                    if (gi < M && j0 + 16 * h + c0 + e < ncols) cp[(int64_t)(c0 + e) * ldc] = rowdiv ? v * dinv : v;
+                    Tq[e] = D == kDigits ? oz_T_f64<kDigits>(v, 1) : 0;
                 }
-                if (j0 + 16 * h < pcols) oz_store_quarter<kDigits>(pout, gi, (pk + j0) / 16 + h, pout_nq, Tq);
-            } else if (gi < M) {
-                const int ei = ea ? ea[gi] : A.e_const;
-                const double dinv = rowdiv ? 1.0 / rowdiv[gi] : 1.0;
 #pragma unroll
-                for (int e = 0; e < 16 * kNH; ++e) {
-                    const int gj = j0 + 64 * (e / 16) + 16 * h + e % 16;
-                    if (gj < ncols) {
-                        const int ej = eb ? eb[gj] : B.e_const;
-                        double v = 0.0;
-                        if (ei > -900 && ej > -900) v = oz_value<STRICT>(Tacc[e], Macc[e], ei + ej - 12);
-                        Cout[gi + (int64_t)gj * ldc] = rowdiv ? v * dinv : v;
-                    }
+                for (int e = 0; e < 16 * kNH - 4; ++e) {
+                    Tacc[e] = Tacc[e + 4];
+                    Macc[e] = Macc[e + 4];
                 }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) Tacc[16 * kNH - 4 + e] = Tq[e];
+            }
+            if constexpr (D == kDigits) {                       // the solve: the digits of F's new columns are now in Tacc
+                if (pout && gi < M && j0 + 16 * h < pcols)
+                    oz_store_quarter<kDigits>(pout, gi, (pk + j0) / 16 + h, pout_nq, Tacc);
             }
         }
         if (!ok && lane == 0) {
