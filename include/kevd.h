@@ -363,8 +363,9 @@ int eig_topk_lowmem(const double* X, int64_t N, int32_t d, double eps, const int
                     void* workspace, size_t ws_bytes, void* stream);
 
 /*
- * kevd_kernel_exp -- the exponential the FP64 engine on the tensor cores uses
- * for the Gaussian kernel values exp(-|x_i - x_s|^2 / eps) of Algorithm 2: out[i]
+ * kevd_kernel_exp -- the table-driven exponential behind the Gaussian kernel values
+ * exp(-|x_i - x_s|^2 / eps) of Algorithm 2 in the FP64 engine on the tensor cores (which
+ * evaluates the same table and series in fixed point throughout): out[i]
  * = exp(t[i]) for t[i] <= 0 within one ulp, 0 for t[i] <= -708 (a
  * table-driven method with its polynomial in fixed point, so that it runs on
  * the integer pipe).  t, out: device double[n] (out may alias t).  Enqueued on

@@ -35,7 +35,8 @@ static int tc_bn(int b) { return b <= 32 ? 32 : b <= 64 ? 64 : 128; }
 // N x b product arrays and the digit planes (OzWs) are carved after the rest;
 // rounds_max bounds the padding of F's planes (16 columns per round).
 static FactorWs carve_factor(void* base, int64_t N, int d, int r, int b, size_t* bytes, bool tc = false,
-                             PanelWs* pw = nullptr, bool oz = false, OzWs* ow = nullptr, int rounds_max = 0) {
+                             PanelWs* pw = nullptr, bool oz = false, OzWs* ow = nullptr, int rounds_max = 0,
+                             bool pl = false) {
     Carver c(base);
     const int64_t nt = (N + kBM - 1) / kBM;
     FactorWs w{};
@@ -57,12 +58,13 @@ static FactorWs carve_factor(void* base, int64_t N, int d, int r, int b, size_t*
     w.Lc = c.take<double>((size_t)b * b);
     if (tc) {
         const int BN = tc_bn(b);
-        PanelWs p;
+        PanelWs p{};
         p.panel = c.take<uint16_t>((size_t)tc_chunks(d, r) * 2 * BN * kTcBK);
         p.Lf = c.take<float>((size_t)BN * BN);
         p.nS = c.take<float>(BN);
         p.pidx = c.take<int64_t>(BN);
         p.err = c.take<int>(4);
+        if (pl) p.planes = c.take<uint16_t>(tc_plane_bytes(N, d, r, &p.nxh, &p.nH) / 2);
         if (pw) *pw = p;
     }
     if (oz && !tc) {
@@ -332,85 +334,176 @@ __global__ void k_blockH(FactorWs w, int d, int b, double inv_eps) {
 
 // ---------------------------------------------------------------------------
 // a4: Algorithm 3 (ARPC) or the greedy acceptance (b = 1, accept iff H > 0).
-// One block; H lives in shared memory (b*b doubles).
+//
+// Algorithm 3 is a chain of b steps (accept H(i,i), scale a column by 1 / sqrt(H(i,i)),
+// subtract its outer product), and one dependent FP64 operation takes 64 cycles and
+// occupies a quarter of an SM's FP64 pipe for as long.  So the steps run in panels of 16
+// columns on four warps, one matrix row per thread: every warp carries the panel's
+// diagonal in its lanes and takes the decision itself (one barrier per accepted
+// proposal, none per rejected one), the square root and the division share one
+// reciprocal root (11 operations instead of ~20), and the columns right of the panel are
+// updated 16 pivots at a time by all CTAs of a cluster, with H in global memory.  Every
+// entry sees the same subtractions in the same order as with one step at a time.
+// Measured per round at b = 128 / 64: 205 / 82 us (one CTA with two barriers and the whole
+// square per step: 556 / 190 us).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void reject_body(FactorWs w, int b, int r, int greedy, uint64_t seed, int rnd,
-                                            int64_t* __restrict__ pivots, double* smem) {
-    double* Hs = smem;                 // b*b
-    double* Lcol = Hs + (size_t)b * b; // b
-    double* rho0 = Lcol + b;           // b
-    double* zs = rho0 + b;             // b
-    __shared__ int s_acc, s_m, s_go;
-    FactorState* st = w.st;
-    const int tid = threadIdx.x;
-    if (tid == 0) {
-        s_go = !st->done;
-        s_m = 0;
-    }
-    __syncthreads();
-    if (!s_go) return;
-    const int k = st->k;
-    for (int e = tid; e < b * b; e += blockDim.x) Hs[e] = w.H[e];
-    __syncthreads();
-    for (int e = tid; e < b; e += blockDim.x) {
-        rho0[e] = Hs[(size_t)e * b + e];
-        zs[e] = greedy ? 0.0 : philox_uniform(seed, 1u, (uint32_t)rnd, (uint32_t)e);   // the z of every proposal
-    }
-    __syncthreads();
-    for (int i = 0; i < b; ++i) {
-        if (tid == 0) {
-            const double hii = Hs[(size_t)i * b + i];
-            int acc;
-            if (greedy) {
-                acc = hii > 0.0;
-            } else {
-                acc = hii > 0.0 && zs[i] * rho0[i] < hii;
-            }
-            if (k + s_m >= r) acc = 0;
-            if (acc) w.tpos[s_m++] = i;
-            s_acc = acc;
-        }
-        __syncthreads();
-        const int accepted = s_acc;
-        __syncthreads();   // every thread has read s_acc before thread 0 rewrites it
-        if (!accepted) continue;
-        const double piv = sqrt(Hs[(size_t)i * b + i]);
-        for (int l = i + tid; l < b; l += blockDim.x) {
-            // greedy divides the residual column by sqrt(H) directly; Algorithm 3
-            // scales the whole column H(i:b, i) by 1/sqrt(H(i,i)).
-            const double v = (greedy && l == i) ? piv : Hs[(size_t)l * b + i] / piv;
-            Lcol[l] = v;
-            w.Lfull[(size_t)l * b + i] = v;
-        }
-        __syncthreads();
-        const int n = b - i - 1;
-        for (int e = tid; e < n * n; e += blockDim.x) {
-            const int l = i + 1 + e / n, mm = i + 1 + e % n;
-            Hs[(size_t)l * b + mm] -= Lcol[l] * Lcol[mm];
-        }
-        __syncthreads();
-    }
-    __syncthreads();
-    const int m = s_m;
-    for (int e = tid; e < m * m; e += blockDim.x) {
-        const int a = e / m, a2 = e % m;
-        w.Lc[(size_t)a * b + a2] = a2 <= a ? w.Lfull[(size_t)w.tpos[a] * b + w.tpos[a2]] : 0.0;
-    }
-    for (int a = tid; a < m; a += blockDim.x) {
-        w.acc_pos[a] = w.tpos[a];
-        pivots[k + a] = w.prop[w.tpos[a]];
-    }
-    if (tid == 0) {
-        st->m = m;
-        if (greedy && m == 0) st->done = 1;   // greedy stops once H <= 0
-    }
+constexpr int kRejW = 16;         // panel columns
+constexpr int kRejThreads = 256;
+constexpr int kRejCluster = 8;    // CTAs per problem
+
+struct RejShared {
+    double L[kRejW][128];         // panel columns: L(c0 + t, c0 + j)
+    double zr[128];               // z_i rho0_i
+    int tpos[128];
+    int m;
+};
+
+// s = sqrt(h) and y = 1 / sqrt(h) for normal h: Halley's iteration on a reciprocal-root
+// estimate (relative error below 2^-22, cubed), then one correction of s = h y by its exact
+// residual (P. Markstein, IBM J. Res. Dev. 34(1), 1990).
+__device__ __forceinline__ void rej_root(double h, double& s, double& y) {
+    double y0;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(h));
+    const double e = fma(-(h * y0), y0, 1.0);
+    y = fma(fma(e, 0.375, 0.5), y0 * e, y0);
+    const double s0 = h * y;
+    s = fma(fma(-s0, s0, h), 0.5 * y, s0);
 }
 
-__global__ void __launch_bounds__(1024) k_reject(FactorWs w, int b, int r, int greedy, uint64_t seed, int rnd,
-                                                 int64_t* __restrict__ pivots) {
-    extern __shared__ double smem_rej[];
-    reject_body(w, b, r, greedy, seed, rnd, pivots, smem_rej);
+// c / s, y = 1 / s up to rounding: the quotient corrected by its exact residual (as above).
+__device__ __forceinline__ double rej_quot(double c, double s, double y) {
+    const double q = c * y;
+    return fma(fma(-q, s, c), y, q);
 }
+
+// All threads of the cluster; what they wrote to global memory before is visible after.
+__device__ __forceinline__ void rej_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// One cluster of kRejCluster CTAs per problem, `cta` the rank in it.  H is overwritten.
+__device__ __forceinline__ void arpc_reject_body(FactorWs w, int b, int r, uint64_t seed, int rnd,
+                                                 int64_t* __restrict__ pivots, RejShared& sh, int cta) {
+    FactorState* st = w.st;
+    if (st->done) return;                                        // the same in every CTA
+    const int k = st->k;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    if (cta == 0) {
+        for (int e = tid; e < b; e += blockDim.x)
+            sh.zr[e] = philox_uniform(seed, 1u, (uint32_t)rnd, (uint32_t)e) * w.H[(size_t)e * b + e];
+        __syncthreads();
+    }
+    int m = 0;
+    for (int c0 = 0; c0 < b; c0 += kRejW) {
+        const int nw = min(kRejW, b - c0);
+        unsigned mask = 0;                                       // accepted columns of the panel
+        if (cta == 0 && wid < 4) {
+            const int l = c0 + tid;                              // this thread's row
+            const bool row = tid < b - c0;
+            double c[kRejW];
+#pragma unroll
+            for (int j = 0; j < kRejW; ++j)
+                c[j] = row && j < nw && l >= c0 + j ? __ldcg(w.H + (size_t)l * b + c0 + j) : 0.0;
+            double d = lane < nw ? __ldcg(w.H + (size_t)(c0 + lane) * (b + 1)) : 0.0;
+            const double zr = lane < nw ? sh.zr[c0 + lane] : 0.0;
+#pragma unroll
+            for (int j = 0; j < kRejW; ++j) {
+                if (j >= nw) break;
+                const double h = __shfl_sync(0xffffffffu, d, j);
+                if (!(h > 0.0 && __shfl_sync(0xffffffffu, zr, j) < h) || k + m >= r) continue;
+                double s, y, v;
+                if (h > 0x1p-900) {
+                    rej_root(h, s, y);
+                    v = rej_quot(c[j], s, y);
+                } else {
+                    s = sqrt(h);
+                    v = c[j] / s;
+                }
+                sh.L[j][tid] = v;
+                asm volatile("bar.sync 1, 128;" ::: "memory");
+                const double lj = sh.L[j][lane & (kRejW - 1)];
+                if (lane > j) d = fma(-lj, lj, d);
+#pragma unroll
+                for (int j2 = j + 1; j2 < kRejW; ++j2) c[j2] = fma(-v, sh.L[j][j2], c[j2]);
+                if (row && l >= c0 + j) w.Lfull[(size_t)l * b + c0 + j] = v;
+                if (tid == 0) sh.tpos[m] = c0 + j;
+                mask |= 1u << j;
+                ++m;
+            }
+            if (tid == 0) {
+                sh.m = m;
+                w.tpos[b - 1] = (int)mask;                       // (free until the end: positions are in sh.tpos)
+            }
+        }
+        const int n0 = c0 + kRejW;
+        rej_sync();
+        if (n0 >= b) break;
+        // columns n0 .. of the rows below the panel, all CTAs: a warp takes a row
+        mask = (unsigned)*(volatile int*)&w.tpos[b - 1];
+        m = cta == 0 ? sh.m : 0;
+        const int cnt = __popc(mask);
+        for (int e = tid; e < cnt * (b - n0); e += blockDim.x) {   // the accepted columns into shared memory, packed
+            const int a = e / (b - n0), l = e % (b - n0);
+            unsigned t = mask;
+            for (int q = 0; q < a; ++q) t &= t - 1;
+            sh.L[a][l] = __ldcg(w.Lfull + (size_t)(n0 + l) * b + c0 + __ffs(t) - 1);
+        }
+        __syncthreads();
+        for (int l = cta * (kRejThreads / 32) + wid; l < b - n0; l += kRejCluster * (kRejThreads / 32)) {
+            double* Hr = w.H + (size_t)(n0 + l) * b + n0;
+            double x[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) x[u] = lane + 32 * u <= l ? __ldcg(Hr + lane + 32 * u) : 0.0;
+            for (int a = 0; a < cnt; ++a) {
+                const double v = sh.L[a][l];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (32 * u <= l) x[u] = fma(-v, sh.L[a][(lane + 32 * u) & 127], x[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (lane + 32 * u <= l) Hr[lane + 32 * u] = x[u];
+        }
+        rej_sync();
+    }
+    if (cta != 0) return;
+    // (CTA 0's own columns of Lfull and its list of positions: ordered by the last barrier)
+    m = sh.m;
+    for (int e = tid; e < m * m; e += blockDim.x) {
+        const int a = e / m, a2 = e % m;
+        w.Lc[(size_t)a * b + a2] = a2 <= a ? w.Lfull[(size_t)sh.tpos[a] * b + sh.tpos[a2]] : 0.0;
+    }
+    for (int a = tid; a < m; a += blockDim.x) {
+        w.acc_pos[a] = sh.tpos[a];
+        pivots[k + a] = w.prop[sh.tpos[a]];
+    }
+    if (tid == 0) st->m = m;
+}
+
+// Greedy (b = 1): accept iff H > 0, L = sqrt(H).
+__device__ __forceinline__ void greedy_reject_body(FactorWs w, int r, int64_t* __restrict__ pivots) {
+    FactorState* st = w.st;
+    if (st->done || threadIdx.x != 0) return;
+    const int k = st->k;
+    const double h = w.H[0];
+    const int m = h > 0.0 && k < r ? 1 : 0;
+    if (m) {
+        w.Lc[0] = sqrt(h);
+        w.acc_pos[0] = 0;
+        pivots[k] = w.prop[0];
+    } else {
+        st->done = 1;                                            // greedy stops once H <= 0
+    }
+    st->m = m;
+}
+
+__global__ void __cluster_dims__(kRejCluster, 1, 1) __launch_bounds__(kRejThreads)
+    k_reject(FactorWs w, int b, int r, uint64_t seed, int rnd, int64_t* __restrict__ pivots) {
+    __shared__ RejShared sh;
+    arpc_reject_body(w, b, r, seed, rnd, pivots, sh, blockIdx.x);
+}
+
+__global__ void k_reject_greedy(FactorWs w, int r, int64_t* __restrict__ pivots) { greedy_reject_body(w, r, pivots); }
 
 // ---------------------------------------------------------------------------
 // a5 + a6: the kernel-column engine (FP64).  Tile = 64 rows x BN = 8*TN columns.
@@ -651,52 +744,79 @@ __global__ void __launch_bounds__(128) k_ozpanel(FactorWs w, OzWs o, int64_t N, 
     gather(o.Fp, o.PFp, o.ldF / 16, st->kp / 16);
 }
 
-// L(T,T)^-1 of the round (lower triangular, m x m) and its digit planes: rows j
-// of Lp (exponent le_j), columns past m and rows past m zero.  One block;
-// thread c forms column c by forward substitution on L e_c (L staged in shared
-// memory, read by broadcast).  Each round's L is the Cholesky factor of
-// Algorithm 3's accepted block, whose accept test keeps it well conditioned, so
-// multiplying by the explicit inverse agrees with substitution to rounding
-// (measured 2e-15 on KS data).
-__global__ void __launch_bounds__(128) k_linv(FactorWs w, OzWs o, int b) {
-    extern __shared__ double Ls[];
+// L(T,T)^-1 of the round (lower triangular, m x m).  Each round's L is the Cholesky
+// factor of Algorithm 3's accepted block, whose accept test keeps it well
+// conditioned, so multiplying by the explicit inverse agrees with substitution to
+// rounding (measured 2e-15 on KS data).  One warp per column c (forward substitution on
+// L x = e_c): lane holds the right-hand sides of rows lane + 32 u; a step divides one of
+// them (by a reciprocal and the residual's correction) and subtracts it from the rows
+// below.  Four warps per CTA, so that each has a quarter of an SM's FP64 pipe to itself
+// (one CTA for all columns: 489 us per round at b = 128, its chain of ~8,000 dependent
+// operations; this one: 62 us, 4 more for the planes).
+constexpr int kLinvWarps = 4;
+__global__ void __launch_bounds__(32 * kLinvWarps) k_linv(FactorWs w, OzWs o, int b) {
+    extern __shared__ double Ls[];                               // column l of L at Ls + l (m + 1), rows l .. m - 1 used
     const FactorState* st = w.st;
     if (st->done || st->m == 0) return;
-    const int m = st->m;
+    const int m = st->m, lane = threadIdx.x & 31;
+    const int c = blockIdx.x * kLinvWarps + (threadIdx.x >> 5);
+    const int cf = blockIdx.x * kLinvWarps;                      // no column of this CTA reads L's columns before cf
+    if (cf >= m) return;
+    const int ld = m + 1;
+    double* inv = Ls + (size_t)m * ld;                            // 1 / L(l, l)
     for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
         const int j = e / m, l = e % m;
-        Ls[e] = l <= j ? w.Lc[(size_t)j * b + l] : 0.0;
+        if (l >= cf && l <= j) Ls[(size_t)l * ld + j] = w.Lc[(size_t)j * b + l];
     }
     __syncthreads();
-    const int c = threadIdx.x;
-    if (c < b) {
-        for (int j = 0; j < b; ++j) {
-            double x = 0.0;
-            if (c < m && j >= c && j < m) {
-                if (j == c) {
-                    x = 1.0 / Ls[j * m + j];
-                } else {
-                    double s = 0.0;
-                    for (int l = c; l < j; ++l) s = fma(Ls[j * m + l], o.Linv[(size_t)l * o.ldLi + c], s);
-                    x = -s / Ls[j * m + j];
-                }
-            }
-            o.Linv[(size_t)j * o.ldLi + c] = x;
-        }
-    }
+    for (int l = cf + threadIdx.x; l < m; l += blockDim.x) inv[l] = 1.0 / Ls[(size_t)l * ld + l];
     __syncthreads();
-    if (c < b) {   // row c: exponent and planes (columns < m hold the row, the rest zero)
-        const double* row = o.Linv + (size_t)c * o.ldLi;
-        double mx = 0.0;
-        for (int l = 0; l < m; ++l) mx = fmax(mx, fabs(row[l]));
-        const int E = exp_of(mx);
-        o.le[c] = E;
-        for (int q = 0; q < o.ldR / 16; ++q) {
-            long long t[16];
+    if (c >= m) return;
+    double x[4];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<kDigits>(16 * q + e < m ? row[16 * q + e] : 0.0, E);
-            oz_store_quarter<kDigits>(o.Lp, c, q, o.ldR / 16, t);
+    for (int u = 0; u < 4; ++u) x[u] = lane + 32 * u == c ? 1.0 : 0.0;
+    for (int l = c; l < m; ++l) {
+        const double* Ll = Ls + (size_t)l * ld;
+        const double rhs = l < 32 ? x[0] : l < 64 ? x[1] : l < 96 ? x[2] : x[3];
+        double v = rhs * inv[l];
+        v = fma(fma(-v, Ll[l], rhs), inv[l], v);
+        v = __shfl_sync(0xffffffffu, v, l & 31);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = lane + 32 * u;
+            if (32 * u + 31 > l) {                               // rows below l in this group
+                if (j == l) x[u] = v;
+                else if (j > l && j < m) x[u] = fma(-Ll[j], v, x[u]);
+            } else if (j == l) {
+                x[u] = v;
+            }
         }
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (lane + 32 * u < m) o.Linv[(size_t)(lane + 32 * u) * o.ldLi + c] = lane + 32 * u >= c ? x[u] : 0.0;
+}
+
+// Digit planes of the rows of L^-1 (columns past the diagonal and rows past m zero) and
+// their exponents; one warp per row.
+__global__ void __launch_bounds__(128) k_linv_planes(FactorWs w, OzWs o, int b) {
+    const FactorState* st = w.st;
+    if (st->done || st->m == 0) return;
+    const int m = st->m, lane = threadIdx.x & 31, j = blockIdx.x * 4 + (threadIdx.x >> 5), nq = o.ldR / 16;
+    if (j >= b) return;
+    const double* row = o.Linv + (size_t)j * o.ldLi;
+    unsigned long long mx = 0;
+    for (int l = lane; l <= j && j < m; l += 32)
+        mx = max(mx, (unsigned long long)__double_as_longlong(row[l]) & 0x7FFFFFFFFFFFFFFFull);
+#pragma unroll
+    for (int q = 16; q; q >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, q));
+    const int E = exp_of(__longlong_as_double((long long)mx));
+    if (lane == 0) o.le[j] = E;
+    if (lane < nq) {
+        long long t[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<kDigits>(j < m && 16 * lane + e <= j ? row[16 * lane + e] : 0.0, E);
+        oz_store_quarter<kDigits>(o.Lp, j, lane, nq, t);
     }
 }
 
@@ -704,7 +824,11 @@ __global__ void __launch_bounds__(128) k_linv(FactorWs w, OzWs o, int b) {
 // values exp(-(|x_i|^2 + |x_s|^2 - 2 x_i.x_s) / eps) (1 at the pivot itself)
 // minus Df, as digit planes with one exponent per row (the row maximum over
 // the round's pivots).  Block: 32 rows x ldR / 16 warps, warp g taking the quarter of
-// 16 pivots [16 g, 16 g + 16).
+// 16 pivots [16 g, 16 g + 16).  Only the squared distance is formed in FP64 (two
+// operations, 17 cycles per warp and SM each); the scaling by 1 / eps, the exponential
+// (kexp_q62), the difference and the digits are 64-bit fixed point.  Bound: the integer
+// pipe (HBM: 30 bytes per value, 0.5 ms).  N = 1M, b = 128: 2.8 ms per round with nine FP64
+// operations per value, 1.6 ms now.
 __global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, double inv_eps,
                                                const unsigned long long* __restrict__ tblg) {
     const FactorState* st = w.st;
@@ -725,44 +849,63 @@ __global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, do
     const int l0 = 16 * g;
     for (int64_t row0 = (int64_t)blockIdx.x * 32; row0 < N; row0 += (int64_t)gridDim.x * 32) {
         const int64_t row = row0 + lane;
-        double R[16], df[16];
         const bool on = row < N;
         const double xi = on ? w.xn[row] : 0.0;
+        long long R[16];                                       // units of 2^-62
+        unsigned long long mx = 0;
+        // four values at a time, the next four in flight; rolled, R moving down
+        double dx[4], df[4];
+        auto load = [&](int u) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int64_t at = row + (int64_t)(l0 + e) * w.ldD;
-            const bool in = on && l0 + e < m;
-            R[e] = in ? w.Dx[at] : 0.0;
-            df[e] = in && k > 0 ? w.Df[at] : 0.0;
-        }
-        unsigned long long mx = 0;                             // max |R| as the bits of a non-negative double
-#pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            const int l = l0 + e;
-            double rv = 0.0;
-            if (on && l < m) {
-                double kv = 1.0;
-                if (s_row[l] != row) {
-                    double d2 = fma(-2.0, R[e], xi + s_xn[l]);
-                    if (__double_as_longlong(d2) < 0) d2 = 0.0;     // negative rounding residue
-                    kv = kexp(-d2 * inv_eps, tbl);
-                }
-                rv = kv - df[e];
+            for (int e = 0; e < 4; ++e) {
+                const int64_t at = row + (int64_t)(l0 + 4 * u + e) * w.ldD;
+                const bool in = on && l0 + 4 * u + e < m;
+                dx[e] = in ? w.Dx[at] : 0.0;
+                df[e] = in && k > 0 ? w.Df[at] : 0.0;
             }
-            R[e] = rv;
-            mx = max(mx, (unsigned long long)__double_as_longlong(rv) & 0x7FFFFFFFFFFFFFFFull);
+        };
+        load(0);
+#pragma unroll 1
+        for (int u = 0; u < 4; ++u) {
+            double cx[4], cf[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                cx[e] = dx[e];
+                cf[e] = df[e];
+            }
+            if (u < 3) load(u + 1);
+#pragma unroll
+            for (int e = 0; e < 12; ++e) R[e] = R[e + 4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int l = l0 + 4 * u + e;
+                long long v = 0;
+                if (on && l < m) {
+                    const long long kv = s_row[l] == row ? 1ll << 62
+                                                         : kexp_q62(fma(-2.0, cx[e], xi + s_xn[l]), inv_eps, tbl);
+                    v = kv - q62_of(cf[e]);
+                    mx = max(mx, (unsigned long long)(v < 0 ? -v : v));
+                }
+                R[12 + e] = v;
+            }
         }
         red[g][lane] = mx;
         __syncthreads();
         for (int q = 0; q < nq; ++q) mx = max(mx, red[q][lane]);
         __syncthreads();                                       // red is rewritten for the next rows
         if (!on) continue;
-        const int E = exp_of(__longlong_as_double((long long)mx));
-        if (g == 0) o.re[row] = E;
-        long long t[16];
+        // max |R| < 2^E, E = bits - 62; T = round(R 2^(54 - E)) of the digits (|T| < 2^54)
+        const int bits = 64 - __clzll((long long)mx);
+        if (g == 0) o.re[row] = mx ? bits - 62 : -900;
+        const int rs = bits - 54;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) t[e] = oz_T_f64<kDigits>(R[e], E);
-        oz_store_quarter<kDigits>(o.Rp, row, g, nq, t);
+        for (int e = 0; e < 16; ++e) {
+            unsigned long long a = (unsigned long long)(R[e] < 0 ? -R[e] : R[e]);
+            a = rs <= 0 ? a << min(-rs, 63) : ((a >> (rs - 1)) + 1) >> 1;
+            a = min(a, 0x3FFFFFFFFFFFFFull);
+            R[e] = R[e] < 0 ? -(long long)a : (long long)a;
+        }
+        oz_store_quarter<kDigits>(o.Rp, row, g, nq, R);
     }
 }
 
@@ -894,10 +1037,8 @@ void launch_blockH(const FactorWs& w, int d, int b, double inv_eps, cudaStream_t
 
 cudaError_t launch_reject(const FactorWs& w, int b, int r, int greedy, uint64_t seed, int rnd, int64_t* pivots,
                           cudaStream_t s) {
-    const size_t smem = ((size_t)b * b + 3 * (size_t)b) * sizeof(double);   // H, L column, rho0, z
-    const cudaError_t e = cudaFuncSetAttribute(k_reject, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_reject<<<1, b >= 32 ? 1024 : 128, smem, s>>>(w, b, r, greedy, seed, rnd, pivots);
+    if (greedy) k_reject_greedy<<<1, 32, 0, s>>>(w, r, pivots);
+    else k_reject<<<kRejCluster, kRejThreads, 0, s>>>(w, b, r, seed, rnd, pivots);
     return cudaGetLastError();
 }
 
@@ -914,10 +1055,20 @@ static int factor_rounds(const kevd_opts* o, int r, int b) {
     return r / b;
 }
 
-static size_t factor_ws_bytes(int64_t N, int d, int r, int b, bool tc, bool oz, int rounds_max) {
+static size_t factor_ws_bytes(int64_t N, int d, int r, int b, bool tc, bool oz, int rounds_max, bool pl) {
     size_t bytes = 0;
-    carve_factor(nullptr, N, d, r, b, &bytes, tc, nullptr, oz, nullptr, rounds_max);
+    carve_factor(nullptr, N, d, r, b, &bytes, tc, nullptr, oz, nullptr, rounds_max, pl);
     return bytes;
+}
+
+// The precision form's engine reads pre-split planes (as large as F) for blocks of b >= 32
+// (a round rewrites the 16-column groups it shares with the last, which smaller blocks would
+// do too often), while they stay within 48 GiB, so that a factor that only just fits the
+// card keeps the engine that needs no copy, and where the caller gives a workspace.
+static bool pl_engine_for(const kevd_opts* o, int64_t N, int d, int r, int b, bool workspace) {
+    int nxh, nH;
+    return workspace && o->precision == KEVD_PREC_BF16X3 && b >= 32 &&
+           tc_plane_bytes(N, d, r, &nxh, &nH) <= ((size_t)48 << 30);
 }
 
 // The FP64 path runs its engine on the tensor cores (FP64-accurate digit planes,
@@ -939,7 +1090,8 @@ size_t kevd_factor_ws_mode(int64_t N, int32_t d, int32_t r, const kevd_opts* o, 
     const int b = o->mode == KEVD_GREEDY ? 1 : o->block_b;
     if (b < 1 || b > 128) return 0;
     const bool tc = o->precision == KEVD_PREC_BF16X3;
-    return factor_ws_bytes(N, d, r, b, tc, oz_engine_for(o, N, b, allow_oz), factor_rounds(o, r, b));
+    return factor_ws_bytes(N, d, r, b, tc, oz_engine_for(o, N, b, allow_oz), factor_rounds(o, r, b),
+                           pl_engine_for(o, N, d, r, b, allow_oz));
 }
 
 size_t kevd_factor_ws(int64_t N, int32_t d, int32_t r, const kevd_opts* o) {
@@ -973,7 +1125,8 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
     PanelWs pw{};
     OzWs ow{};
     const bool oz = oz_engine_for(opts, N, b, allow_oz);
-    FactorWs w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b));
+    FactorWs w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b),
+                              pl_engine_for(opts, N, d, r, b, allow_oz));
     if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return KEVD_EWORKSPACE;
     // the digit planes: X and F (A operands), the pivot panels (B), R and L^-1 of each round
     const unsigned long long* exp_tbl = nullptr;
@@ -994,6 +1147,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
         if (tc) {
             KEVD_CUDA_TRY(cudaMemsetAsync(pw.err, 0, sizeof(int), s));
             k_prepare<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(Xf, N, d, w, rho);
+            if (pw.planes) launch_xsplit(Xf, N, d, pw, s);
         } else {
             k_prepare<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(Xd, N, d, w, rho);
             if (oz) {
@@ -1004,12 +1158,9 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
         }
     }
     KEVD_LAUNCH_CHECK();
-    const size_t rej_smem = ((size_t)b * b + 3 * (size_t)b) * sizeof(double);   // H, L column, rho0, z
-    KEVD_CUDA_TRY(cudaFuncSetAttribute(k_reject, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rej_smem));
     if (oz)
         KEVD_CUDA_TRY(cudaFuncSetAttribute(k_linv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)((size_t)b * b * sizeof(double))));
-    const int rej_threads = b >= 32 ? 1024 : 128;
+                                           (int)(((size_t)b * b + 2 * b) * sizeof(double))));
     const int tn = b <= 8 ? 1 : b <= 16 ? 2 : b <= 32 ? 4 : b <= 64 ? 8 : 16;
     switch (tn) {
         case 1: KEVD_CUDA_TRY(prepare_engine<1>()); break;
@@ -1036,7 +1187,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
         }
         {
             TraceScope tr(kStReject, s);
-            k_reject<<<1, rej_threads, rej_smem, s>>>(w, b, r, greedy, opts->seed, rnd, pivots);
+            KEVD_CUDA_TRY(launch_reject(w, b, r, greedy, opts->seed, rnd, pivots, s));
         }
         if (tc) {
             TraceScope tr(kStEngine, s);
@@ -1054,7 +1205,9 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
                 // R = K(:, T) - F F(T,:)^T; G = R L^-T into F(:, k:k+m), on the tensor cores; rho
                 k_rprep<<<(unsigned)std::min<int64_t>((N + 31) / 32, 152 * 8), 2 * ow.ldR, 0, s>>>(w, ow, N, inv_eps,
                                                                                                    exp_tbl);
-                k_linv<<<1, 128, (size_t)b * b * sizeof(double), s>>>(w, ow, b);
+                k_linv<<<(b + kLinvWarps - 1) / kLinvWarps, 32 * kLinvWarps, ((size_t)b * b + 2 * b) * sizeof(double), s>>>(
+                    w, ow, b);
+                k_linv_planes<<<(b + 3) / 4, 128, 0, s>>>(w, ow, b);
                 KEVD_CUDA_TRY(launch_ozmm(oR, oL, N, b, -2, w.st, Fd, ldf, ldf, ow.Fp, ow.ldF / 16, ow.flags, s));
                 k_rho_update<<<(unsigned)((N + 63) / 64), 256, 0, s>>>(w, Fd, ldf, rho, N);
             } else {
@@ -1170,10 +1323,11 @@ __global__ void k_blockH_b(const BatchProb* __restrict__ P) {
     blockH_body(p.w, p.d, p.b, p.inv_eps, blockIdx.x * kBlockHWarps + (threadIdx.x >> 5));   // pairs past b*b return
 }
 
-__global__ void __launch_bounds__(1024) k_reject_b(const BatchProb* __restrict__ P, int rnd) {
-    extern __shared__ double smem_rb[];
-    const BatchProb& p = P[blockIdx.x];
-    reject_body(p.w, p.b, p.r, 0, p.seed, rnd, p.pivots, smem_rb);
+__global__ void __cluster_dims__(kRejCluster, 1, 1) __launch_bounds__(kRejThreads)
+    k_reject_b(const BatchProb* __restrict__ P, int rnd) {   // a cluster per problem
+    __shared__ RejShared sh;
+    const BatchProb& p = P[blockIdx.y];
+    arpc_reject_body(p.w, p.b, p.r, p.seed, rnd, p.pivots, sh, blockIdx.x);
 }
 
 // Persistent engine over the work list; tile_off[q] = first item of problem q.
@@ -1264,13 +1418,12 @@ static int batch_enqueue_any(kevd_batch* h, cudaStream_t s) {
     using namespace kevd;
     const int np = h->nprob;
     k_prepare_b<<<dim3((unsigned)((h->nmax + 255) / 256), np), 256, 0, s>>>(h->dprobs);
-    const size_t rej_smem = ((size_t)h->bmax * h->bmax + 3 * (size_t)h->bmax) * sizeof(double);
     for (int rnd = 0; rnd < h->rounds; ++rnd) {
         k_propose_b<<<np, 1024, 0, s>>>(h->dprobs, rnd);
         k_gather_b<<<dim3((unsigned)((h->dmax + h->rmax + 7) / 8), np), 256, 0, s>>>(h->dprobs);
         k_blockH_b<<<dim3((h->bmax * h->bmax + kBlockHWarps - 1) / kBlockHWarps, 1, np), 32 * kBlockHWarps, 0, s>>>(
             h->dprobs);
-        k_reject_b<<<np, h->bmax >= 32 ? 1024 : 128, rej_smem, s>>>(h->dprobs, rnd);
+        k_reject_b<<<dim3(kRejCluster, np), kRejThreads, 0, s>>>(h->dprobs, rnd);
         for (const auto& g : h->groups) {
             int st;
             switch (g.tn) {
@@ -1358,10 +1511,8 @@ extern "C" int kevd_batch_create(const kevd_problem* probs, int nprob, int use_g
         b.w = carve_factor(base + offs[q], p.N, p.d, p.r, p.b, &bytes);
         h->states.push_back(b.w.st);
     }
-    const size_t rej_smem = ((size_t)bmax * bmax + 3 * (size_t)bmax) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_reject_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rej_smem);
-    bool ok = e == cudaSuccess &&
-              cudaMemcpyAsync(h->dprobs, hp.data(), sizeof(BatchProb) * nprob, cudaMemcpyHostToDevice, s) == cudaSuccess;
+    cudaError_t e = cudaSuccess;
+    bool ok = cudaMemcpyAsync(h->dprobs, hp.data(), sizeof(BatchProb) * nprob, cudaMemcpyHostToDevice, s) == cudaSuccess;
     // engine groups
     std::vector<std::vector<BatchProb>> gp(5);
     std::vector<std::vector<int64_t>> gt(5, std::vector<int64_t>(1, 0));

@@ -79,6 +79,9 @@ struct PanelWs {
     float* nS;         // BN: |x_s|^2 of the accepted pivots (FP32)
     int64_t* pidx;     // BN: row index of accepted pivot l (-1 past m)
     int* err;          // device-side wait timeout flag
+    // the engine from planes (null: the operands are split inside every round):
+    uint16_t* planes;  // BF16 hi/lo tiles of X (nxh half chunks of 32 columns) and F, per row block nH of them
+    int nxh, nH;
 };
 
 constexpr int kTcBM = 128;   // rows per tensor-core tile (UMMA M)
@@ -97,6 +100,14 @@ void launch_blockH(const FactorWs& w, int d, int b, double inv_eps, cudaStream_t
 cudaError_t launch_reject(const FactorWs& w, int b, int r, int greedy, uint64_t seed, int rnd, int64_t* pivots,
                           cudaStream_t s);
 void launch_finalize(const FactorWs& w, const double* rho, int64_t N, cudaStream_t s);
+
+// Bytes of PanelWs::planes, and the half chunks of X and of a row block.
+inline size_t tc_plane_bytes(int64_t N, int d, int r, int* nxh, int* nH) {
+    *nxh = (d + 31) / 32;
+    *nH = *nxh + (r + 31) / 32;
+    return (size_t)((N + 127) / 128) * *nH * 16384;
+}
+void launch_xsplit(const float* X, int64_t N, int d, const PanelWs& p, cudaStream_t s);
 
 // Host launcher of the tensor-core engine (engine_tc.cu).
 cudaError_t launch_engine_tc(const FactorWs& w, const PanelWs& p, const float* X, float* F, int64_t ldf,

@@ -210,3 +210,20 @@ def test_engine_exp_matches_cuda_exp(kevd):
     assert ours[t == 0].eq(1.0).all()
     low = torch.tensor([-708.0, -709.5, -745.2, -1e4, -float("inf")], dtype=torch.float64).cuda()
     assert kevd.kernel_exp(low).eq(0.0).all()
+
+
+# Algorithm 3 in panels of 16 columns on a cluster, the explicit inverse and the digit
+# planes of the round at the edges of panels (15, 16, 17), warps (31 .. 33), 64-row tiles
+# and the largest block; r = 2 b, so that the second round sees H after a first one.  N = 705
+# leaves a row block of 128 ragged.  Bars as test_arpc_matches_oracle.
+@pytest.mark.parametrize("b", [1, 2, 15, 16, 17, 31, 32, 33, 64, 100, 127, 128])
+def test_reject_panel_edges(kevd, b):
+    X, eps, _ = make_config("ks200k", N=705)
+    ref = arpc(X, eps, 2 * b, b, 5)
+    out = kevd.rpchol_factor(_gpu(X), eps, 2 * b, mode="arpc", b=b, seed=5)
+    if any(_near_edge(ref["log"], rnd) for rnd in range(len(ref["log"]))):
+        pytest.skip("a draw of the oracle lies at an edge")
+    assert out["pivots"].cpu().numpy()[: out["rank"]].tolist() == ref["pivots"].tolist()
+    F = out["F"].cpu().numpy().T[:, : out["rank"]]
+    assert np.max(np.abs(F - ref["F"])) < 1e-10
+    assert np.max(np.abs(out["rho"].cpu().numpy() - ref["rho"])) < 1e-10
