@@ -380,7 +380,11 @@ int kevd_kernel_exp(const double* t, int64_t n, double* out, void* stream);
  * low-memory calls, k only for the eigen calls; opts may be NULL except for
  * the two factors).  KEVD_WS_NORMALIZE sizes for an FP64 factor, whose
  * tensor-core Grams keep the digit planes of one slab of rows (at most 6 GiB),
- * unless opts->precision is KEVD_PREC_BF16X3 (an FP32 factor: no planes).
+ * or, with opts->precision = KEVD_PREC_BF16X3, for an FP32 factor, whose Grams keep
+ * the slices of one slab (at most 12 GiB; given a workspace without room for them the
+ * calls use a slower kernel with the same results).  KEVD_WS_FACTOR with
+ * KEVD_PREC_BF16X3 and b >= 32 includes the split operands of X and F (4 bytes per
+ * entry, up to 48 GiB).
  * Returns 0 for invalid sizes.  The KEVD_WS_EIG and
  * KEVD_WS_LOWMEM_EIG sizes query the eigensolver and therefore need a CUDA
  * device.

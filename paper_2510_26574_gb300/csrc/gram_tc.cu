@@ -44,9 +44,11 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstdint>
 
 #include "common.cuh"
 #include "gram_tc.cuh"
+#include "oz_mma.cuh"
 #include "tc_ptx.cuh"
 
 namespace kevd {
@@ -317,6 +319,303 @@ __global__ void __launch_bounds__(kGtThreads, 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(Cfg::kCols) : "memory");
 }
 
+// ---------------------------------------------------------------------------
+// The same products from pre-cut slices.  With every CTA slicing its own raw tiles, sixteen
+// warps of arithmetic and shared-memory stores set the pace (tensor pipe 34 % active), and
+// each entry of F is sliced once per tile of its block row.  k_gt_cut slices a slab of row
+// splits once into the MMA operands as they stand: per stage of 64 rows and block of 128
+// columns, 16 KB tiles (128 columns x 64 rows, K-major, 128-byte swizzle) of F hi, F mid,
+// wa F hi, wc F hi, wa F mid, wc F mid (one Gram: F hi, F mid, wa F hi, wa F mid).  A stage of
+// k_gram_pl is then two bulk copies (block I's F tiles, block J's weighted ones).  Splits,
+// 1,024-row chunks, MMA order and the FP32 running sums are k_gram_tc's: the same bits.
+// Bound: the tensor pipe (4 x 128 cycles per 16 rows) and L2 (96 KB per 2,048 cycles and SM).
+// N = 2M, rank 1,848, both Grams with the cut and the column maxima: 48.1 ms (k_gram_tc:
+// 79.5 ms).
+// ---------------------------------------------------------------------------
+constexpr size_t kGpBudget = (size_t)12 << 30;      // bytes of slices per slab
+constexpr uint32_t kGpTile = 128 * 128;             // one tile: 128 columns x 64 rows of BF16
+constexpr int kGpChunk = 16;                        // stages per exact chunk: 1,024 rows
+constexpr int kGpThreads = 10 * 32;
+
+template <bool TWO>
+struct GpCfg {
+    static constexpr int NV = TWO ? 256 : 128;
+    static constexpr int kTiles = TWO ? 6 : 4;                     // tiles per stage and column block
+    static constexpr uint32_t kU = 2 * kGpTile, kV = (kTiles - 2) * kGpTile;
+    static constexpr uint32_t kStage = kU + kV;
+    static constexpr int kStages = TWO ? 2 : 3;
+    static constexpr size_t kSmem = (size_t)kStages * kStage + 1024;
+};
+
+// 8 rows of one column, scaled by w, sliced as in slice4: 16 bytes of hi and of mid.
+static __device__ __forceinline__ void cut8(const float (&x)[8], const float (&w)[8], float M, uint8_t* hi, uint8_t* mid) {
+    uint32_t h[4], m[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const float v0 = __fmul_rn(w[2 * e], x[2 * e]), v1 = __fmul_rn(w[2 * e + 1], x[2 * e + 1]);
+        const float h0 = __fsub_rn(__fadd_rn(v0, M), M), h1 = __fsub_rn(__fadd_rn(v1, M), M);
+        h[e] = __byte_perm(__float_as_uint(h0), __float_as_uint(h1), 0x7632);
+        const __nv_bfloat162 mm = __floats2bfloat162_rn(__fsub_rn(v0, h0), __fsub_rn(v1, h1));
+        m[e] = *reinterpret_cast<const uint32_t*>(&mm);
+    }
+    *reinterpret_cast<uint4*>(hi) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(mid) = make_uint4(m[0], m[1], m[2], m[3]);
+}
+
+// Slices of the stages [0, gridDim.y) of the slab starting at row row0.  Block: 8 warps x 4
+// columns; a warp's loads cover 256 consecutive bytes of each column, its stores 512.
+template <bool TWO>
+__global__ void __launch_bounds__(256) k_gt_cut(const float* __restrict__ F, int64_t ldf, int64_t N, int rank, int nb,
+                                                int64_t row0, const float* __restrict__ wa,
+                                                const float* __restrict__ wc, const float* __restrict__ mag,
+                                                uint8_t* __restrict__ P) {
+    const int lane = threadIdx.x & 31, g = lane & 7;
+    const int c = blockIdx.x * 32 + (threadIdx.x >> 5) * 4 + (lane >> 3);
+    const int64_t i = row0 + (int64_t)blockIdx.y * 64 + 8 * g;
+    const bool on = c < rank;
+    const float tiny = 1.5f * 0x1p-100f;
+    float x[8], a[8], q[8], one[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        x[e] = 0.f;
+        one[e] = 1.f;
+        a[e] = i + e < N ? wa[i + e] : 0.f;
+        q[e] = TWO && i + e < N ? wc[i + e] : 0.f;
+    }
+    if (on) {
+        const float* f = F + (int64_t)c * ldf + i;                 // 16-byte aligned (gram_tc_eligible)
+        if (i + 8 <= N) {
+            const float4 u = *reinterpret_cast<const float4*>(f), v = *reinterpret_cast<const float4*>(f + 4);
+            x[0] = u.x; x[1] = u.y; x[2] = u.z; x[3] = u.w;
+            x[4] = v.x; x[5] = v.y; x[6] = v.z; x[7] = v.w;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (i + e < N) x[e] = f[e];
+        }
+    }
+    constexpr int T = GpCfg<TWO>::kTiles;
+    uint8_t* dst = P + ((size_t)blockIdx.y * nb + (c >> 7)) * T * kGpTile + swz(c & 127, g);
+    cut8(x, one, on ? mag[c] : tiny, dst, dst + kGpTile);
+    uint8_t* va = dst + 2 * kGpTile;
+    cut8(x, a, on ? mag[rank + c] : tiny, va, va + (T / 2 - 1) * kGpTile);
+    if (TWO) cut8(x, q, on ? mag[2 * rank + c] : tiny, va + kGpTile, va + 3 * kGpTile);
+}
+
+// Warp 0: copies (one lane); warp 1: MMA issue (one lane); warps 2-9 drain (TMEM lane
+// quarter w % 4, accumulator columns [h NV / 2, + NV / 2), h = (w - 2) / 4).  blockIdx.y: the
+// split within the slab, `split0` its first; `stages`: stages per split in the slab.
+template <bool TWO>
+__global__ void __launch_bounds__(kGpThreads, 1)
+    k_gram_pl(const uint8_t* __restrict__ P, int64_t row0, int64_t N, int nb, int64_t per, int split0,
+              float* __restrict__ gpart, int ntri, int* __restrict__ flags) {
+    using Cfg = GpCfg<TWO>;
+    constexpr int NV = Cfg::NV, S = Cfg::kStages, CW = NV / 2;
+    constexpr uint32_t kIdesc = idesc_bf16(128, NV);
+    constexpr uint32_t kCols = 2 * NV;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t bars[2 * S + 2];   // full[S], empty[S], acc_full, acc_empty
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile int s_fail;
+
+    int I, J;
+    tri_decode(blockIdx.x, nb, I, J);
+    const int64_t i0 = row0 + (int64_t)blockIdx.y * per, i1 = min(i0 + per, N);
+    const int nst = i0 < i1 ? (int)((i1 - i0 + 63) / 64) : 0;
+    const int nch = (nst + kGpChunk - 1) / kGpChunk;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t base = (raw + 1023u) & ~1023u;
+    const uint32_t bar0 = smem_u32(&bars[0]);
+    auto full = [&](int s2) { return bar0 + 8u * s2; };
+    auto empty = [&](int s2) { return bar0 + 8u * (S + s2); };
+    const uint32_t acc_full = bar0 + 8u * (2 * S), acc_empty = bar0 + 8u * (2 * S + 1);
+    if (tid == 0) {
+        for (int s2 = 0; s2 < S; ++s2) {
+            mbar_init(full(s2), 1);
+            mbar_init(empty(s2), 1);
+        }
+        mbar_init(acc_full, 1);
+        mbar_init(acc_empty, 8);
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_async_smem();
+    }
+    if (wid == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)),
+                     "r"(kCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+
+    if (wid == 0) {
+        if (lane == 0) {
+            const size_t row = (size_t)nb * Cfg::kTiles * kGpTile;         // bytes of one stage of all column blocks
+            const uint8_t* st = P + (size_t)((i0 - row0) / 64) * row;
+            const uint8_t* pu = st + (size_t)I * Cfg::kTiles * kGpTile;
+            const uint8_t* pv = st + ((size_t)J * Cfg::kTiles + 2) * kGpTile;
+            bool ok = true;
+            int s2 = 0;
+            uint32_t ph = 1;                                               // the first pass finds the stages empty
+            for (int t = 0; t < nst; ++t, pu += row, pv += row) {
+                ok = mbar_wait_quick(empty(s2), ph, &s_fail);
+                if (!ok) break;
+                mbar_expect_tx(full(s2), Cfg::kStage);
+                bulk_g2s(base + s2 * Cfg::kStage, pu, Cfg::kU, full(s2));
+                bulk_g2s(base + s2 * Cfg::kStage + Cfg::kU, pv, Cfg::kV, full(s2));
+                if (++s2 == S) {
+                    s2 = 0;
+                    ph ^= 1;
+                }
+            }
+            if (!ok) {
+                s_fail = 1;
+                atomicOr(flags, 4);
+            }
+            for (int j = 0; j < S; ++j) mbar_wait(full(j), j < s2 ? ph ^ 1 : ph);   // this CTA's copies have landed
+        }
+    } else if (wid == 1) {
+        if (elect_one()) {
+            const uint32_t d0 = tmem, d1 = tmem + NV;
+            bool ok = true;
+            int s2 = 0, prev = -1, c = 0;
+            uint32_t ph = 0, prev_ph = 0;
+            for (int t = 0; t < nst; ++t) {
+                const bool first = (t % kGpChunk) == 0;
+                ok = mbar_wait_quick(full(s2), ph, &s_fail) &&
+                     (!first || c == 0 || mbar_wait_quick(acc_empty, (uint32_t)(c - 1) & 1, &s_fail));
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t su = base + s2 * Cfg::kStage, sv = su + Cfg::kU;
+                const uint64_t uh = sw128_desc(su), um = sw128_desc(su + kGpTile);
+                const uint64_t vh = sw128_desc(sv), vm = sw128_desc(sv + Cfg::kV / 2);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {                              // 16 rows: 32 bytes further
+                    const uint32_t acc = (first && j == 0) ? 0u : 1u;
+                    umma_bf16(d0, uh + 2 * j, vh + 2 * j, kIdesc, acc);
+                    umma_bf16(d1, uh + 2 * j, vm + 2 * j, kIdesc, acc);
+                    umma_bf16(d1, um + 2 * j, vh + 2 * j, kIdesc, 1u);
+                    umma_bf16(d1, um + 2 * j, vm + 2 * j, kIdesc, 1u);
+                }
+                umma_commit(empty(s2));
+                if ((t % kGpChunk) == kGpChunk - 1 || t == nst - 1) {
+                    umma_commit(acc_full);
+                    ++c;
+                }
+                prev = s2;
+                prev_ph = ph;
+                if (++s2 == S) {
+                    s2 = 0;
+                    ph ^= 1;
+                }
+            }
+            if (!ok) {
+                s_fail = 1;
+                atomicOr(flags, 4);
+            }
+            if (prev >= 0) mbar_wait(empty(prev), prev_ph);                // the last commit covers the earlier MMAs
+        }
+        __syncwarp();
+    } else {
+        const int wq = wid & 3, h = (wid - 2) >> 2;
+        const int m = 32 * wq + lane;
+        const uint32_t at = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)(h * CW);
+        float run[CW];
+#pragma unroll
+        for (int e = 0; e < CW; ++e) run[e] = 0.f;
+        bool ok = true;
+        for (int c = 0; c < nch; ++c) {
+            ok = __all_sync(0xffffffffu, mbar_wait_sleep(acc_full, (uint32_t)c & 1, &s_fail, 256));
+            if (!ok) break;
+            tc_fence_after();
+#pragma unroll
+            for (int cb = 0; cb < CW / 16; ++cb) {
+                uint32_t r0[16], r1[16];
+                tmem_ld16_async(at + 16 * cb, r0);
+                tmem_ld16_async(at + NV + 16 * cb, r1);
+                tmem_wait_ld32(r0, r1);
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    run[16 * cb + e] += __fadd_rn(__uint_as_float(r0[e]), __uint_as_float(r1[e]));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty);
+        }
+        if (!ok) {
+            if (lane == 0) {
+                s_fail = 1;
+                atomicOr(flags, 4);
+            }
+        } else {
+            float* o = gpart + ((size_t)(split0 + blockIdx.y) * ntri + blockIdx.x) * 2 * 128 * 128 +
+                       ((size_t)((h * CW) / 128) * 128 + m) * 128 + (h * CW) % 128;
+#pragma unroll
+            for (int e = 0; e < CW; e += 4)
+                *reinterpret_cast<float4*>(o + e) = make_float4(run[e], run[e + 1], run[e + 2], run[e + 3]);
+        }
+    }
+
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (wid == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kCols) : "memory");
+}
+
+// Row splits per slab for k_gram_pl (0: one split's slices exceed the budget, or F is so large
+// that the card may not hold the slices beside it): the count with the fewest waves of one
+// CTA per SM over all slabs.
+static int gp_slab_splits(int64_t N, int rank, int ngram, int64_t per, int ns, int ntri, int nsm) {
+    const int nb = (rank + 127) / 128;
+    const size_t one = (size_t)((per + 63) / 64) * nb * (ngram == 2 ? 6 : 4) * kGpTile;
+    if ((size_t)N * rank * 4 > ((size_t)128 << 30)) return 0;
+    const int most = (int)std::min<size_t>(ns, kGpBudget / one);
+    int best = 0;
+    int64_t best_waves = INT64_MAX;
+    for (int q = 1; q <= most; ++q) {
+        int64_t waves = 0;
+        for (int s0 = 0; s0 < ns; s0 += q) waves += ((int64_t)ntri * std::min(q, ns - s0) + nsm - 1) / nsm;
+        if (waves < best_waves) {
+            best_waves = waves;
+            best = q;
+        }
+    }
+    return best;
+}
+
+size_t gram_tc_plane_bytes(int64_t N, int rank, int ngram, int nsm) {
+    const int nb = (rank + 127) / 128, ntri = nb * (nb + 1) / 2;
+    int ns = 1;
+    const int64_t per = gram_tc_per(N, ntri, nsm, &ns);
+    return (size_t)gp_slab_splits(N, rank, ngram, per, ns, ntri, nsm) * ((per + 63) / 64) * nb * (ngram == 2 ? 6 : 4) *
+           kGpTile;
+}
+
+template <bool TWO>
+static cudaError_t gram_pl_slabs(const float* F, int64_t ldf, int64_t N, int rank, const float* wa, const float* wc,
+                                 const float* mag, float* gpart, uint8_t* planes, int* flags, int nb, int ntri,
+                                 int64_t per, int ns, int q, cudaStream_t s) {
+    cudaError_t e = cudaFuncSetAttribute(k_gram_pl<TWO>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)GpCfg<TWO>::kSmem);
+    if (e != cudaSuccess) return e;
+    for (int s0 = 0; s0 < ns; s0 += q) {
+        const int cnt = std::min(q, ns - s0);
+        const int64_t row0 = (int64_t)s0 * per, rows = std::min<int64_t>((int64_t)cnt * per, N - row0);
+        k_gt_cut<TWO><<<dim3(4 * nb, (unsigned)((rows + 63) / 64)), 256, 0, s>>>(F, ldf, N, rank, nb, row0, wa, wc, mag,
+                                                                                planes);
+        k_gram_pl<TWO><<<dim3(ntri, cnt), kGpThreads, GpCfg<TWO>::kSmem, s>>>(planes, row0, N, nb, per, s0, gpart, ntri,
+                                                                             flags);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 // Column maxima of |F|, |wa F| and |wc F| (as float bits, atomically maxed into
 // cmax[0..rank), [rank..2 rank), [2 rank..3 rank); cmax zeroed beforehand).
 // Block: 8 warps = 8 columns; blockIdx.y = row split of `per` rows.
@@ -423,8 +722,8 @@ static EncodeTiledFn encode_tiled() {
 }
 
 cudaError_t launch_gram_tc(const float* F, int64_t ldf, int64_t N, int rank, const float* wa, const float* wc,
-                           unsigned* cmax, float* mag, float* gpart, int* flags, int nb, int ntri, int64_t per,
-                           int nsplit, cudaStream_t s) {
+                           unsigned* cmax, float* mag, float* gpart, uint16_t* planes, int* flags, int nb, int ntri,
+                           int64_t per, int nsplit, int nsm, cudaStream_t s) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(cmax, 0, 3 * (size_t)rank * sizeof(unsigned), s)) != cudaSuccess) return e;
     {
@@ -433,6 +732,12 @@ cudaError_t launch_gram_tc(const float* F, int64_t ldf, int64_t N, int rank, con
         k_colmax3<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(F, ldf, N, rank, pr, wa, wc,
                                                                                        cmax);
         k_magic<<<(3 * rank + 255) / 256, 256, 0, s>>>(cmax, 3 * rank, mag);
+    }
+    const int q = planes ? gp_slab_splits(N, rank, wc ? 2 : 1, per, nsplit, ntri, nsm) : 0;
+    if (q > 0) {
+        uint8_t* P = reinterpret_cast<uint8_t*>(planes);
+        return wc ? gram_pl_slabs<true>(F, ldf, N, rank, wa, wc, mag, gpart, P, flags, nb, ntri, per, nsplit, q, s)
+                  : gram_pl_slabs<false>(F, ldf, N, rank, wa, nullptr, mag, gpart, P, flags, nb, ntri, per, nsplit, q, s);
     }
     EncodeTiledFn enc = encode_tiled();
     if (!enc) return cudaErrorNotSupported;

@@ -18,8 +18,11 @@ int64_t gram_tc_per(int64_t N, int64_t ntri, int nsm, int* nsplit);
 // NULL: the first Gram only); cmax, mag: 3 x rank scratch; flags bit 2 is set
 // if a bounded wait gave up.
 cudaError_t launch_gram_tc(const float* F, int64_t ldf, int64_t N, int rank, const float* wa, const float* wc,
-                           unsigned* cmax, float* mag, float* gpart, int* flags, int nb, int ntri, int64_t per,
-                           int nsplit, cudaStream_t s);
+                           unsigned* cmax, float* mag, float* gpart, uint16_t* planes, int* flags, int nb, int ntri,
+                           int64_t per, int nsplit, int nsm, cudaStream_t s);
+// Bytes of `planes` (16-byte aligned; 0: the kernel that slices its own tiles is used, as
+// with planes == NULL).
+size_t gram_tc_plane_bytes(int64_t N, int rank, int ngram, int nsm);
 
 // FP64 factor: weighted Grams on the tensor cores at FP64 accuracy (gram_oz.cu),
 // A = (sa F)^T (sa F) and C = (sc F)^T (sc F).  sa, sc: N row scales (sc NULL: A

@@ -35,7 +35,8 @@ struct NormWs {
     float* mag;     // 3 x rank: their grid magic numbers
     uint32_t* cmax64;   // 2 x rank: keys of the column maxima of the scaled FP64 F
     int* ecol;      // 2 x rank: their exponents
-    uint16_t* planes;   // FP64 Gram: digit planes of one slab of rows
+    uint16_t* planes;   // Gram: digit planes (FP64 F) or slices (FP32 F) of one slab of rows
+    size_t plane_off;   // bytes of everything before the planes (the last array)
     double* gpart;  // nsplit x ntri x 2 x 64 x 64 Gram partials (128 x 128 for FP32 F)
 };
 
@@ -97,8 +98,10 @@ static NormWs carve_norm(void* base, int64_t N, int rank, size_t* bytes, bool fp
     w.cmax64 = c.take<uint32_t>(2 * (size_t)rank);
     w.ecol = c.take<int>(2 * (size_t)rank);
     w.gpart = c.take<double>(std::max(std::max(gp64, gp32), gpoz));
-    w.planes = fp64 ? c.take<uint16_t>(std::max(gram_oz_plane_bytes(N, rank, 2), gram_oz_plane_bytes(N, rank, 1)) / 2)
-                    : nullptr;
+    const size_t pl = fp64 ? std::max(gram_oz_plane_bytes(N, rank, 2), gram_oz_plane_bytes(N, rank, 1))
+                           : std::max(gram_tc_plane_bytes(N, rank, 2, kSMs), gram_tc_plane_bytes(N, rank, 1, kSMs));
+    w.plane_off = c.off;
+    w.planes = pl ? c.take<uint16_t>(pl / 2) : nullptr;
     *bytes = c.off;
     return w;
 }
@@ -612,7 +615,8 @@ static cudaError_t gram32(const float* F, int64_t ldf, int64_t N, int rank, cons
         {
             TraceScope tr(kStGram, s);
             float* gp32 = reinterpret_cast<float*>(gpart);
-            cudaError_t e = launch_gram_tc(F, ldf, N, rank, wa, wc, w.cmax, w.mag, gp32, w.flags, nb, ntri, per, ns, s);
+            cudaError_t e = launch_gram_tc(F, ldf, N, rank, wa, wc, w.cmax, w.mag, gp32, w.planes, w.flags, nb,
+                                          ntri, per, ns, kSMs, s);
             if (e != cudaSuccess) return e;
         }
         {
@@ -751,6 +755,10 @@ extern "C" int bistoch_normalize(const void* F, int f_dtype, int64_t N, int32_t 
     if (N < 1 || rank < 1 || rank > N || ldf < N || (f_dtype != KEVD_F64 && f_dtype != KEVD_F32)) return KEVD_EINVAL;
     size_t need = 0;
     NormWs w = carve_norm(workspace, N, rank, &need, f_dtype == KEVD_F64);
+    if (f_dtype == KEVD_F32 && ws_bytes < need) {   // no room for the slices: the Gram kernel that needs none
+        need = w.plane_off;
+        w.planes = nullptr;
+    }
     if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return KEVD_EWORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (f_dtype == KEVD_F32)
@@ -834,6 +842,10 @@ extern "C" int symmetric_normalize(const void* F, int f_dtype, int64_t N, int32_
     if (N < 1 || rank < 1 || rank > N || ldf < N || (f_dtype != KEVD_F64 && f_dtype != KEVD_F32)) return KEVD_EINVAL;
     size_t need = 0;
     NormWs w = carve_norm(workspace, N, rank, &need, f_dtype == KEVD_F64);
+    if (f_dtype == KEVD_F32 && ws_bytes < need) {   // no room for the slices: the Gram kernel that needs none
+        need = w.plane_off;
+        w.planes = nullptr;
+    }
     if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return KEVD_EWORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     if (f_dtype == KEVD_F32)

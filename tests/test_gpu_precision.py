@@ -394,3 +394,34 @@ def test_subspace_topk_vsa2m_without_fallback(kevd):
     print("rank %d, lambda_k %.3e, eig rel %.2e, max cluster angle %.2e" % (rk, ev_s[-1], erel, ang))
     assert erel < 1e-6, erel
     assert ang < 1e-3, ang
+
+
+# The Grams of an FP32 factor from pre-cut slices against the kernel that slices its own
+# tiles, which a workspace without room for the slices selects: the same bits, in both Grams
+# and in the symmetric form.  N ends inside a 64-row stage, at a 1,024-row chunk and past
+# one; 20,480 and 70,004 rows have several splits; rank 129 leaves a 128-column block ragged.
+@pytest.mark.parametrize("N,rank", [(64, 5), (1024, 128), (1028, 129), (4100, 200), (20480, 130), (70004, 129)])
+def test_fp32_grams_from_slices_same_bits(kevd, N, rank):
+    import ctypes
+    from paper_2510_26574_gb300 import kevd as K
+    g = torch.Generator().manual_seed(N + rank)
+    F = (torch.rand(rank, N, generator=g) * torch.logspace(0, -3, rank)[:, None]).float().cuda()
+    ref = kevd.bistoch_normalize(F, rank)
+    sym = kevd.symmetric_normalize(F, rank)
+    o = K.make_opts(precision="bf16x3")
+    full = K.workspace_bytes(K.KEVD_WS_NORMALIZE, N, 1, rank, 1, o)
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    out = [torch.empty_like(t) for t in ref]
+    small = None
+    for nb in range(full - 256, 0, -max(256, full // 64 // 256 * 256)):      # the largest size below full that still runs
+        st = K.lib().bistoch_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, *[K._ptr(t) for t in out], K._ptr(ws), nb,
+                                       K._stream(F.device))
+        if st == K.KEVD_OK:
+            small = nb
+            break
+    assert small is not None
+    assert all(torch.equal(a, b) for a, b in zip(ref, out))
+    d, A = torch.empty_like(sym[0]), torch.empty_like(sym[1])
+    assert K.lib().symmetric_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, K._ptr(d), K._ptr(A), K._ptr(ws), small,
+                                       K._stream(F.device)) == K.KEVD_OK
+    assert torch.equal(sym[0], d) and torch.equal(sym[1], A)
