@@ -426,9 +426,9 @@ __global__ void k_colexp_f64(const uint32_t* __restrict__ cmax, int n, int* __re
 
 // Sum of the split partials in a fixed order; entry (a, c) of tile (I, J) is
 // Gram entry (128 I + a, 64 J + c), written with its mirror when it lies in the
-// upper triangle (each unordered pair has exactly one such owner).
+// upper triangle (each unordered pair has exactly one such owner); acc adds to A and C.
 __global__ void k_gram_oz_final(const double* __restrict__ gpart, int nsplit, int ntiles, int nbi, int nbj, int rank,
-                                int ngram, const int* __restrict__ Ecol, double* __restrict__ A,
+                                int ngram, const int* __restrict__ Ecol, int acc, double* __restrict__ A,
                                 double* __restrict__ C) {
     int I, J;
     oz_tile_decode(blockIdx.x, nbi, nbj, I, J);
@@ -444,6 +444,7 @@ __global__ void k_gram_oz_final(const double* __restrict__ gpart, int nsplit, in
             sum += gpart[(((size_t)gram * nsplit + q) * ntiles + blockIdx.x) * (kOzM * kOzN) + e];
         if (Ecol[gram * rank + ra] == kOzNonFinite || Ecol[gram * rank + rc] == kOzNonFinite)
             sum = __longlong_as_double(0x7FF8000000000000ll);
+        if (acc) sum += G[(int64_t)rc * rank + ra];                // (each unordered pair has one thread)
         G[(int64_t)rc * rank + ra] = sum;
         G[(int64_t)ra * rank + rc] = sum;
     }
@@ -478,12 +479,12 @@ static int64_t oz_slab_rows(int64_t N, int rank, int ngram, int D) {
 // Row splits per slab (the same in every slab): ntiles x ngram x nsplit CTAs
 // filling whole waves of one CTA per SM, at least 4,096 rows per split and at most
 // kOzNarrowK.
-static int oz_nsplit(int64_t S, int64_t nctas, int nsm) {
+static int oz_nsplit(int64_t S, int64_t nctas, int nsm, int64_t least = 4096) {
     const int lo = (int)((S + kOzNarrowK - 1) / kOzNarrowK);
     int best = lo;
     double best_eff = -1.0;
     for (int sp = lo; sp <= lo + 8; ++sp) {
-        if (sp > lo && S / sp < 4096) break;
+        if (sp > lo && S / sp < least) break;
         const int64_t blocks = nctas * sp;
         const double eff = (double)blocks / (double)(((blocks + nsm - 1) / nsm) * nsm);
         if (eff > best_eff + 0.01) {
@@ -527,13 +528,12 @@ static bool oz_plane_map(EncodeTiledFnOz enc, CUtensorMap* map, uint16_t* base, 
 }
 
 template <int D>
-static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t ldf, int64_t N, int rank,
-                                 const double* sa, const double* sc, const int* Ecol, double* gpart, uint16_t* planes,
-                                 int* flags, double* A, double* C, int nsm, cudaStream_t s) {
+static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, int64_t S, int ns, int acc, const double* F, int64_t ldf,
+                                 int64_t N, int rank, const double* sa, const double* sc, const int* Ecol, double* gpart,
+                                 uint16_t* planes, int* flags, double* A, double* C, cudaStream_t s) {
     cudaError_t e;
     const int ngram = sc ? 2 : 1;
     const int rank_pad = oz_rank_pad(rank);
-    const int64_t S = oz_slab_rows(N, rank, ngram, D);
     const size_t set = (size_t)D * rank_pad * S;                  // BF16 elements per set
     CUtensorMap mua, mva, muc, mvc;
     uint16_t* pc = planes + (ngram == 2 ? set : 0);
@@ -542,7 +542,6 @@ static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t l
         return cudaErrorInvalidValue;
     const int nbi = (rank + kOzM - 1) / kOzM, nbj = (rank + kOzN - 1) / kOzN;
     const int nt = oz_ntiles(rank);
-    const int ns = oz_nsplit(S, (int64_t)nt * ngram, nsm);
     if ((e = cudaFuncSetAttribute(k_gram_oz<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)OzGramCfg<D>::kSmem)) != cudaSuccess)
         return e;
@@ -556,24 +555,23 @@ static cudaError_t gram_oz_slabs(EncodeTiledFnOz enc, const double* F, int64_t l
             mua, mva, muc, mvc, Ecol, rank, rows, nbi, nbj, per, gpart, nt, row0 > 0 ? 1 : 0, flags);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
-    k_gram_oz_final<<<dim3((unsigned)nt, (unsigned)ngram), 256, 0, s>>>(gpart, ns, nt, nbi, nbj, rank, ngram, Ecol, A,
-                                                                        C);
+    k_gram_oz_final<<<dim3((unsigned)nt, (unsigned)ngram), 256, 0, s>>>(gpart, ns, nt, nbi, nbj, rank, ngram, Ecol, acc,
+                                                                        A, C);
     return cudaGetLastError();
 }
 
-cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* sa, const double* sc,
-                           uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, double* gpart,
-                           uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s) {
+// Column exponents of the scaled F, then the tensor-map encoder.
+static cudaError_t gram_oz_begin(const double* F, int64_t ldf, int64_t N, int rank, const double* sa, const double* sc,
+                                 uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, EncodeTiledFnOz* out,
+                                 cudaStream_t s) {
     cudaError_t e;
     if ((e = cudaMemsetAsync(cmax, 0, 2 * (size_t)rank * sizeof(uint32_t), s)) != cudaSuccess) return e;
-    {
-        const int ncs = (int)std::max<int64_t>(1, std::min<int64_t>(64, N / 8192));
-        const int64_t pr = ((N + ncs - 1) / ncs + 255) / 256 * 256;
-        k_weights_hi<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(sa, sc, N, sa_hi, sc ? sc_hi : nullptr);
-        k_colmax_f64<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(
-            F, ldf, N, rank, pr, sa_hi, sc ? sc_hi : nullptr, cmax);
-        k_colexp_f64<<<(2 * rank + 255) / 256, 256, 0, s>>>(cmax, 2 * rank, Ecol);
-    }
+    const int ncs = (int)std::max<int64_t>(1, std::min<int64_t>(64, N / 8192));
+    const int64_t pr = ((N + ncs - 1) / ncs + 255) / 256 * 256;
+    k_weights_hi<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(sa, sc, N, sa_hi, sc ? sc_hi : nullptr);
+    k_colmax_f64<<<dim3((rank + 7) / 8, (unsigned)((N + pr - 1) / pr)), 256, 0, s>>>(F, ldf, N, rank, pr, sa_hi,
+                                                                                    sc ? sc_hi : nullptr, cmax);
+    k_colexp_f64<<<(2 * rank + 255) / 256, 256, 0, s>>>(cmax, 2 * rank, Ecol);
     static EncodeTiledFnOz enc = nullptr;
     if (!enc) {
         void* p = nullptr;
@@ -584,9 +582,51 @@ cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, co
             return cudaErrorNotSupported;
         enc = reinterpret_cast<EncodeTiledFnOz>(p);
     }
-    return oz_gram_digits(F, ldf) == 6
-               ? gram_oz_slabs<6>(enc, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, nsm, s)
-               : gram_oz_slabs<7>(enc, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, nsm, s);
+    *out = enc;
+    return cudaSuccess;
+}
+
+cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, const double* sa, const double* sc,
+                           uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, double* gpart,
+                           uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s) {
+    EncodeTiledFnOz enc;
+    const cudaError_t e = gram_oz_begin(F, ldf, N, rank, sa, sc, sa_hi, sc_hi, cmax, Ecol, &enc, s);
+    if (e != cudaSuccess) return e;
+    const int D = oz_gram_digits(F, ldf), ngram = sc ? 2 : 1;
+    const int64_t S = oz_slab_rows(N, rank, ngram, D);
+    const int ns = oz_nsplit(S, (int64_t)oz_ntiles(rank) * ngram, nsm);
+    return D == 6 ? gram_oz_slabs<6>(enc, S, ns, 0, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, s)
+                  : gram_oz_slabs<7>(enc, S, ns, 0, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, s);
+}
+
+// Panels of the low-memory form: the planes stay within 256 MiB (its panel takes 128), and a
+// split may be as short as 1,024 rows, since one panel has few tiles.  Seven digits, as the
+// FP64-pipe Grams that it replaces have the error of.  Measured on N = 60,000, rank 512
+// (factor and normalisation without stored F): 61.2 ms, 80.4 with the FP64-pipe Grams.
+constexpr size_t kOzPanelBudget = (size_t)256 << 20;
+static int64_t oz_panel_rows(int64_t P, int rank) {
+    const int64_t most = (int64_t)(kOzPanelBudget / ((size_t)2 * kDigits * oz_rank_pad(rank) * 2)) / 256 * 256;
+    const int64_t nslab = (P + std::max<int64_t>(most, 256) - 1) / std::max<int64_t>(most, 256);
+    return ((P + nslab - 1) / nslab + 255) / 256 * 256;
+}
+static int oz_panel_splits(int64_t P, int rank, int nsm) {
+    return oz_nsplit(oz_panel_rows(P, rank), (int64_t)oz_ntiles(rank) * 2, nsm, 1024);
+}
+size_t gram_oz_panel_partial_doubles(int64_t P, int rank, int nsm) {
+    return (size_t)2 * oz_panel_splits(P, rank, nsm) * oz_ntiles(rank) * kOzM * kOzN;
+}
+size_t gram_oz_panel_plane_bytes(int64_t P, int rank) {
+    return (size_t)2 * kDigits * oz_rank_pad(rank) * oz_panel_rows(P, rank) * 2;
+}
+cudaError_t launch_gram_oz_panel(const double* F, int64_t ldf, int64_t P, int64_t N, int rank, const double* sa,
+                                 const double* sc, uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol,
+                                 double* gpart, uint16_t* planes, int* flags, double* A, double* C, int acc, int nsm,
+                                 cudaStream_t s) {
+    EncodeTiledFnOz enc;
+    const cudaError_t e = gram_oz_begin(F, ldf, N, rank, sa, sc, sa_hi, sc_hi, cmax, Ecol, &enc, s);
+    if (e != cudaSuccess) return e;
+    return gram_oz_slabs<kDigits>(enc, oz_panel_rows(P, rank), oz_panel_splits(P, rank, nsm), acc, F, ldf, N, rank, sa,
+                                  sc, Ecol, gpart, planes, flags, A, C, s);
 }
 
 }  // namespace kevd

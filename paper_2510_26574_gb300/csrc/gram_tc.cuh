@@ -37,4 +37,13 @@ cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, co
                            uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol, double* gpart,
                            uint16_t* planes, int* flags, double* A, double* C, int nsm, cudaStream_t s);
 
+// The same for one panel of N <= P rows with seven digits (the error of the FP64-pipe
+// kernel), acc adding to A and C; gpart and planes as sized for P rows.
+size_t gram_oz_panel_partial_doubles(int64_t P, int rank, int nsm);
+size_t gram_oz_panel_plane_bytes(int64_t P, int rank);
+cudaError_t launch_gram_oz_panel(const double* F, int64_t ldf, int64_t P, int64_t N, int rank, const double* sa,
+                                 const double* sc, uint32_t* sa_hi, uint32_t* sc_hi, uint32_t* cmax, int* Ecol,
+                                 double* gpart, uint16_t* planes, int* flags, double* A, double* C, int acc, int nsm,
+                                 cudaStream_t s);
+
 }  // namespace kevd

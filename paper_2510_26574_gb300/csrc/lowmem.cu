@@ -23,7 +23,8 @@
 //   1  s_K = K(S,:) 1                       y = W^-T W^-1 s_K  (so F s = K(:,S) y)
 //   2  d~ = K(:,S) y,  t_K = K(S,:) d~^-1   z = W^-T W^-1 t_K
 //   3  q~ = K(:,S) z;  F_p = K(p,S) W^-T;  A += F_p^T D~^-2 F_p,
-//      C += F_p^T Q~^-1 F_p (the normalisation's Gram kernel, accumulated).
+//      C += F_p^T Q~^-1 F_p (the normalisation's Gram kernels, accumulated: tensor cores,
+//      or the FP64 pipe in a workspace without room for the digit planes).
 // The vectors come from K(:,S) times a solved vector, which agrees with the
 // rebuilt-F definition to ~1e-14 even at cond(W) ~ 3e5.  The Grams use the
 // rebuilt F_p: W^-1 (K^T D K) W^-T loses accuracy with cond(W)^2 (2e-10 at
@@ -42,6 +43,7 @@
 
 #include "common.cuh"
 #include "factor.cuh"
+#include "gram_tc.cuh"
 #include "lowmem.cuh"
 #include "trace.cuh"
 
@@ -287,15 +289,18 @@ __global__ void k_lm_recip(const double* __restrict__ d, int64_t n, double* __re
     out[i] = 1.0 / d[i];
 }
 
-// Gram weights 1/d~^2 and 1/q~ of a panel's rows; flags bit 1 where q~ <= 0.
-__global__ void k_lm_weights(const double* __restrict__ d, const double* __restrict__ q, int64_t n,
+// Gram weights of a panel's rows, 1/d~^2 and 1/q~ (with root the row scales 1/d~ and
+// 1/sqrt(q~) that the tensor-core Grams take); flags bit 1 where q~ <= 0.
+__global__ void k_lm_weights(const double* __restrict__ d, const double* __restrict__ q, int64_t n, int root,
                              double* __restrict__ wa, double* __restrict__ wc, int* __restrict__ flags) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (!(q[i] > 0.0)) atomicOr(flags, 2);
-    wa[i] = 1.0 / (d[i] * d[i]);
-    wc[i] = 1.0 / q[i];
+    wa[i] = 1.0 / (root ? d[i] : d[i] * d[i]);
+    wc[i] = 1.0 / (root ? sqrt(q[i]) : q[i]);
 }
+
+constexpr int kLmSMs = 152;   // wave sizing of the Gram grids (a performance choice only)
 
 static int grid1(int64_t n) { return (int)((n + 255) / 256); }
 
@@ -327,15 +332,21 @@ struct LmNormWs {
     double* vec;    // rank: K(S,:) 1, then K(S,:) d~^-1
     double* y;      // rank: the solved vectors
     double* pv;     // P: 1/d~ of the panel's rows
-    double* wa;     // P: 1/d~^2
-    double* wc;     // P: 1/q~
+    double* wa;     // P: 1/d~^2 (tensor-core Grams: 1/d~)
+    double* wc;     // P: 1/q~ (tensor-core Grams: 1/sqrt(q~))
     double* gpart;  // Gram split partials of one panel
-    int* flags;     // bit 0: d~ <= 0, bit 1: q~ <= 0, bit 2: pivot out of range
+    int* flags;     // [0] bit 0: d~ <= 0, bit 1: q~ <= 0, bit 2: pivot out of range; [1]: the Grams' flags
+    // tensor-core Grams of one panel
+    uint32_t *sa_hi, *sc_hi, *cmax;
+    int* ecol;
+    uint16_t* planes;
 };
 
-static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, size_t* bytes) {
+// tc: with the buffers of the tensor-core Grams (without them a smaller workspace still
+// serves, by the FP64-pipe Grams).
+static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, bool tc, size_t* bytes) {
     Carver c(base);
-    LmNormWs L;
+    LmNormWs L{};
     L.p = carve_panel(c, N, d, rank);
     const int64_t P = L.p.P;
     L.ones = c.take<double>(P);
@@ -344,8 +355,16 @@ static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, size_t* by
     L.pv = c.take<double>(P);
     L.wa = c.take<double>(P);
     L.wc = c.take<double>(P);
-    L.gpart = c.take<double>(kevd_gram_partial_doubles(P, rank));
+    L.gpart = c.take<double>(std::max(kevd_gram_partial_doubles(P, rank),
+                                      tc ? gram_oz_panel_partial_doubles(P, rank, kLmSMs) : (size_t)0));
     L.flags = c.take<int>(4);
+    if (tc) {
+        L.sa_hi = c.take<uint32_t>(P);
+        L.sc_hi = c.take<uint32_t>(P);
+        L.cmax = c.take<uint32_t>(2 * (size_t)rank);
+        L.ecol = c.take<int>(2 * (size_t)rank);
+        L.planes = c.take<uint16_t>(gram_oz_panel_plane_bytes(P, rank) / 2);
+    }
     *bytes = c.off;
     return L;
 }
@@ -380,7 +399,7 @@ size_t kevd_lowmem_factor_ws(int64_t N, int32_t d, int32_t r, const kevd_opts* o
 size_t kevd_lowmem_normalize_ws(int64_t N, int32_t d, int32_t rank) {
     if (N < 1 || d < 1 || rank < 1 || rank > N) return 0;
     size_t bytes = 0;
-    carve_lm_norm(nullptr, N, d, rank, &bytes);
+    carve_lm_norm(nullptr, N, d, rank, true, &bytes);
     return bytes;
 }
 
@@ -503,7 +522,9 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
     if (N < 1 || N > INT_MAX || d < 1 || rank < 1 || rank > N || ldw < rank || ldw > INT_MAX) return KEVD_EINVAL;
     if (!(eps > 0.0) || !isfinite(eps)) return KEVD_EINVAL;
     size_t need = 0;
-    LmNormWs L = carve_lm_norm(workspace, N, d, rank, &need);
+    LmNormWs L = carve_lm_norm(workspace, N, d, rank, true, &need);
+    const bool tc = gram_oz_eligible(N, rank) && ws_bytes >= need;
+    if (!tc) L = carve_lm_norm(workspace, N, d, rank, false, &need);
     if (!workspace || ws_bytes < need || !aligned(workspace)) return KEVD_EWORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cublasHandle_t h = lm_blas(s);
@@ -553,20 +574,25 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
                 (st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s)) != KEVD_OK)
                 return st;
             LM_BLAS(cublasDgemv(h, CUBLAS_OP_N, (int)Pc, rank, &one, p.Kp, (int)p.P, L.y, 1, &zero, qtil + i0, 1));
-            k_lm_weights<<<grid1(Pc), 256, 0, s>>>(dtil + i0, qtil + i0, Pc, L.wa, L.wc, L.flags);
+            k_lm_weights<<<grid1(Pc), 256, 0, s>>>(dtil + i0, qtil + i0, Pc, tc, L.wa, L.wc, L.flags);
             KEVD_LAUNCH_CHECK();
             LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT, (int)Pc,
                                 rank, &one, W, (int)ldw, p.Kp, (int)p.P));
-            KEVD_CUDA_TRY(kevd_gram_weighted(p.Kp, p.P, Pc, rank, L.wa, L.wc, L.gpart, A, C, i0 > 0, s));
+            if (tc)
+                KEVD_CUDA_TRY(launch_gram_oz_panel(p.Kp, p.P, p.P, Pc, rank, L.wa, L.wc, L.sa_hi, L.sc_hi, L.cmax,
+                                                   L.ecol, L.gpart, L.planes, L.flags + 1, A, C, i0 > 0, kLmSMs, s));
+            else
+                KEVD_CUDA_TRY(kevd_gram_weighted(p.Kp, p.P, Pc, rank, L.wa, L.wc, L.gpart, A, C, i0 > 0, s));
         }
     }
-    int flags = 0;
-    KEVD_CUDA_TRY(cudaMemcpyAsync(&flags, L.flags, sizeof(int), cudaMemcpyDeviceToHost, s));
+    int flags[2] = {0, 0};
+    KEVD_CUDA_TRY(cudaMemcpyAsync(flags, L.flags, sizeof(flags), cudaMemcpyDeviceToHost, s));
     KEVD_CUDA_TRY(cudaStreamSynchronize(s));
     trace_flush();
-    if (flags & 4) return KEVD_EINVAL;
-    if (flags & 1) return KEVD_ED_NONPOS;
-    if (flags & 2) return KEVD_EQ_NONPOS;
+    if (flags[0] & 4) return KEVD_EINVAL;
+    if (flags[0] & 1) return KEVD_ED_NONPOS;
+    if (flags[0] & 2) return KEVD_EQ_NONPOS;
+    if (flags[1]) return KEVD_ETIMEOUT;
     return KEVD_OK;
 }
 

@@ -149,6 +149,29 @@ def test_normalize_and_eig_match_oracle(kevd, monkeypatch, panel):
     assert np.max(np.abs(U.T @ U - np.eye(k))) < 1e-10
 
 
+# The panels' Grams on the tensor cores (seven digit planes) against the FP64-pipe Grams of
+# the same panels: rank 65 / 129 leave one column in the last 64- and 128-column tile, N = 257
+# and 3,001 end in short panels, "64" makes a panel shorter than one 256-row chunk and 65 / 129
+# rows of W per panel.  Bar: the same F and weights on both sides, so only the sums differ, by
+# at most one rounding (2^-53) per term and side, over terms whose sum is at most the largest entry.
+@pytest.mark.parametrize("N,r,panel", [(40, 16, None), (257, 65, "64"), (3001, 129, "192"), (9001, 130, None)])
+def test_panel_grams_tensor_core_and_fp64_pipe(kevd, monkeypatch, N, r, panel):
+    if panel:
+        monkeypatch.setenv("KEVD_LOWMEM_PANEL", panel)
+    X, eps, _ = make_config("ks200k", N=N)
+    Xg = _gpu(X)
+    out = kevd.rpchol_factor_lowmem(Xg, eps, r, b=8, seed=5)
+    rk = out["rank"]
+    got = kevd.bistoch_normalize_lowmem(Xg, eps, out["pivots"], out["W"], rk)
+    monkeypatch.setenv("KEVD_GRAM", "fp64")
+    ref = kevd.bistoch_normalize_lowmem(Xg, eps, out["pivots"], out["W"], rk)
+    for i in range(2):
+        assert torch.equal(got[i], ref[i])
+    for i in range(2, 4):
+        assert torch.equal(got[i], got[i].T)
+        assert torch.max(torch.abs(got[i] - ref[i])) <= (N + 32) * 2.0 ** -52 * torch.max(torch.abs(ref[i]))
+
+
 def test_out_of_range_pivot_is_an_error(kevd):
     X, eps, _ = make_config("ks200k", N=1000)
     Xg = _gpu(X)
