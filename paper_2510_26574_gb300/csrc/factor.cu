@@ -29,6 +29,8 @@
 
 namespace kevd {
 
+constexpr int kPropChunks = 1024;   // chunks of the tile sums in a proposal step
+
 static int tc_bn(int b) { return b <= 32 ? 32 : b <= 64 ? 64 : 128; }
 
 // oz: the FP64 path with the engine on the tensor cores (ozmm.cu): the two
@@ -45,8 +47,7 @@ static FactorWs carve_factor(void* base, int64_t N, int d, int r, int b, size_t*
     w.tile_sum = c.take<double>(nt);
     w.tile_max = c.take<double>(nt);
     w.tile_idx = c.take<int64_t>(nt);
-    w.pre_incl = c.take<double>(nt);
-    w.pre_excl = c.take<double>(nt);
+    w.pre = c.take<double>(kPropChunks + 32);
     w.prop = c.take<int64_t>(b);
     w.acc_pos = c.take<int32_t>(b);
     w.tpos = c.take<int32_t>(b);
@@ -138,122 +139,165 @@ __device__ __forceinline__ double warp_incl_scan(double v) {
     return v;
 }
 
+// All threads of the cluster; what they wrote to global memory before is visible after.
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
-// a2: pivot proposal.  One block of 1024 threads.
+// a2: pivot proposal.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void propose_body(FactorWs w, const double* __restrict__ rho, int64_t N, int64_t ntiles,
-                                             int b, int r, int greedy, uint64_t seed, int rnd,
-                                             int64_t* __restrict__ proposals_out, double floor_sum = 0.0) {
-    __shared__ double sh[33];
+
+// Commits the previous round (one thread).
+__device__ __forceinline__ void commit_round(FactorState* st) {
+    if (st->m > 0) {
+        st->sum_k += st->k;
+        st->eng_rounds += 1;
+    }
+    st->k += st->m;
+    st->kp += (st->m + 15) & ~15;
+    st->sum_m_sq += (long long)st->m * st->m;
+    st->m = 0;
+}
+
+// Greedy: the argmax of rho from the tile (max, index) pairs.  One block of 1024 threads.
+__global__ void __launch_bounds__(1024) k_propose_greedy(FactorWs w, int64_t ntiles, int r, int rnd,
+                                                         int64_t* __restrict__ proposals_out) {
+    __shared__ double sh[32];
     __shared__ int64_t shi[32];
     __shared__ int s_go;
     FactorState* st = w.st;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     if (tid == 0) {
-        if (st->m > 0) {
-            st->sum_k += st->k;
-            st->eng_rounds += 1;
-        }
-        st->k += st->m;
-        st->kp += (st->m + 15) & ~15;
-        st->sum_m_sq += (long long)st->m * st->m;
-        st->m = 0;
+        commit_round(st);
         if (st->k >= r) st->done = 1;
         s_go = !st->done;
     }
     __syncthreads();
     if (!s_go) return;
-
-    if (greedy) {
-        double v = -1.0;
-        int64_t idx = LLONG_MAX;
-        for (int64_t t = tid; t < ntiles; t += blockDim.x) argmax_merge(v, idx, w.tile_max[t], w.tile_idx[t]);
-        warp_argmax(v, idx);
-        if (lane == 0) {
-            sh[wid] = v;
-            shi[wid] = idx;
-        }
-        __syncthreads();
-        if (wid == 0) {
-            v = lane < nw ? sh[lane] : -1.0;
-            idx = lane < nw ? shi[lane] : LLONG_MAX;
-            warp_argmax(v, idx);
-            if (lane == 0) {
-                if (!(v > 0.0)) {
-                    st->done = 1;
-                } else {
-                    w.prop[0] = idx;
-                    st->total = v;
-                    st->rounds += 1;
-                    if (proposals_out) proposals_out[rnd] = idx;
-                }
-            }
-        }
-        return;
+    double v = -1.0;
+    int64_t idx = LLONG_MAX;
+    for (int64_t t = tid; t < ntiles; t += blockDim.x) argmax_merge(v, idx, w.tile_max[t], w.tile_idx[t]);
+    warp_argmax(v, idx);
+    if (lane == 0) {
+        sh[wid] = v;
+        shi[wid] = idx;
     }
-
-    // Exclusive/inclusive prefix of the tile sums; each thread owns a
-    // contiguous chunk, chunks are combined by a block scan.
-    const int64_t chunk = (ntiles + blockDim.x - 1) / blockDim.x;
-    const int64_t t0 = min((int64_t)tid * chunk, ntiles), t1 = min(t0 + chunk, ntiles);
-    double loc = 0.0;
-    for (int64_t t = t0; t < t1; ++t) loc += w.tile_sum[t];
-    double inc = warp_incl_scan(loc);
-    if (lane == 31) sh[wid] = inc;
     __syncthreads();
     if (wid == 0) {
-        double wv = lane < nw ? sh[lane] : 0.0;
-        double wi = warp_incl_scan(wv);
-        sh[lane] = wi - wv;            // exclusive warp offsets
-        if (lane == 31) sh[32] = wi;   // block total
+        v = lane < nw ? sh[lane] : -1.0;
+        idx = lane < nw ? shi[lane] : LLONG_MAX;
+        warp_argmax(v, idx);
+        if (lane == 0) {
+            if (!(v > 0.0)) {
+                st->done = 1;
+            } else {
+                w.prop[0] = idx;
+                st->total = v;
+                st->rounds += 1;
+                if (proposals_out) proposals_out[rnd] = idx;
+            }
+        }
     }
-    __syncthreads();
-    double run = sh[wid] + inc - loc;
-    const double S = sh[32];
-    for (int64_t t = t0; t < t1; ++t) {
-        w.pre_excl[t] = run;
-        run += w.tile_sum[t];
-        w.pre_incl[t] = run;
+}
+
+// ARPC: b inverse-CDF draws from rho.  The tile sums are cut into 1,024 chunks, one thread
+// each, whose offsets are found by a scan; a draw then looks for its chunk among the
+// offsets (two loads per lane), its tile in the chunk and its row in the tile, 32 at a time.
+// An FP64 operation takes a quarter of an SM's pipe for 17 cycles, so the chunks and the
+// draws are spread over a cluster of 8 CTAs, with a warp per draw at b = 128: per round
+// 16 / 11 us at N = 2,000,000 / 524,288 (one CTA, prefixes of all tiles written and
+// searched: 96 / 59 us).
+constexpr int kPropCluster = 8;
+constexpr int kPropThreads = 512;
+
+__device__ __forceinline__ void propose_body(FactorWs w, const double* __restrict__ rho, int64_t N, int64_t ntiles,
+                                             int b, int r, uint64_t seed, int rnd, int64_t* __restrict__ proposals_out,
+                                             double floor_sum, int cta) {
+    constexpr unsigned kAll = 0xffffffffu;
+    FactorState* st = w.st;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const bool go = !st->done && st->k + st->m < r;           // the same in every CTA
+    const int64_t chunk = (ntiles + kPropChunks - 1) / kPropChunks;
+    constexpr int kPer = kPropChunks / kPropCluster;
+    double loc = 0.0, inc = 0.0;
+    if (go && tid < kPer) {
+        const int64_t t0 = min((int64_t)(cta * kPer + tid) * chunk, ntiles), t1 = min(t0 + chunk, ntiles);
+#pragma unroll 8
+        for (int64_t t = t0; t < t1; ++t) loc += w.tile_sum[t];
+        inc = warp_incl_scan(loc);
+        if (lane == 31) w.pre[kPropChunks + cta * (kPer / 32) + wid] = inc;
     }
-    __syncthreads();
+    cluster_sync();                                           // every CTA has read the state
+    if (cta == 0 && tid == 0) {
+        commit_round(st);
+        if (!go) st->done = 1;
+    }
+    if (!go) return;
+    const double wv = __ldcg(w.pre + kPropChunks + lane);
+    const double wi = warp_incl_scan(wv);
+    const double S = __shfl_sync(kAll, wi, 31);
+    if (tid < kPer) w.pre[cta * kPer + tid] = __shfl_sync(kAll, wi - wv, cta * (kPer / 32) + wid) + inc - loc;
     if (!(S > floor_sum)) {   // sum(rho) = 0, or at the caller's floor tol * N
-        if (tid == 0) st->done = 1;
+        if (cta == 0 && tid == 0) st->done = 1;
         return;
     }
-    if (tid == 0) {
+    if (cta == 0 && tid == 0) {
         st->total = S;
         st->rounds += 1;
     }
-    for (int j = wid; j < b; j += nw) {
+    cluster_sync();
+    for (int j = cta + kPropCluster * wid; j < b; j += kPropCluster * (kPropThreads / 32)) {
         const double u = philox_uniform(seed, 0u, (uint32_t)rnd, (uint32_t)j);
         const double target = u * S;
-        // smallest tile t with pre_incl[t] > target
-        int64_t lo = 0, hi = ntiles;
-        while (lo < hi) {
-            int64_t mid = (lo + hi) >> 1;
-            if (w.pre_incl[mid] > target) hi = mid; else lo = mid + 1;
+        // the first chunk that ends above target
+        int64_t t = -1;
+        double acc = 0.0;
+        unsigned hit = __ballot_sync(kAll, (lane < 31 ? __ldcg(w.pre + 32 * lane + 32) : S) > target);
+        int i = kPropChunks - 1;
+        if (hit) {
+            i = 32 * (__ffs(hit) - 1);
+            const int e = i + lane + 1;
+            hit = __ballot_sync(kAll, (e < kPropChunks ? __ldcg(w.pre + e) : S) > target);
+            i += __ffs(hit) - 1;
+            acc = __ldcg(w.pre + i);
+            // the first tile with mass in it that ends above target
+            const int64_t t1 = min((i + 1) * chunk, ntiles);
+            for (int64_t c0 = i * chunk; c0 < t1; c0 += 32) {
+                const double v = c0 + lane < t1 ? w.tile_sum[c0 + lane] : 0.0;
+                const double sv = warp_incl_scan(v);
+                hit = __ballot_sync(kAll, v > 0.0 && acc + sv > target);
+                if (hit) {
+                    const int f = __ffs(hit) - 1;
+                    const double before = __shfl_sync(kAll, sv, max(f - 1, 0));
+                    if (f > 0) acc += before;
+                    t = c0 + f;
+                    break;
+                }
+                acc += __shfl_sync(kAll, sv, 31);
+            }
         }
-        int64_t t = lo;
-        if (t == ntiles) {   // u*S rounded to >= S: last tile with mass
-            t = ntiles - 1;
+        if (t < 0) {   // u*S rounded to >= S, or a chunk's sum to below its end: the last tile with mass up to there
+            t = min((i + 1) * chunk, ntiles) - 1;
             while (t > 0 && !(w.tile_sum[t] > 0.0)) --t;
+            while (t < ntiles - 1 && !(w.tile_sum[t] > 0.0)) ++t;
+            acc = -INFINITY;
         }
         const int64_t base = t * kBM;
         const int cnt = (int)min((int64_t)kBM, N - base);
-        double acc = w.pre_excl[t];
         int64_t found = -1, last_pos = -1;
         for (int c0 = 0; c0 < cnt; c0 += 32) {
             const int rr = c0 + lane;
             const double v = rr < cnt ? rho[base + rr] : 0.0;
             const double sv = warp_incl_scan(v);
-            const unsigned pos = __ballot_sync(0xffffffffu, rr < cnt && v > 0.0);
+            const unsigned pos = __ballot_sync(kAll, rr < cnt && v > 0.0);
             if (pos) last_pos = base + c0 + 31 - __clz(pos);
-            const unsigned hit = __ballot_sync(0xffffffffu, rr < cnt && v > 0.0 && acc + sv > target);
+            hit = __ballot_sync(kAll, rr < cnt && v > 0.0 && acc + sv > target);
             if (hit) {
                 found = base + c0 + __ffs(hit) - 1;
                 break;
             }
-            acc += __shfl_sync(0xffffffffu, sv, 31);
+            acc += __shfl_sync(kAll, sv, 31);
         }
         if (found < 0) found = last_pos;   // rounding at the tile's upper edge
         if (found < 0) found = base;       // unreachable: the tile has mass
@@ -264,10 +308,10 @@ __device__ __forceinline__ void propose_body(FactorWs w, const double* __restric
     }
 }
 
-__global__ void __launch_bounds__(1024) k_propose(FactorWs w, const double* __restrict__ rho, int64_t N,
-                                                  int64_t ntiles, int b, int r, int greedy, uint64_t seed, int rnd,
-                                                  int64_t* __restrict__ proposals_out, double floor_sum) {
-    propose_body(w, rho, N, ntiles, b, r, greedy, seed, rnd, proposals_out, floor_sum);
+__global__ void __cluster_dims__(kPropCluster, 1, 1) __launch_bounds__(kPropThreads)
+    k_propose(FactorWs w, const double* __restrict__ rho, int64_t N, int64_t ntiles, int b, int r, uint64_t seed,
+              int rnd, int64_t* __restrict__ proposals_out, double floor_sum) {
+    propose_body(w, rho, N, ntiles, b, r, seed, rnd, proposals_out, floor_sum, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -376,11 +420,6 @@ __device__ __forceinline__ double rej_quot(double c, double s, double y) {
     return fma(fma(-q, s, c), y, q);
 }
 
-// All threads of the cluster; what they wrote to global memory before is visible after.
-__device__ __forceinline__ void rej_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // One cluster of kRejCluster CTAs per problem, `cta` the rank in it.  H is overwritten.
 __device__ __forceinline__ void arpc_reject_body(FactorWs w, int b, int r, uint64_t seed, int rnd,
                                                  int64_t* __restrict__ pivots, RejShared& sh, int cta) {
@@ -436,7 +475,7 @@ __device__ __forceinline__ void arpc_reject_body(FactorWs w, int b, int r, uint6
             }
         }
         const int n0 = c0 + kRejW;
-        rej_sync();
+        cluster_sync();
         if (n0 >= b) break;
         // columns n0 .. of the rows below the panel, all CTAs: a warp takes a row
         mask = (unsigned)*(volatile int*)&w.tpos[b - 1];
@@ -464,7 +503,7 @@ __device__ __forceinline__ void arpc_reject_body(FactorWs w, int b, int r, uint6
             for (int u = 0; u < 4; ++u)
                 if (lane + 32 * u <= l) Hr[lane + 32 * u] = x[u];
         }
-        rej_sync();
+        cluster_sync();
     }
     if (cta != 0) return;
     // (CTA 0's own columns of Lfull and its list of positions: ordered by the last barrier)
@@ -1028,7 +1067,11 @@ void launch_prepare_fp64(const double* X, int64_t N, int d, const FactorWs& w, d
 
 void launch_propose(const FactorWs& w, const double* rho, int64_t N, int b, int r, int greedy, uint64_t seed, int rnd,
                     int64_t* proposals, double floor_sum, cudaStream_t s) {
-    k_propose<<<1, 1024, 0, s>>>(w, rho, N, (N + kBM - 1) / kBM, b, r, greedy, seed, rnd, proposals, floor_sum);
+    const int64_t ntiles = (N + kBM - 1) / kBM;
+    if (greedy)
+        k_propose_greedy<<<1, 1024, 0, s>>>(w, ntiles, r, rnd, proposals);
+    else
+        k_propose<<<kPropCluster, kPropThreads, 0, s>>>(w, rho, N, ntiles, b, r, seed, rnd, proposals, floor_sum);
 }
 
 void launch_blockH(const FactorWs& w, int d, int b, double inv_eps, cudaStream_t s) {
@@ -1173,7 +1216,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
     for (int rnd = 0; rnd < rounds; ++rnd) {
         {
             TraceScope tr(kStPropose, s);
-            k_propose<<<1, 1024, 0, s>>>(w, rho, N, ntiles, b, r, greedy, opts->seed, rnd, proposals, opts->tol * N);
+            launch_propose(w, rho, N, b, r, greedy, opts->seed, rnd, proposals, opts->tol * N, s);
         }
         {
             TraceScope tr(kStGather, s);
@@ -1293,24 +1336,17 @@ __global__ void k_prepare_b(const BatchProb* __restrict__ P) {
     prepare_body(p.X, p.N, p.d, p.w, p.rho, blockIdx.x);
 }
 
-__global__ void __launch_bounds__(1024) k_propose_b(const BatchProb* __restrict__ P, int rnd) {
-    const BatchProb& p = P[blockIdx.x];
+__global__ void __cluster_dims__(kPropCluster, 1, 1) __launch_bounds__(kPropThreads)
+    k_propose_b(const BatchProb* __restrict__ P, int rnd) {   // a cluster per problem
+    const BatchProb& p = P[blockIdx.y];
     if (rnd >= p.rounds) {   // this problem has run its t = r/b rounds
-        if (threadIdx.x == 0) {
-            FactorState* st = p.w.st;
-            if (st->m > 0) {
-                st->sum_k += st->k;
-                st->eng_rounds += 1;
-            }
-            st->k += st->m;
-            st->kp += (st->m + 15) & ~15;
-            st->sum_m_sq += (long long)st->m * st->m;
-            st->m = 0;
-            st->done = 1;
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            commit_round(p.w.st);
+            p.w.st->done = 1;
         }
         return;
     }
-    propose_body(p.w, p.rho, p.N, p.ntiles, p.b, p.r, 0, p.seed, rnd, nullptr);
+    propose_body(p.w, p.rho, p.N, p.ntiles, p.b, p.r, p.seed, rnd, nullptr, 0.0, blockIdx.x);
 }
 
 __global__ void k_gather_b(const BatchProb* __restrict__ P) {
@@ -1419,7 +1455,7 @@ static int batch_enqueue_any(kevd_batch* h, cudaStream_t s) {
     const int np = h->nprob;
     k_prepare_b<<<dim3((unsigned)((h->nmax + 255) / 256), np), 256, 0, s>>>(h->dprobs);
     for (int rnd = 0; rnd < h->rounds; ++rnd) {
-        k_propose_b<<<np, 1024, 0, s>>>(h->dprobs, rnd);
+        k_propose_b<<<dim3(kPropCluster, np), kPropThreads, 0, s>>>(h->dprobs, rnd);
         k_gather_b<<<dim3((unsigned)((h->dmax + h->rmax + 7) / 8), np), 256, 0, s>>>(h->dprobs);
         k_blockH_b<<<dim3((h->bmax * h->bmax + kBlockHWarps - 1) / kBlockHWarps, 1, np), 32 * kBlockHWarps, 0, s>>>(
             h->dprobs);

@@ -31,8 +31,7 @@ struct FactorWs {
     double* tile_sum;  // ntiles: sum of rho over the tile
     double* tile_max;  // ntiles: max rho over the tile
     int64_t* tile_idx; // ntiles: lowest index attaining tile_max
-    double* pre_incl;  // ntiles: inclusive prefix of tile_sum
-    double* pre_excl;  // ntiles: exclusive prefix of tile_sum
+    double* pre;       // proposals: chunk offsets of the tile sums, then their 32 warp totals
     int64_t* prop;     // b: proposals of the round
     int32_t* acc_pos;  // b: accepted positions into prop
     int32_t* tpos;     // b: scratch of k_reject

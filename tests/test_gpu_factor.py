@@ -227,3 +227,23 @@ def test_reject_panel_edges(kevd, b):
     F = out["F"].cpu().numpy().T[:, : out["rank"]]
     assert np.max(np.abs(F - ref["F"])) < 1e-10
     assert np.max(np.abs(out["rho"].cpu().numpy() - ref["rho"])) < 1e-10
+
+
+# Proposals from 1,024 chunks of 64-row tiles: fewer tiles than lanes (1), one tile per chunk
+# with chunks left over (66,000 -> 1,032 tiles: two per chunk, the last half empty) and a short
+# last tile (70,001; 131,137).  same: all but 2,000 rows are one point, so that after a
+# round most tiles and chunks carry next to no mass.  Blocks of 3 and 5 leave the 4 x 4
+# tiles of H ragged.  The proposals are whole numbers and have to be the oracle's.
+@pytest.mark.parametrize("N,b,same", [(40, 3, False), (66000, 128, False), (70001, 16, True), (131137, 5, True)])
+def test_proposal_chunks(kevd, N, b, same):
+    X, eps, _ = make_config("ks200k", N=N)
+    if same:
+        X = X.copy()
+        X[1000:N - 1000] = X[1000]
+    ref = arpc(X, eps, 3 * b, b, 9)
+    out = kevd.rpchol_factor(_gpu(X), eps, 3 * b, mode="arpc", b=b, seed=9, record_proposals=True)
+    if any(_near_edge(ref["log"], rnd) for rnd in range(len(ref["log"]))):
+        pytest.skip("a draw of the oracle lies at an edge")
+    props = out["proposals"].cpu().numpy()
+    assert [p.tolist() for p in props[:len(ref["log"])]] == [lg["proposals"].tolist() for lg in ref["log"]]
+    assert out["pivots"].cpu().numpy()[: out["rank"]].tolist() == ref["pivots"].tolist()
