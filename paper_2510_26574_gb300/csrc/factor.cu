@@ -340,40 +340,73 @@ __global__ void k_gather(FactorWs w, const TX* __restrict__ X, const TF* __restr
 }
 
 // ---------------------------------------------------------------------------
-// a3 (part 2): H = K(S',S') - F(S',:) F(S',:)^T.  One warp per entry (j, l):
-// the lanes split the d- and k-long dot products and a shuffle tree adds them,
-// so each entry is a chain of ~(d + k)/32 FMAs instead of d + k.  H(j,l) and
-// H(l,j) go through the same lane assignment and the same tree, with the two
-// factors of each product swapped (fma is commutative in its first two
-// operands), so H is exactly symmetric.
+// a3 (part 2): H = K(S',S') - F(S',:) F(S',:)^T.  Lower-triangle tiles of 4 x 4
+// entries, a block each: a thread owns one entry and the terms c = g mod 8 of its sums (g the
+// thread's group), in four accumulators by c mod 32, which a fixed tree adds.  Both
+// halves of H come from one thread (the same value for (j, l) and (l, j)), so H is exactly
+// symmetric.  Bound: the FP64 pipe (17 cycles per warp operation and SM) over b^2 / 2
+// entries; 4 x 4 tiles leave 3 or 4 to each SM at b = 128.  Measured per round, b = 128, mean
+// k of 900: 21 us (one warp per entry of both halves with strided loads and a shuffle
+// tree per entry: 122 us; b = 64, mean k of 400: 12, was 28).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void blockH_body(FactorWs w, int d, int b, double inv_eps, int pair) {
+constexpr int kBlockHThreads = 128;   // 16 entries x 8 groups of terms
+
+// Terms c = g, g + 8, g + 16, ... of P(:,j) . P(:,l), P n x b row-major; partial sums per
+// c mod 32, added as a butterfly over 32 lanes adds them (16 first, then 8).
+__device__ __forceinline__ double pair_terms(const double* __restrict__ P, int b, int n, int j, int l, int g) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    int c0 = g;
+#pragma unroll 2
+    for (; c0 + 24 < n; c0 += 32) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const double* row = P + (size_t)(c0 + 8 * i) * b;
+            a[i] = fma(row[j], row[l], a[i]);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+        if (c0 + 8 * i < n) {
+            const double* row = P + (size_t)(c0 + 8 * i) * b;
+            a[i] = fma(row[j], row[l], a[i]);
+        }
+    return (a[0] + a[2]) + (a[1] + a[3]);
+}
+
+static int blockH_blocks(int b) { return ((b + 3) / 4) * ((b + 3) / 4 + 1) / 2; }
+
+__device__ __forceinline__ void blockH_body(FactorWs w, int d, int b, double inv_eps, int blk) {
+    __shared__ double part[2][8][16];
     const FactorState* st = w.st;
-    if (st->done) return;
-    if (pair >= b * b) return;
-    const int k = st->k;
-    const int j = pair / b, l = pair % b;
-    const int lane = threadIdx.x & 31;
-    double dx = 0.0, df = 0.0;
-    for (int c = lane; c < d; c += 32) dx = fma(w.XSP[(size_t)c * b + j], w.XSP[(size_t)c * b + l], dx);
-    for (int c = lane; c < k; c += 32) df = fma(w.FSP[(size_t)c * b + j], w.FSP[(size_t)c * b + l], df);
-    dx = warp_sum(dx);
-    df = warp_sum(df);
-    if (lane != 0) return;
+    const int nt = (b + 3) / 4;
+    if (st->done || blk >= nt * (nt + 1) / 2) return;
+    int J = (int)((sqrtf(8.f * blk + 1.f) - 1.f) * 0.5f);
+    while (J * (J + 1) / 2 > blk) --J;
+    while ((J + 1) * (J + 2) / 2 <= blk) ++J;
+    const int p = threadIdx.x & 15, g = threadIdx.x >> 4;
+    const int j = 4 * J + (p >> 2), l = 4 * (blk - J * (J + 1) / 2) + (p & 3);
+    const int jc = min(j, b - 1), lc = min(l, b - 1);
+    part[0][g][p] = pair_terms(w.XSP, b, d, jc, lc, g);
+    part[1][g][p] = pair_terms(w.FSP, b, st->k, jc, lc, g);
+    __syncthreads();
+    if (threadIdx.x >= 16 || j >= b || l > j) return;
+    double sum[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+        sum[q] = ((part[q][0][p] + part[q][4][p]) + (part[q][2][p] + part[q][6][p])) +
+                 ((part[q][1][p] + part[q][5][p]) + (part[q][3][p] + part[q][7][p]));
     double kv;
     if (w.prop[j] == w.prop[l]) {
         kv = 1.0;   // k(x, x) = exp(0)
     } else {
-        const double d2 = fmax(w.xnS[j] + w.xnS[l] - 2.0 * dx, 0.0);
+        const double d2 = fmax(w.xnS[j] + w.xnS[l] - 2.0 * sum[0], 0.0);
         kv = exp(-d2 * inv_eps);
     }
-    w.H[(size_t)j * b + l] = kv - df;
+    w.H[(size_t)j * b + l] = w.H[(size_t)l * b + j] = kv - sum[1];
 }
 
-constexpr int kBlockHWarps = 8;   // entries per 256-thread block
-
-__global__ void k_blockH(FactorWs w, int d, int b, double inv_eps) {
-    blockH_body(w, d, b, inv_eps, blockIdx.x * kBlockHWarps + (threadIdx.x >> 5));
+__global__ void __launch_bounds__(kBlockHThreads) k_blockH(FactorWs w, int d, int b, double inv_eps) {
+    blockH_body(w, d, b, inv_eps, blockIdx.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -1075,7 +1108,7 @@ void launch_propose(const FactorWs& w, const double* rho, int64_t N, int b, int 
 }
 
 void launch_blockH(const FactorWs& w, int d, int b, double inv_eps, cudaStream_t s) {
-    k_blockH<<<(unsigned)((b * b + kBlockHWarps - 1) / kBlockHWarps), 32 * kBlockHWarps, 0, s>>>(w, d, b, inv_eps);
+    k_blockH<<<blockH_blocks(b), kBlockHThreads, 0, s>>>(w, d, b, inv_eps);
 }
 
 cudaError_t launch_reject(const FactorWs& w, int b, int r, int greedy, uint64_t seed, int rnd, int64_t* pivots,
@@ -1225,8 +1258,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
         }
         {
             TraceScope tr(kStBlockH, s);
-            k_blockH<<<(unsigned)((b * b + kBlockHWarps - 1) / kBlockHWarps), 32 * kBlockHWarps, 0, s>>>(w, d, b,
-                                                                                                      inv_eps);
+            launch_blockH(w, d, b, inv_eps, s);
         }
         {
             TraceScope tr(kStReject, s);
@@ -1356,7 +1388,7 @@ __global__ void k_gather_b(const BatchProb* __restrict__ P) {
 
 __global__ void k_blockH_b(const BatchProb* __restrict__ P) {
     const BatchProb& p = P[blockIdx.z];
-    blockH_body(p.w, p.d, p.b, p.inv_eps, blockIdx.x * kBlockHWarps + (threadIdx.x >> 5));   // pairs past b*b return
+    blockH_body(p.w, p.d, p.b, p.inv_eps, blockIdx.x);   // blocks past the last tile return
 }
 
 __global__ void __cluster_dims__(kRejCluster, 1, 1) __launch_bounds__(kRejThreads)
@@ -1457,8 +1489,7 @@ static int batch_enqueue_any(kevd_batch* h, cudaStream_t s) {
     for (int rnd = 0; rnd < h->rounds; ++rnd) {
         k_propose_b<<<dim3(kPropCluster, np), kPropThreads, 0, s>>>(h->dprobs, rnd);
         k_gather_b<<<dim3((unsigned)((h->dmax + h->rmax + 7) / 8), np), 256, 0, s>>>(h->dprobs);
-        k_blockH_b<<<dim3((h->bmax * h->bmax + kBlockHWarps - 1) / kBlockHWarps, 1, np), 32 * kBlockHWarps, 0, s>>>(
-            h->dprobs);
+        k_blockH_b<<<dim3(blockH_blocks(h->bmax), 1, np), kBlockHThreads, 0, s>>>(h->dprobs);
         k_reject_b<<<dim3(kRejCluster, np), kRejThreads, 0, s>>>(h->dprobs, rnd);
         for (const auto& g : h->groups) {
             int st;
