@@ -1078,6 +1078,207 @@ static size_t engine_smem() {
     return std::max(stage, rtile);
 }
 
+// ---------------------------------------------------------------------------
+// Greedy rounds of an FP64 factor in one cooperative launch, for N <= 65,536.
+//
+// A greedy round is a step of r dependent ones, and in launches of its own (proposal,
+// gather, H, acceptance, engine) it is mostly their latency: 48 us at N = 2,048, d = 64.
+// Here a CTA owns a 64-row tile for all rounds, a thread a row (its residual in a register),
+// a third warp takes H and its root meanwhile, and a round has one grid barrier, after which
+// every CTA finds the argmax of the tiles' (max, index) pairs by itself.  What bounds it is
+// the chain of d + k dependent FP64 operations of 64 cycles that a row's value is defined by:
+// same operations in the same order as the kernels above, so the same bits: 15 us a round at
+// N = 2,048, k up to 128.  The line at 1,024 tiles: up to there a pair of tile statistics per thread and
+// 16 loads find the argmax, and all CTAs are resident (7 of 64 + 32 threads per SM); above,
+// a round's work on the FP64 pipe outweighs the launches.  Pairs alternate between two
+// buffers, since a CTA may be one round ahead of another's reading.
+// ---------------------------------------------------------------------------
+constexpr int kGreedyTiles = 1024;
+constexpr int kGreedyThreads = kBM + 32;
+constexpr int kGreedyChunk = 512;         // columns of X(p,:) and F(p,:) in shared memory
+constexpr int kGreedyPolls = 1 << 22;     // of the barrier, seconds in all
+
+__global__ void __launch_bounds__(kGreedyThreads) k_greedy(FactorWs w, const double* __restrict__ X, double* F,
+                                                           int64_t ldf, double* __restrict__ rho, int64_t N, int d,
+                                                           int r, int rounds, double inv_eps,
+                                                           int64_t* __restrict__ pivots,
+                                                           int64_t* __restrict__ proposals_out) {
+    __shared__ double sx[kGreedyChunk], sf[kGreedyChunk];
+    __shared__ double sv[3];
+    __shared__ int64_t si[3];
+    __shared__ double s_h, s_root;
+    __shared__ int s_ok;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const int ntiles = gridDim.x;
+    const int64_t row = (int64_t)blockIdx.x * kBM + tid;
+    const bool owns = tid < kBM && row < N;
+    const bool first = blockIdx.x == 0 && tid == 0;
+    int* const arrived = w.tpos;              // zero at launch
+    const double xi = owns ? w.xn[row] : 0.0;
+    const double* const Xi = X + (owns ? row : 0) * d;
+    const double* const Fi = F + (owns ? row : 0);
+    double rv = owns ? rho[row] : 0.0, total = 0.0;
+    int k = 0, ran = 0, done = 0;
+    long long sum_k = 0;
+    for (int rnd = 0; rnd < rounds; ++rnd) {
+        if (k >= r) {
+            done = 1;
+            break;
+        }
+        // ---- argmax of rho ----
+        const double* tmax = rnd & 1 ? w.pre : w.tile_max;
+        const int64_t* tidx = rnd & 1 ? reinterpret_cast<const int64_t*>(w.tile_sum) : w.tile_idx;
+        double v = -1.0;
+        int64_t p = LLONG_MAX;
+        for (int t = tid; t < ntiles; t += kGreedyThreads) argmax_merge(v, p, __ldcg(tmax + t), __ldcg(tidx + t));
+        warp_argmax(v, p);
+        if (lane == 0) {
+            sv[wid] = v;
+            si[wid] = p;
+        }
+        __syncthreads();
+        v = sv[0];
+        p = si[0];
+        argmax_merge(v, p, sv[1], si[1]);
+        argmax_merge(v, p, sv[2], si[2]);
+        if (!(v > 0.0)) {
+            done = 1;
+            break;
+        }
+        total = v;
+        ++ran;
+        if (first && proposals_out) proposals_out[rnd] = p;
+        // ---- X(p,:), F(p,:k) to shared memory, a chunk at a time; the row's chains; H in warp 2 ----
+        auto stage_x = [&](int c0) {
+            for (int c = tid; c < min(kGreedyChunk, d - c0); c += kGreedyThreads) sx[c] = X[p * d + c0 + c];
+        };
+        auto stage_f = [&](int c0) {
+            for (int c = tid; c < min(kGreedyChunk, k - c0); c += kGreedyThreads)
+                sf[c] = __ldcg(F + (int64_t)(c0 + c) * ldf + p);
+        };
+        const double xp = w.xn[p];
+        stage_x(0);
+        stage_f(0);
+        __syncthreads();
+        double acc = 0.0;                     // warp 2: terms c = lane mod 32 of F(p,:) . F(p,:)
+        for (int c0 = 0; c0 < d; c0 += kGreedyChunk) {
+            if (c0 > 0) {
+                __syncthreads();
+                stage_x(c0);
+                __syncthreads();
+            }
+            const int n = min(kGreedyChunk, d - c0);
+            if (owns) {
+#pragma unroll 16
+                for (int c = 0; c < n; ++c) acc = fma(Xi[c0 + c], sx[c], acc);
+            }
+        }
+        if (owns) acc = p == row ? 1.0 : exp(-fmax(xi + xp - 2.0 * acc, 0.0) * inv_eps);
+        for (int c0 = 0; c0 < k; c0 += kGreedyChunk) {
+            if (c0 > 0) {
+                __syncthreads();
+                stage_f(c0);
+                __syncthreads();
+            }
+            const int n = min(kGreedyChunk, k - c0);
+            if (owns) {
+#pragma unroll 16
+                for (int c = 0; c < n; ++c) acc = fma(-Fi[(int64_t)(c0 + c) * ldf], sf[c], acc);
+            } else if (wid == 2) {
+                for (int c = lane; c < n; c += 32) acc = fma(sf[c], sf[c], acc);
+            }
+        }
+        if (wid == 2) {
+            const double h = 1.0 - warp_sum(acc);
+            if (lane == 0) {
+                s_h = h;
+                s_root = sqrt(h);
+            }
+        }
+        __syncthreads();
+        if (!(s_h > 0.0)) {                   // greedy stops once H <= 0
+            done = 1;
+            break;
+        }
+        // ---- column k of F, the residual, the tile's (max, lowest index) ----
+        double rmax = -1.0;
+        int64_t ridx = LLONG_MAX;
+        if (owns) {
+            const double g = acc / s_root;
+            F[(int64_t)k * ldf + row] = g;
+            rv = fmax(rv - __dmul_rn(g, g), 0.0);
+            rmax = rv;
+            ridx = row;
+        }
+        if (first) pivots[k] = p;
+        sum_k += k;
+        ++k;
+        if (rnd + 1 == rounds) break;
+        if (wid < 2) {
+            warp_argmax(rmax, ridx);
+            if (lane == 0) {
+                sv[wid] = rmax;
+                si[wid] = ridx;
+            }
+        }
+        __syncthreads();
+        // ---- publish and wait for all tiles ----
+        if (tid == 0) {
+            argmax_merge(rmax, ridx, sv[1], si[1]);
+            (rnd & 1 ? w.tile_max : w.pre)[blockIdx.x] = rmax;
+            (rnd & 1 ? w.tile_idx : reinterpret_cast<int64_t*>(w.tile_sum))[blockIdx.x] = ridx;
+            __threadfence();
+            atomicAdd(arrived, 1);
+            const int want = (rnd + 1) * ntiles;
+            int got = 0;
+            for (int i = 0; i < kGreedyPolls; ++i) {
+                asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(got) : "l"(arrived) : "memory");
+                if (got >= want) break;
+            }
+            s_ok = got >= want;
+            if (got < want) w.st->timeout = 1;
+        }
+        __syncthreads();
+        if (!s_ok) break;
+    }
+    if (owns) rho[row] = rv;
+    if (first) {
+        FactorState* st = w.st;
+        st->k = k;
+        st->kp = 16 * k;
+        st->rounds = ran;
+        st->done = done;
+        st->total = total;
+        st->sum_m_sq = k;
+        st->sum_k = sum_k;
+        st->eng_rounds = k;
+    }
+}
+
+// CTAs of k_greedy for N rows, 0 where they cannot all be resident, N is past its line, or a
+// round's chain of d steps could outlast the barrier's polls.
+static int greedy_ctas(int64_t N, int d) {
+    const int64_t ntiles = (N + kBM - 1) / kBM;
+    if (ntiles > kGreedyTiles || d > (1 << 16)) return 0;
+    int dev = 0, nsm = 0, per_sm = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_greedy, kGreedyThreads, 0) != cudaSuccess)
+        return 0;
+    return coop && ntiles <= (int64_t)nsm * per_sm ? (int)ntiles : 0;
+}
+
+static cudaError_t launch_greedy(int ctas, FactorWs w, const double* X, double* F, int64_t ldf, double* rho, int64_t N,
+                                 int d, int r, int rounds, double inv_eps, int64_t* pivots, int64_t* proposals,
+                                 cudaStream_t s) {
+    cudaError_t e = cudaMemsetAsync(w.tpos, 0, sizeof(int32_t), s);
+    if (e != cudaSuccess) return e;
+    void* args[] = {&w, &X, &F, &ldf, &rho, &N, &d, &r, &rounds, &inv_eps, &pivots, &proposals};
+    return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(k_greedy), dim3(ctas), dim3(kGreedyThreads), args, 0,
+                                       s);
+}
+
 template <int TN>
 static cudaError_t prepare_engine() {
     return cudaFuncSetAttribute(k_engine<TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)engine_smem<TN>());
@@ -1246,7 +1447,12 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
         default: KEVD_CUDA_TRY(prepare_engine<16>()); break;
     }
 
-    for (int rnd = 0; rnd < rounds; ++rnd) {
+    const int gctas = greedy && !tc ? greedy_ctas(N, d) : 0;
+    if (gctas > 0) {
+        TraceScope tr(kStEngine, s);
+        KEVD_CUDA_TRY(launch_greedy(gctas, w, Xd, Fd, ldf, rho, N, d, r, rounds, inv_eps, pivots, proposals, s));
+    }
+    for (int rnd = 0; rnd < rounds && gctas == 0; ++rnd) {
         {
             TraceScope tr(kStPropose, s);
             launch_propose(w, rho, N, b, r, greedy, opts->seed, rnd, proposals, opts->tol * N, s);
@@ -1319,7 +1525,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
     if (oz) KEVD_CUDA_TRY(cudaMemcpyAsync(&herr, ow.flags, sizeof(int), cudaMemcpyDeviceToHost, s));
     KEVD_CUDA_TRY(cudaStreamSynchronize(s));
     trace_flush();
-    if (herr) return KEVD_ETIMEOUT;
+    if (herr || hs.timeout) return KEVD_ETIMEOUT;
     info->rank = hs.k;
     info->rounds = hs.rounds;
     info->trace_err = hs.final_sum;

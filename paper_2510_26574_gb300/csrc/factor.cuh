@@ -22,7 +22,7 @@ struct FactorState {
     long long sum_m_sq; // sum over rounds of m^2
     long long sum_k;    // sum over rounds with m > 0 of the rank before the round
     int32_t eng_rounds; // rounds with m > 0
-    int32_t pad2;
+    int32_t timeout;    // 1 if a bounded wait of the greedy rounds gave up
 };
 
 struct FactorWs {

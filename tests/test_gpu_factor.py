@@ -247,3 +247,25 @@ def test_proposal_chunks(kevd, N, b, same):
     props = out["proposals"].cpu().numpy()
     assert [p.tolist() for p in props[:len(ref["log"])]] == [lg["proposals"].tolist() for lg in ref["log"]]
     assert out["pivots"].cpu().numpy()[: out["rank"]].tolist() == ref["pivots"].tolist()
+
+
+# Greedy rounds in one launch (N <= 65,536) against the round's own kernels (more rows): the
+# second run appends copies of row 0, the first pivot, whose residual is 0 from then on, so that
+# no pivot and no other row's value may change by a bit.  N = 1 .. 65 are the edges of a
+# 64-row tile, 65,536 is the last N of the rule, d = 513 and 700 columns pass a 512-column chunk,
+# N = 40 with d = 1 stops before r (H <= 0 or rho = 0).
+@pytest.mark.parametrize("N,d,r", [(1, 3, 1), (40, 1, 40), (63, 7, 20), (64, 8, 64), (65, 513, 33), (900, 5, 700),
+                                   (65536, 4, 40)])
+def test_greedy_rounds_in_one_launch(kevd, N, d, r):
+    g = torch.Generator().manual_seed(N + d)
+    X = torch.rand(N, d, generator=g, dtype=torch.float64)
+    long = torch.cat([X, X[:1].expand(65600 - N, d)])
+    eps = 0.02 * d
+    a = kevd.rpchol_factor(X.cuda(), eps, r, mode="greedy", record_proposals=True)
+    b = kevd.rpchol_factor(long.cuda(), eps, r, mode="greedy", record_proposals=True)
+    assert a["rank"] == b["rank"] and a["rounds"] == b["rounds"]
+    k = a["rank"]
+    assert torch.equal(a["pivots"][:k], b["pivots"][:k])
+    assert torch.equal(a["proposals"][:a["rounds"]], b["proposals"][:a["rounds"]])
+    assert torch.equal(a["F"][:, :N], b["F"][:, :N])
+    assert torch.equal(a["rho"][:N], b["rho"][:N])
