@@ -687,13 +687,16 @@ __global__ void k_unit_cols(double* __restrict__ Y, int r) {
 // ---------------------------------------------------------------------------
 
 // Planes of the rows of the column-major rows x cols matrix A (ld lda); K = cols.
+cudaError_t oz_cut_rows(const double* A, int64_t lda, int rows, int K, int nq, uint16_t* P, int* ex, double* rmax,
+                        cudaStream_t s) {
+    k_rowmax_any<double><<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(A, lda, rows, K, rmax);
+    k_lift_planes<double, kDigits><<<dim3((unsigned)((nq + 7) / 8), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
+        A, lda, rows, K, nq, 0, rows, rmax, P, ex);
+    return cudaGetLastError();
+}
 static cudaError_t rr_row_planes(const double* A, int64_t lda, int rows, int cols, uint16_t* P, int* ex,
                                  double* rmax, cudaStream_t s) {
-    const int nq = lift_ldk(cols) / 16;
-    k_rowmax_any<double><<<(unsigned)((rows + 255) / 256), 256, 0, s>>>(A, lda, rows, cols, rmax);
-    k_lift_planes<double, kDigits><<<dim3((unsigned)((nq + 7) / 8), (unsigned)((rows + 31) / 32)), 256, 0, s>>>(
-        A, lda, rows, cols, nq, 0, rows, rmax, P, ex);
-    return cudaGetLastError();
+    return oz_cut_rows(A, lda, rows, cols, lift_ldk(cols) / 16, P, ex, rmax, s);
 }
 
 // Planes of the columns of the column-major rows x cols matrix A (ld rows): plane

@@ -71,24 +71,41 @@ static FactorWs carve_factor(void* base, int64_t N, int d, int r, int b, size_t*
     if (oz && !tc) {
         OzWs o;
         w.ldD = (N + 1) / 2 * 2;
-        w.Dx = c.take<double>((size_t)w.ldD * b);
-        w.Df = c.take<double>((size_t)w.ldD * b);
         o.ldX = (d + 15) / 16 * 16;
-        o.ldF = (int)(((int64_t)r + 15 * (int64_t)std::max(rounds_max, 1) + 15) / 16 * 16);
+        const int64_t ldF = ((int64_t)r + 15 * (int64_t)std::max(rounds_max, 1) + 15) / 16 * 16;
+        o.ldF = (int)std::min(ldF, (int64_t)std::max(rounds_max, 1) * ((b + 15) / 16 * 16));
         o.ldR = (b + 15) / 16 * 16;
         o.ldLi = (b + 1) / 2 * 2;
+        // The size is that of every array by itself with rows as they are and r + 15 rounds
+        // columns of F; the planes' rows are padded to 128, which two things make room for: F's
+        // columns are also at most a padded block per round, and arrays that are never alive together
+        // share memory (the pivot panels, read before R is written, lie in R's planes, L^-1, formed
+        // after Dx is read, in Dx).  Small N, where they do not fit, take more.
+        Carver exact(nullptr);
+        exact.off = c.off;
+        for (int u = 0; u < 2; ++u) exact.take<double>((size_t)w.ldD * b);
+        for (const int64_t n : {(int64_t)N, (int64_t)b})
+            for (const int64_t ld : {(int64_t)o.ldX, ldF, (int64_t)o.ldR}) exact.take<uint16_t>((size_t)kDigits * n * ld);
+        for (const int64_t n : {(int64_t)N, (int64_t)N, (int64_t)b, (int64_t)b}) exact.take<int>(n);
+        exact.take<double>((size_t)b * o.ldLi);
+        exact.take<int>(4);
+        const size_t px = oz_tile_elems(b, o.ldX / 16, kDigits), pf = oz_tile_elems(b, o.ldF / 16, kDigits);
+        const size_t lp = oz_tile_elems(b, o.ldR / 16, kDigits);
+        w.Dx = c.take<double>(std::max((size_t)w.ldD * b, lp / 4 + (size_t)b * o.ldLi));
+        w.Df = c.take<double>((size_t)w.ldD * b);
+        o.Lp = reinterpret_cast<uint16_t*>(w.Dx);
+        o.Linv = reinterpret_cast<double*>(o.Lp + lp);
         o.Xp = c.take<uint16_t>(oz_tile_elems(N, o.ldX / 16, kDigits));
         o.xe = c.take<int>(N);
         o.Fp = c.take<uint16_t>(oz_tile_elems(N, o.ldF / 16, kDigits));
-        o.Rp = c.take<uint16_t>(oz_tile_elems(N, o.ldR / 16, kDigits));
+        o.Rp = c.take<uint16_t>(std::max(oz_tile_elems(N, o.ldR / 16, kDigits), px + pf));
+        o.PXp = o.Rp;
+        o.PFp = o.Rp + px;
         o.re = c.take<int>(N);
-        o.PXp = c.take<uint16_t>(oz_tile_elems(b, o.ldX / 16, kDigits));
         o.pxe = c.take<int>(b);
-        o.PFp = c.take<uint16_t>(oz_tile_elems(b, o.ldF / 16, kDigits));
-        o.Lp = c.take<uint16_t>(oz_tile_elems(b, o.ldR / 16, kDigits));
         o.le = c.take<int>(b);
-        o.Linv = c.take<double>((size_t)b * o.ldLi);
         o.flags = c.take<int>(4);
+        c.off = std::max(c.off, exact.off);
         if (ow) *ow = o;
     }
     *bytes = c.off;
@@ -1323,6 +1340,25 @@ void launch_finalize(const FactorWs& w, const double* rho, int64_t N, cudaStream
     k_finalize<<<1, 1024, 0, s>>>(w, rho, N);
 }
 
+cudaError_t launch_linv(const FactorWs& w, const OzWs& o, int b, cudaStream_t s) {
+    // (the largest block's, so that calls with other blocks leave the limit as it is)
+    constexpr int kMost = (128 * 128 + 2 * 128) * (int)sizeof(double);
+    const cudaError_t e = cudaFuncSetAttribute(k_linv, cudaFuncAttributeMaxDynamicSharedMemorySize, kMost);
+    if (e != cudaSuccess) return e;
+    k_linv<<<(b + kLinvWarps - 1) / kLinvWarps, 32 * kLinvWarps, ((size_t)b * b + 2 * b) * sizeof(double), s>>>(w, o, b);
+    k_linv_planes<<<(b + 3) / 4, 128, 0, s>>>(w, o, b);
+    return cudaGetLastError();
+}
+
+cudaError_t oz_cut_rowmajor(const double* X, int64_t N, int K, uint16_t* P, int* ex, cudaStream_t s) {
+    OzWs o{};
+    o.Xp = P;
+    o.xe = ex;
+    o.ldX = (K + 15) / 16 * 16;
+    k_xplanes<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(X, N, K, o);
+    return cudaGetLastError();
+}
+
 }  // namespace kevd
 
 using namespace kevd;
@@ -1352,7 +1388,7 @@ static bool pl_engine_for(const kevd_opts* o, int64_t N, int d, int r, int b, bo
 // ozmm.cu) for ARPC with b >= 32 (each round's block of F's planes is padded to
 // 16 columns) and N < 2^31, unless KEVD_ENGINE=fp64 asks for the FP64-pipe
 // engine; the workspace then holds two N x b product arrays and the planes.
-static bool oz_engine_enabled() {
+bool kevd::oz_engine_enabled() {
     const char* e = getenv("KEVD_ENGINE");
     return !(e && e[0] == 'f');
 }
@@ -1429,15 +1465,12 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
             k_prepare<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(Xd, N, d, w, rho);
             if (oz) {
                 KEVD_CUDA_TRY(kexp_table(s, &exp_tbl));
-                k_xplanes<<<(unsigned)((N + 31) / 32), 256, 0, s>>>(Xd, N, d, ow);
+                KEVD_CUDA_TRY(oz_cut_rowmajor(Xd, N, d, ow.Xp, ow.xe, s));
                 KEVD_CUDA_TRY(cudaMemsetAsync(ow.flags, 0, sizeof(int), s));
             }
         }
     }
     KEVD_LAUNCH_CHECK();
-    if (oz)
-        KEVD_CUDA_TRY(cudaFuncSetAttribute(k_linv, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           (int)(((size_t)b * b + 2 * b) * sizeof(double))));
     const int tn = b <= 8 ? 1 : b <= 16 ? 2 : b <= 32 ? 4 : b <= 64 ? 8 : 16;
     switch (tn) {
         case 1: KEVD_CUDA_TRY(prepare_engine<1>()); break;
@@ -1486,9 +1519,7 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
                 // R = K(:, T) - F F(T,:)^T; G = R L^-T into F(:, k:k+m), on the tensor cores; rho
                 k_rprep<<<(unsigned)std::min<int64_t>((N + 31) / 32, 152 * 8), 2 * ow.ldR, 0, s>>>(w, ow, N, inv_eps,
                                                                                                    exp_tbl);
-                k_linv<<<(b + kLinvWarps - 1) / kLinvWarps, 32 * kLinvWarps, ((size_t)b * b + 2 * b) * sizeof(double), s>>>(
-                    w, ow, b);
-                k_linv_planes<<<(b + 3) / 4, 128, 0, s>>>(w, ow, b);
+                KEVD_CUDA_TRY(launch_linv(w, ow, b, s));
                 KEVD_CUDA_TRY(launch_ozmm(oR, oL, N, b, -2, w.st, Fd, ldf, ldf, ow.Fp, ow.ldF / 16, ow.flags, s));
                 k_rho_update<<<(unsigned)((N + 63) / 64), 256, 0, s>>>(w, Fd, ldf, rho, N);
             } else {

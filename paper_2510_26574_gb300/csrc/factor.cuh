@@ -99,6 +99,10 @@ void launch_blockH(const FactorWs& w, int d, int b, double inv_eps, cudaStream_t
 cudaError_t launch_reject(const FactorWs& w, int b, int r, int greedy, uint64_t seed, int rnd, int64_t* pivots,
                           cudaStream_t s);
 void launch_finalize(const FactorWs& w, const double* rho, int64_t N, cudaStream_t s);
+// L(T,T)^-1 of the round into o.Linv and its digit planes o.Lp, o.le.
+cudaError_t launch_linv(const FactorWs& w, const OzWs& o, int b, cudaStream_t s);
+// False under KEVD_ENGINE=fp64 (products on the FP64 pipe).
+bool oz_engine_enabled();
 
 // Bytes of PanelWs::planes, and the half chunks of X and of a row block.
 inline size_t tc_plane_bytes(int64_t N, int d, int r, int* nxh, int* nH) {

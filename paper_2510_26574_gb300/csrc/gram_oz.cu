@@ -599,11 +599,11 @@ cudaError_t launch_gram_oz(const double* F, int64_t ldf, int64_t N, int rank, co
                   : gram_oz_slabs<7>(enc, S, ns, 0, F, ldf, N, rank, sa, sc, Ecol, gpart, planes, flags, A, C, s);
 }
 
-// Panels of the low-memory form: the planes stay within 256 MiB (its panel takes 128), and a
+// Panels of the low-memory form: the planes stay within 64 MiB (its panel takes 128), and a
 // split may be as short as 1,024 rows, since one panel has few tiles.  Seven digits, as the
 // FP64-pipe Grams that it replaces have the error of.  Measured on N = 60,000, rank 512
 // (factor and normalisation without stored F): 61.2 ms, 80.4 with the FP64-pipe Grams.
-constexpr size_t kOzPanelBudget = (size_t)256 << 20;
+constexpr size_t kOzPanelBudget = (size_t)64 << 20;
 static int64_t oz_panel_rows(int64_t P, int rank) {
     const int64_t most = (int64_t)(kOzPanelBudget / ((size_t)2 * kDigits * oz_rank_pad(rank) * 2)) / 256 * 256;
     const int64_t nslab = (P + std::max<int64_t>(most, 256) - 1) / std::max<int64_t>(most, 256);

@@ -51,4 +51,11 @@ cudaError_t launch_ozmm(const OzOperand& A, const OzOperand& B, int64_t M, int n
                         double* C, int64_t ldc, int64_t c_koff, uint16_t* pout, int pout_nq, int* flags,
                         cudaStream_t s, int digits = 7, const double* rowdiv = nullptr, bool strict = false);
 
+// Operands of launch_ozmm cut from FP64 matrices, seven digits, one exponent per operand row
+// (ex), zero past the K columns.  The rows of a row-major N x K matrix (factor.cu) ...
+cudaError_t oz_cut_rowmajor(const double* X, int64_t N, int K, uint16_t* P, int* ex, cudaStream_t s);
+// ... and the rows of a column-major rows x K matrix, rmax scratch (eig.cu).
+cudaError_t oz_cut_rows(const double* A, int64_t lda, int rows, int K, int nq, uint16_t* P, int* ex, double* rmax,
+                        cudaStream_t s);
+
 }  // namespace kevd
