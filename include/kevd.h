@@ -345,9 +345,9 @@ int constant_eigvec_fix(double* U, int64_t N, int32_t k, void* workspace, size_t
  *   pivots    device int64[rank]; an index outside [0, N) gives KEVD_EINVAL.
  *   W, ldw    the factor's W (its leading rank x rank block).
  *   dtil, qtil, A, C, errors  as bistoch_normalize.
- *   The Grams run on the tensor cores, with at most 256 MiB of digit planes
- *   beside the panel; a workspace without them (O(N + r d + P r) doubles) is
- *   accepted and takes the FP64-pipe Grams.
+ *   The products, the solve and the Grams run on the tensor cores, with at most
+ *   64 MiB of digit planes beside the panel; a workspace without them
+ *   (O(N + r d + P r) doubles) is accepted and takes the FP64-pipe forms.
  *
  * eig_topk_lowmem -- eig_topk for the same factor: the r x r stage is
  * eig_topk's; the lift is U = D~^-1 K(:,S) (W^-T Y) per panel.  N <= 2^31 - 1.

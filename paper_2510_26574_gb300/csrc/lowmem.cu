@@ -32,9 +32,11 @@
 //
 // The lift of eig_topk_lowmem: U = D~^-1 K(:,S) (W^-T Y), per panel.
 //
-// DGEMM, DGEMV and the triangular solves are cuBLAS calls (plain library
-// products); set-up, exp, residual update, statistics and Grams are kernels of
-// this library.
+// The panels' dot products, the products with L^-1 and the solve with W run on the tensor
+// cores from seven digit planes (ozmm.cu); K(p,S) Z, DGEMV and the small triangular solves are
+// cuBLAS calls, and so are all products below the rules' lines (lm_round, carve_lm_norm)
+// and under KEVD_ENGINE=fp64.  Set-up, exp, residual update, statistics and Grams are kernels
+// of this library.
 #include <cublas_v2.h>
 
 #include <algorithm>
@@ -45,6 +47,8 @@
 #include "factor.cuh"
 #include "gram_tc.cuh"
 #include "lowmem.cuh"
+#include "oz_digits.cuh"
+#include "ozgemm.cuh"
 #include "trace.cuh"
 
 cudaError_t kevd_gram_weighted(const double* F, int64_t ldf, int64_t N, int rank, const double* wa, const double* wc,
@@ -106,6 +110,35 @@ static LmPanel carve_panel(Carver& c, int64_t N, int d, int r, bool own_xn = tru
     return p;
 }
 
+// Scratch of the products on the tensor cores (seven digit planes, ozmm.cu) for `rows`
+// rows of a panel at a time.  One buffer holds the left operand of each product in turn.
+struct LmOz {
+    uint16_t *Ap, *Bp;    // the rows' operand; columns of Z, or rows of W
+    uint16_t* XSp;        // X(S,:)
+    int *ae, *be, *xse;
+    double* rmax;         // row maxima
+    double *C, *C2;       // products
+    int* flags;           // bit 2: a bounded wait gave up
+    int nqx;
+    int64_t rows;
+};
+constexpr int kLmBlock = 128;                          // columns of F solved at a time in the normalisation
+constexpr int64_t kLmOzRows = 1024;                    // fewest rows worth a launch
+constexpr size_t kLmScratch = (size_t)64 << 20;        // of the normalisation
+
+// The parts that depend on the rows: aq quarters of the left operand, bn x bq quarters of the
+// right one, cn columns of the product.
+static void carve_lm_oz(Carver& c, LmOz& o, int64_t rows, int aq, int bn, int bq, int cn) {
+    o.rows = rows;
+    o.Ap = c.take<uint16_t>(oz_tile_elems(rows, aq, kDigits));
+    o.Bp = c.take<uint16_t>(oz_tile_elems(bn, bq, kDigits));
+    o.ae = c.take<int>(rows);
+    o.be = c.take<int>(bn);
+    o.rmax = c.take<double>(std::max<int64_t>(rows, bn));
+    o.C = c.take<double>((size_t)rows * cn);
+    o.C2 = c.take<double>((size_t)rows * cn);
+}
+
 // |x_i|^2, summed in the order of the FP64 path's set-up kernel.
 __global__ void k_lm_norms(const double* __restrict__ X, int64_t N, int d, double* __restrict__ xn) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -155,15 +188,72 @@ __global__ void k_lm_kexp(double* __restrict__ Kp, int64_t P, int64_t Pc, int n,
     *kp = v;
 }
 
+// A -= C, a column per grid row, `rows` of the rows of both.
+__global__ void k_lm_sub(double* __restrict__ A, int64_t lda, const double* __restrict__ C, int64_t ldc, int64_t rows) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < rows) A[blockIdx.y * lda + i] -= C[blockIdx.y * ldc + i];
+}
+
+// A = C + D, likewise.
+__global__ void k_lm_sum(double* __restrict__ A, int64_t lda, const double* __restrict__ C,
+                         const double* __restrict__ D, int64_t ldc, int64_t rows) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < rows) A[blockIdx.y * lda + i] = C[blockIdx.y * ldc + i] + D[blockIdx.y * ldc + i];
+}
+
+// The diagonal blocks of W (lower triangles), kLmBlock columns, zero elsewhere.
+__global__ void k_lm_diag(const double* __restrict__ W, int64_t ldw, double* __restrict__ E, int r) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= r) return;
+    const int j0 = a / kLmBlock * kLmBlock, c = blockIdx.y;
+    E[(size_t)c * r + a] = j0 + c <= a ? W[(int64_t)(j0 + c) * ldw + a] : 0.0;
+}
+
+// The unit blocks of the diagonal, kLmBlock columns: E(a, a mod kLmBlock) = 1.
+__global__ void k_lm_unit(double* __restrict__ E, int r) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a < r) E[(size_t)(a % kLmBlock) * r + a] = 1.0;
+}
+
 // Kp(0:Pc, 0:n) = K(i0:i0+Pc, S_0:S_n) [/ rowdiv]: one DGEMM of the panel's
 // rows of X against X(S,:), then the exp kernel.
 static int kernel_panel(cublasHandle_t h, const double* X, int d, int64_t i0, int64_t Pc, int n, const LmPanel& p,
-                        const int64_t* piv, double inv_eps, const double* rowdiv, cudaStream_t s) {
+                        const int64_t* piv, double inv_eps, const double* rowdiv, cudaStream_t s,
+                        const LmOz* o = nullptr) {
     const double one = 1.0, zero = 0.0;
-    LM_BLAS(cublasDgemm(h, CUBLAS_OP_T, CUBLAS_OP_N, (int)Pc, n, d, &one, X + i0 * d, d, p.XS, d, &zero, p.Kp,
-                        (int)p.P));
+    if (o) {   // the planes of X(S,:) are the caller's
+        for (int64_t r0 = 0; r0 < Pc; r0 += o->rows) {
+            const int64_t rows = std::min(o->rows, Pc - r0);
+            KEVD_CUDA_TRY(oz_cut_rowmajor(X + (i0 + r0) * d, rows, d, o->Ap, o->ae, s));
+            KEVD_CUDA_TRY(launch_ozmm(OzOperand{o->Ap, o->nqx, o->ae, 0}, OzOperand{o->XSp, o->nqx, o->xse, 0}, rows, n,
+                                      16 * o->nqx, nullptr, p.Kp + r0, p.P, 0, nullptr, 0, o->flags, s));
+        }
+    } else {
+        LM_BLAS(cublasDgemm(h, CUBLAS_OP_T, CUBLAS_OP_N, (int)Pc, n, d, &one, X + i0 * d, d, p.XS, d, &zero, p.Kp,
+                            (int)p.P));
+    }
     const int64_t tot = Pc * n;
     k_lm_kexp<<<(unsigned)((tot + 255) / 256), 256, 0, s>>>(p.Kp, p.P, Pc, n, i0, p.xn, p.xnS, piv, inv_eps, rowdiv);
+    KEVD_LAUNCH_CHECK();
+    return KEVD_OK;
+}
+
+// G = R M^-T for nb <= 128 columns of `rows` rows of the panel, in place, from the planes of M
+// and of its explicit inverse: the product with the inverse, corrected once by its residual,
+// without which the error against 64 bits was up to three times that of a triangular solve.
+static int solve_block(const LmOz& o, double* R, int64_t P, int rows, int nb, const OzOperand& mat,
+                       const OzOperand& inv, cudaStream_t s) {
+    const int nq = (nb + 15) / 16;
+    const dim3 grid((rows + 255) / 256, nb);
+    const OzOperand A{o.Ap, nq, o.ae, 0};
+    KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
+    KEVD_CUDA_TRY(launch_ozmm(A, inv, rows, nb, 16 * nq, nullptr, o.C, o.rows, 0, nullptr, 0, o.flags, s));
+    KEVD_CUDA_TRY(oz_cut_rows(o.C, o.rows, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
+    KEVD_CUDA_TRY(launch_ozmm(A, mat, rows, nb, 16 * nq, nullptr, o.C2, o.rows, 0, nullptr, 0, o.flags, s));
+    k_lm_sub<<<grid, 256, 0, s>>>(R, P, o.C2, o.rows, rows);
+    KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
+    KEVD_CUDA_TRY(launch_ozmm(A, inv, rows, nb, 16 * nq, nullptr, o.C2, o.rows, 0, nullptr, 0, o.flags, s));
+    k_lm_sum<<<grid, 256, 0, s>>>(R, P, o.C, o.C2, o.rows, rows);
     KEVD_LAUNCH_CHECK();
     return KEVD_OK;
 }
@@ -314,7 +404,7 @@ struct LmFactorWs {
 };
 
 static LmFactorWs carve_lm_factor(void* base, int64_t N, int d, int r, int b, size_t* bytes) {
-    LmFactorWs L;
+    LmFactorWs L{};
     size_t fb = 0;
     L.w = carve_factor_fp64(base, N, d, r, b, &fb);
     Carver c(base);
@@ -326,6 +416,51 @@ static LmFactorWs carve_lm_factor(void* base, int64_t N, int d, int r, int b, si
     return L;
 }
 
+// The factor's dot products X X(S,:)^T and its products with L^-1 run on the tensor cores, with
+// their scratch taken out of the panel's own memory, so that the workspace stays as it is:
+// `rows` of the P rows are formed at a time, and the rest of the buffer holds the operands (14
+// max(d, 128) bytes a row beside the panel's 8 r).  K(p,S) Z stays with the library's FP64
+// GEMM: Z's entries reach far above 1, and digits cut by the largest entry of a row left rho
+// with 1.4 times the GEMM's error against 64 bits.  For blocks from 32 on (the FP64 path's line:
+// below, a block leaves most of a 128-row tile of the right operand empty) and from 1,024
+// rows on; otherwise the library's FP64 products and solves serve.
+struct LmRound {
+    LmPanel p;     // Kp and P of the rows formed at a time
+    LmOz o;
+    OzWs li;       // L(T,T)^-1
+};
+static size_t carve_lm_round(Carver& c, LmRound& q, int64_t rows, int d, int r, int b) {
+    q.o.nqx = (d + 15) / 16;
+    q.p.P = rows;
+    q.p.Kp = c.take<double>((size_t)rows * r);
+    carve_lm_oz(c, q.o, rows, std::max(q.o.nqx, kLmBlock / 16), 0, 0, 0);
+    q.o.XSp = c.take<uint16_t>(oz_tile_elems(r, q.o.nqx, kDigits));
+    q.o.xse = c.take<int>(r);
+    q.o.flags = c.take<int>(4);
+    q.li.ldR = (b + 15) / 16 * 16;
+    q.li.ldLi = (b + 1) / 2 * 2;
+    q.li.Lp = c.take<uint16_t>(oz_tile_elems(b, q.li.ldR / 16, kDigits));
+    q.li.le = c.take<int>(b);
+    q.li.Linv = c.take<double>((size_t)b * q.li.ldLi);
+    return c.off;
+}
+static bool lm_round(const LmPanel& p, int64_t N, int d, int r, int b, LmRound* q) {
+    if (b < 32 || !oz_engine_enabled()) return false;
+    const size_t bytes = (size_t)p.P * r * sizeof(double);
+    q->p = p;
+    int64_t lo = 0, hi = std::min<int64_t>(p.P, (N + 127) / 128 * 128) / 128;   // in tiles of 128 rows
+    while (lo < hi) {
+        const int64_t mid = (lo + hi + 1) / 2;
+        Carver c(nullptr);
+        LmRound t{};
+        if (carve_lm_round(c, t, 128 * mid, d, r, b) <= bytes) lo = mid; else hi = mid - 1;
+    }
+    if (128 * lo < kLmOzRows) return false;
+    Carver c(p.Kp);
+    carve_lm_round(c, *q, 128 * lo, d, r, b);
+    return true;
+}
+
 struct LmNormWs {
     LmPanel p;
     double* ones;   // P
@@ -335,12 +470,26 @@ struct LmNormWs {
     double* wa;     // P: 1/d~^2 (tensor-core Grams: 1/d~)
     double* wc;     // P: 1/q~ (tensor-core Grams: 1/sqrt(q~))
     double* gpart;  // Gram split partials of one panel
-    int* flags;     // [0] bit 0: d~ <= 0, bit 1: q~ <= 0, bit 2: pivot out of range; [1]: the Grams' flags
+    int* flags;     // [0] bit 0: d~ <= 0, bit 1: q~ <= 0, bit 2: pivot out of range; [1], [2]: a bounded wait of
+                    // the Grams, of the products gave up (bit 2)
     // tensor-core Grams of one panel
     uint32_t *sa_hi, *sc_hi, *cmax;
     int* ecol;
     uint16_t* planes;
+    // tensor-core products and solve, o.rows rows of the panel at a time, in the memory of
+    // the Grams' planes; o.rows = 0: the library's FP64 products
+    LmOz o;
+    double* Winv;     // rank x kLmBlock: W's diagonal blocks, then their inverses
+    uint16_t *Wd, *Wp;   // the planes of both
+    int *wde, *we;
 };
+
+// The products' scratch for `rows` rows, in base (a size with base = NULL).
+static size_t carve_lm_solve(void* base, LmOz& o, int64_t rows, int rank) {
+    Carver c(base);
+    carve_lm_oz(c, o, rows, std::max(o.nqx, kLmBlock / 16), rank, kLmBlock / 16, kLmBlock);
+    return c.off;
+}
 
 // tc: with the buffers of the tensor-core Grams (without them a smaller workspace still
 // serves, by the FP64-pipe Grams).
@@ -363,7 +512,28 @@ static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, bool tc, s
         L.sc_hi = c.take<uint32_t>(P);
         L.cmax = c.take<uint32_t>(2 * (size_t)rank);
         L.ecol = c.take<int>(2 * (size_t)rank);
-        L.planes = c.take<uint16_t>(gram_oz_panel_plane_bytes(P, rank) / 2);
+        // products and solve from rank 32 on, with as many rows as 64 MiB hold (of X's planes, or
+        // of 128 columns of F and of a product), at least 1,024
+        L.o.nqx = (d + 15) / 16;
+        int64_t rows = (std::min<int64_t>(P, N) + 127) / 128 * 128;
+        LmOz t = L.o;
+        while (rows >= kLmOzRows && carve_lm_solve(nullptr, t, rows, rank) > kLmScratch) rows = rows / 256 * 128;
+        if (rank < 32 || rows < kLmOzRows) rows = 0;
+        const size_t solve = rows ? carve_lm_solve(nullptr, t, rows, rank) : 0;
+        char* scratch = c.take<char>(std::max(solve, gram_oz_panel_plane_bytes(P, rank)));
+        L.planes = reinterpret_cast<uint16_t*>(scratch);
+        if (rows) {
+            if (base) carve_lm_solve(scratch, L.o, rows, rank);
+            L.o.rows = rows;
+            L.o.XSp = c.take<uint16_t>(oz_tile_elems(rank, L.o.nqx, kDigits));
+            L.o.xse = c.take<int>(rank);
+            L.Winv = c.take<double>((size_t)rank * kLmBlock);
+            L.Wd = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
+            L.Wp = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
+            L.wde = c.take<int>(rank);
+            L.we = c.take<int>(rank);
+        }
+        L.o.flags = L.flags + 2;
     }
     *bytes = c.off;
     return L;
@@ -380,6 +550,58 @@ static bool aligned(const void* p) { return reinterpret_cast<uintptr_t>(p) % kAl
 static int solve_ww(cublasHandle_t h, const double* W, int64_t ldw, int rank, double* y) {
     LM_BLAS(cublasDtrsv(h, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, rank, W, (int)ldw, y, 1));
     LM_BLAS(cublasDtrsv(h, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT, rank, W, (int)ldw, y, 1));
+    return KEVD_OK;
+}
+
+// The planes of W's diagonal blocks and of their inverses.
+static int solve_setup(cublasHandle_t h, const double* W, int64_t ldw, int rank, const LmNormWs& L, cudaStream_t s) {
+    const double one = 1.0;
+    k_lm_diag<<<dim3(grid1(rank), kLmBlock), 256, 0, s>>>(W, ldw, L.Winv, rank);
+    KEVD_CUDA_TRY(oz_cut_rows(L.Winv, rank, rank, kLmBlock, kLmBlock / 16, L.Wd, L.wde, L.o.rmax, s));
+    KEVD_CUDA_TRY(cudaMemsetAsync(L.Winv, 0, (size_t)rank * kLmBlock * sizeof(double), s));
+    k_lm_unit<<<grid1(rank), 256, 0, s>>>(L.Winv, rank);
+    KEVD_LAUNCH_CHECK();
+    for (int j = 0; j < rank; j += kLmBlock) {
+        const int nb = std::min(kLmBlock, rank - j);
+        LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_LEFT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, nb, nb, &one,
+                            W + (int64_t)j * ldw + j, (int)ldw, L.Winv + j, rank));
+    }
+    KEVD_CUDA_TRY(oz_cut_rows(L.Winv, rank, rank, kLmBlock, kLmBlock / 16, L.Wp, L.we, L.o.rmax, s));
+    return KEVD_OK;
+}
+
+// F_p = K(p,S) W^-T in place on the tensor cores, 128 columns at a time: F_J = R_J W_JJ^-T with
+// the block's explicit inverse, then R(:, > J) -= F_J W(> J, J)^T.  Exponents are per row, so
+// that W may be of any scale.  Measured at N = 60,000, rank 356: 7.0 ms of the Gram
+// stage, 18.5 with the library's triangular solve.
+static int solve_panel(const double* W, int64_t ldw, int rank, int64_t Pc, const LmNormWs& L, cudaStream_t s) {
+    const LmOz& o = L.o;
+    const int64_t P = L.p.P;
+    constexpr int nq = kLmBlock / 16;
+    const size_t tile = oz_tile_elems(kLmBlock, nq, kDigits);   // a diagonal block's planes
+    for (int j = 0; j < rank; j += kLmBlock) {
+        const int nb = std::min(kLmBlock, rank - j), rest = rank - j - nb;
+        if (rest > 0)
+            KEVD_CUDA_TRY(oz_cut_rows(W + (int64_t)j * ldw + j + nb, ldw, rest, nb, nq, o.Bp, o.be, o.rmax, s));
+        for (int64_t r0 = 0; r0 < Pc; r0 += o.rows) {
+            const int rows = (int)std::min(o.rows, Pc - r0);
+            double* R = L.p.Kp + (int64_t)j * P + r0;
+            const size_t at = (size_t)(j / kLmBlock) * tile;
+            const int st = solve_block(o, R, P, rows, nb, OzOperand{L.Wd + at, nq, L.wde + j, 0},
+                                       OzOperand{L.Wp + at, nq, L.we + j, 0}, s);
+            if (st != KEVD_OK) return st;
+            if (rest == 0) continue;
+            KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
+            for (int c = 0; c < rest; c += kLmBlock) {
+                const int n = std::min(kLmBlock, rest - c);
+                KEVD_CUDA_TRY(launch_ozmm(OzOperand{o.Ap, nq, o.ae, 0},
+                                          OzOperand{o.Bp + (size_t)(c / kLmBlock) * tile, nq, o.be + c, 0}, rows, n,
+                                          kLmBlock, nullptr, o.C, o.rows, 0, nullptr, 0, o.flags, s));
+                k_lm_sub<<<dim3(grid1(rows), n), 256, 0, s>>>(R + (int64_t)(nb + c) * P, P, o.C, o.rows, rows);
+            }
+        }
+    }
+    KEVD_LAUNCH_CHECK();
     return KEVD_OK;
 }
 
@@ -433,12 +655,16 @@ extern "C" int rpchol_factor_lowmem(const double* X, int64_t N, int32_t d, doubl
     cublasHandle_t h = lm_blas(s);
     if (!h) return KEVD_ECUDA;
     const FactorWs& w = L.w;
-    const LmPanel& p = L.p;
+    LmRound q{};
+    const bool tc = lm_round(L.p, N, d, r, b, &q);
+    const LmOz& o = q.o;
+    const LmPanel& p = tc ? q.p : L.p;
     const double inv_eps = 1.0 / eps, one = 1.0, mone = -1.0;
     {
         TraceScope tr(kStOther, s);
         KEVD_CUDA_TRY(cudaMemset2DAsync(W, (size_t)ldw * sizeof(double), 0, (size_t)r * sizeof(double), r, s));
         launch_prepare_fp64(X, N, d, w, rho, s);
+        if (tc) KEVD_CUDA_TRY(cudaMemsetAsync(o.flags, 0, sizeof(int), s));
     }
     KEVD_LAUNCH_CHECK();
 
@@ -480,17 +706,29 @@ extern "C" int rpchol_factor_lowmem(const double* X, int64_t N, int32_t d, doubl
         if (k > 0)   // Z = W^-T F(T,:)^T with the leading k x k block of W
             LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_LEFT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT, k, m,
                                 &one, W, (int)ldw, L.Zt, k));
+        // Measured at N = 60,000, r = 512, b = 64: 17.6 ms of engine time, 32.7 with the library's
+        // products and solves only.
+        const int nm = (m + 15) / 16;
+        if (tc) {
+            KEVD_CUDA_TRY(oz_cut_rowmajor(p.XS, k + m, d, o.XSp, o.xse, s));
+            KEVD_CUDA_TRY(launch_linv(w, q.li, b, s));
+        }
         for (int64_t i0 = 0; i0 < N; i0 += p.P) {
             const int64_t Pc = std::min(p.P, N - i0);
-            const int st = kernel_panel(h, X, d, i0, Pc, k + m, p, pivots, inv_eps, nullptr, s);
+            const int st = kernel_panel(h, X, d, i0, Pc, k + m, p, pivots, inv_eps, nullptr, s, tc ? &o : nullptr);
             if (st != KEVD_OK) return st;
             double* R = p.Kp + (int64_t)k * p.P;
             if (k > 0)   // R = K(p,T) - K(p,S) Z
                 LM_BLAS(cublasDgemm(h, CUBLAS_OP_N, CUBLAS_OP_N, (int)Pc, m, k, &mone, p.Kp, (int)p.P, L.Zt, k, &one,
                                     R, (int)p.P));
-            // G = R L^-T: Lc is L row-major (ld b), i.e. L^T column-major
-            LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, (int)Pc,
-                                m, &one, w.Lc, b, R, (int)p.P));
+            if (tc) {   // G = R L^-T
+                KEVD_CUDA_TRY(oz_cut_rows(R, p.P, (int)Pc, m, nm, o.Ap, o.ae, o.rmax, s));
+                KEVD_CUDA_TRY(launch_ozmm(OzOperand{o.Ap, nm, o.ae, 0}, OzOperand{q.li.Lp, q.li.ldR / 16, q.li.le, 0},
+                                          Pc, m, 16 * nm, nullptr, R, p.P, 0, nullptr, 0, o.flags, s));
+            } else {    // Lc is L row-major (ld b), i.e. L^T column-major
+                LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, (int)Pc,
+                                    m, &one, w.Lc, b, R, (int)p.P));
+            }
             k_lm_rho<<<grid1(Pc), 256, 0, s>>>(w, R, p.P, Pc, m, i0, rho);
             KEVD_LAUNCH_CHECK();
         }
@@ -502,9 +740,12 @@ extern "C" int rpchol_factor_lowmem(const double* X, int64_t N, int32_t d, doubl
     }
     KEVD_LAUNCH_CHECK();
     FactorState hs;
+    int gave_up = 0;
     KEVD_CUDA_TRY(cudaMemcpyAsync(&hs, w.st, sizeof(hs), cudaMemcpyDeviceToHost, s));
+    if (tc) KEVD_CUDA_TRY(cudaMemcpyAsync(&gave_up, o.flags, sizeof(int), cudaMemcpyDeviceToHost, s));
     KEVD_CUDA_TRY(cudaStreamSynchronize(s));
     trace_flush();
+    if (gave_up) return KEVD_ETIMEOUT;
     info->rank = hs.k;
     info->rounds = hs.rounds;
     info->trace_err = hs.final_sum;
@@ -523,14 +764,17 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
     if (!(eps > 0.0) || !isfinite(eps)) return KEVD_EINVAL;
     size_t need = 0;
     LmNormWs L = carve_lm_norm(workspace, N, d, rank, true, &need);
+    const size_t need_tc = need;
     const bool tc = gram_oz_eligible(N, rank) && ws_bytes >= need;
-    if (!tc) L = carve_lm_norm(workspace, N, d, rank, false, &need);
+    if (ws_bytes < need) L = carve_lm_norm(workspace, N, d, rank, false, &need);
     if (!workspace || ws_bytes < need || !aligned(workspace)) return KEVD_EWORKSPACE;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     cublasHandle_t h = lm_blas(s);
     if (!h) return KEVD_ECUDA;
     const LmPanel& p = L.p;
     const double inv_eps = 1.0 / eps, one = 1.0, zero = 0.0;
+    // (the products follow KEVD_ENGINE, the Grams KEVD_GRAM)
+    const LmOz* po = ws_bytes >= need_tc && L.o.rows > 0 && oz_engine_enabled() ? &L.o : nullptr;
     const bool one_panel = N <= p.P;   // the panel is formed once and kept for all three passes
     int st;
 
@@ -541,11 +785,14 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
         k_lm_gather<<<grid1((int64_t)rank * d), 256, 0, s>>>(X, N, d, pivots, rank, p.xn, p.XS, p.xnS, L.flags);
         k_lm_fill<<<grid1(p.P), 256, 0, s>>>(L.ones, p.P, 1.0);
         KEVD_LAUNCH_CHECK();
+        if (po) {
+            KEVD_CUDA_TRY(oz_cut_rowmajor(p.XS, rank, d, po->XSp, po->xse, s));
+        }
         // pass 1: K(S,:) 1, then y = W^-T W^-1 K(S,:) 1
         KEVD_CUDA_TRY(cudaMemsetAsync(L.vec, 0, (size_t)rank * sizeof(double), s));
         for (int64_t i0 = 0; i0 < N; i0 += p.P) {
             const int64_t Pc = std::min(p.P, N - i0);
-            if ((st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s)) != KEVD_OK) return st;
+            if ((st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s, po)) != KEVD_OK) return st;
             LM_BLAS(cublasDgemv(h, CUBLAS_OP_T, (int)Pc, rank, &one, p.Kp, (int)p.P, L.ones, 1, &one, L.vec, 1));
         }
         KEVD_CUDA_TRY(cudaMemcpyAsync(L.y, L.vec, (size_t)rank * sizeof(double), cudaMemcpyDeviceToDevice, s));
@@ -555,7 +802,7 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
         for (int64_t i0 = 0; i0 < N; i0 += p.P) {
             const int64_t Pc = std::min(p.P, N - i0);
             if (!one_panel &&
-                (st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s)) != KEVD_OK)
+                (st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s, po)) != KEVD_OK)
                 return st;
             LM_BLAS(cublasDgemv(h, CUBLAS_OP_N, (int)Pc, rank, &one, p.Kp, (int)p.P, L.y, 1, &zero, dtil + i0, 1));
             k_lm_recip<<<grid1(Pc), 256, 0, s>>>(dtil + i0, Pc, L.pv, L.flags);
@@ -571,13 +818,18 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
         for (int64_t i0 = 0; i0 < N; i0 += p.P) {
             const int64_t Pc = std::min(p.P, N - i0);
             if (!one_panel &&
-                (st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s)) != KEVD_OK)
+                (st = kernel_panel(h, X, d, i0, Pc, rank, p, pivots, inv_eps, nullptr, s, po)) != KEVD_OK)
                 return st;
             LM_BLAS(cublasDgemv(h, CUBLAS_OP_N, (int)Pc, rank, &one, p.Kp, (int)p.P, L.y, 1, &zero, qtil + i0, 1));
             k_lm_weights<<<grid1(Pc), 256, 0, s>>>(dtil + i0, qtil + i0, Pc, tc, L.wa, L.wc, L.flags);
             KEVD_LAUNCH_CHECK();
-            LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT, (int)Pc,
-                                rank, &one, W, (int)ldw, p.Kp, (int)p.P));
+            if (po) {
+                if (i0 == 0 && (st = solve_setup(h, W, ldw, rank, L, s)) != KEVD_OK) return st;
+                if ((st = solve_panel(W, ldw, rank, Pc, L, s)) != KEVD_OK) return st;
+            } else {
+                LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_LOWER, CUBLAS_OP_T, CUBLAS_DIAG_NON_UNIT,
+                                    (int)Pc, rank, &one, W, (int)ldw, p.Kp, (int)p.P));
+            }
             if (tc)
                 KEVD_CUDA_TRY(launch_gram_oz_panel(p.Kp, p.P, p.P, Pc, rank, L.wa, L.wc, L.sa_hi, L.sc_hi, L.cmax,
                                                    L.ecol, L.gpart, L.planes, L.flags + 1, A, C, i0 > 0, kLmSMs, s));
@@ -585,14 +837,14 @@ extern "C" int bistoch_normalize_lowmem(const double* X, int64_t N, int32_t d, d
                 KEVD_CUDA_TRY(kevd_gram_weighted(p.Kp, p.P, Pc, rank, L.wa, L.wc, L.gpart, A, C, i0 > 0, s));
         }
     }
-    int flags[2] = {0, 0};
+    int flags[3] = {0, 0, 0};
     KEVD_CUDA_TRY(cudaMemcpyAsync(flags, L.flags, sizeof(flags), cudaMemcpyDeviceToHost, s));
     KEVD_CUDA_TRY(cudaStreamSynchronize(s));
     trace_flush();
     if (flags[0] & 4) return KEVD_EINVAL;
     if (flags[0] & 1) return KEVD_ED_NONPOS;
     if (flags[0] & 2) return KEVD_EQ_NONPOS;
-    if (flags[1]) return KEVD_ETIMEOUT;
+    if (flags[1] | flags[2]) return KEVD_ETIMEOUT;
     return KEVD_OK;
 }
 

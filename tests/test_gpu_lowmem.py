@@ -172,6 +172,38 @@ def test_panel_grams_tensor_core_and_fp64_pipe(kevd, monkeypatch, N, r, panel):
         assert torch.max(torch.abs(got[i] - ref[i])) <= (N + 32) * 2.0 ** -52 * torch.max(torch.abs(ref[i]))
 
 
+# The panel's products and solves on the tensor cores against the library's FP64 ones
+# (KEVD_ENGINE=fp64): blocks of 32 and 128 with a ragged last panel, ranks that end at, one past and well
+# past a 128-column block of the solve, and W scaled by 1000 (F by 1 / 1000, so A and C as it was, d~
+# and q~ too since both sides scale alike).  Bars as test_normalize_and_eig_match_oracle.
+@pytest.mark.parametrize("N,r,b,panel", [(300, 32, 32, "64"), (3001, 128, 128, "192"), (3001, 160, 32, None),
+                                         (5000, 300, 100, "256")])
+def test_products_tensor_core_and_library(kevd, monkeypatch, N, r, b, panel):
+    if panel:
+        monkeypatch.setenv("KEVD_LOWMEM_PANEL", panel)
+    X, eps, _ = make_config("ks200k", N=N)
+    Xg = _gpu(X)
+
+    def passes():
+        o = kevd.rpchol_factor_lowmem(Xg, eps, r, b=b, seed=3)
+        n = [kevd.bistoch_normalize_lowmem(Xg, eps, o["pivots"], s * o["W"], o["rank"]) for s in (1.0, 1000.0)]
+        return o, n
+
+    out, norm = passes()
+    monkeypatch.setenv("KEVD_ENGINE", "fp64")
+    ref, norm0 = passes()
+    rk = ref["rank"]
+    assert out["rank"] == rk and torch.equal(out["pivots"][:rk], ref["pivots"][:rk])
+    assert torch.max(torch.abs(out["W"] - ref["W"])) < 1e-10
+    assert torch.max(torch.abs(out["rho"] - ref["rho"])) < 1e-10
+    for got, want in zip(norm, norm0):
+        for i in range(2):
+            assert torch.max(torch.abs(got[i] - want[i]) / want[i]) < 1e-12
+        for i in range(2, 4):
+            assert torch.equal(got[i], got[i].T)
+            assert torch.max(torch.abs(got[i] - want[i])) < 1e-10 * torch.max(torch.abs(want[i]))
+
+
 def test_out_of_range_pivot_is_an_error(kevd):
     X, eps, _ = make_config("ks200k", N=1000)
     Xg = _gpu(X)
