@@ -134,12 +134,6 @@ __device__ __forceinline__ uint32_t oz_word(long long T0, long long T1, int s) {
     return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
 }
 
-// Digit planes of two values x0, x1 on a row with exponent E (max |row| < 2^E,
-// E = -900 for a zero row).
-__device__ __forceinline__ void digits2_e(double x0, double x1, int E, uint32_t (&w)[kDigits]) {
-    digits2(x0, x1, E > -900 ? 1021 + E : 4096, w);
-}
-
 // Layout of the planes of an R x 16 nq operand of k_ozmm: tiles of 128 rows x 16
 // columns (32 bytes per row, the 16-byte halves exchanged in rows 4-7 of every eight:
 // the 32-byte-swizzled K-major MMA operand), the D planes of a tile one after the

@@ -45,28 +45,20 @@ static __device__ __forceinline__ bool elect_one() {
     return p != 0;
 }
 
-// umma_bf16 with a use of A's collector buffer: 0 none, 1 fill, 2 use, 3 last use.
-template <int COL>
+// umma_bf16 that fills (FILL) or uses A's collector buffer.
+template <bool FILL>
 static __device__ __forceinline__ void umma_bf16_col(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                                      uint32_t accumulate) {
-    if constexpr (COL == 0) {
-        umma_bf16(dtmem, adesc, bdesc, idesc, accumulate);
-    } else if constexpr (COL == 1) {
+    if constexpr (FILL) {
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
             "tcgen05.mma.cta_group::1.kind::f16.collector::a::fill [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
             "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
-    } else if constexpr (COL == 2) {
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
-            "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-            : "memory");
     } else {
         asm volatile(
             "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-            "tcgen05.mma.cta_group::1.kind::f16.collector::a::lastuse [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+            "tcgen05.mma.cta_group::1.kind::f16.collector::a::use [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
             "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
             : "memory");
     }
@@ -137,8 +129,8 @@ struct OzIssuer {
                 if (!oz_pair<D>(s, t) || (STRICT && s + t > 4)) continue;
                 const uint32_t d = tmem + (uint32_t)(N * oz_acc_of<D>(s + t, s));
                 const uint64_t pda = da + (uint64_t)(s * pa), pdb = db + (uint64_t)(t * pb);
-                if (t == 0) umma_bf16_col<1>(d, pda, pdb, idesc, 1u);
-                else umma_bf16_col<2>(d, pda, pdb, idesc, 1u);
+                if (t == 0) umma_bf16_col<true>(d, pda, pdb, idesc, 1u);
+                else umma_bf16_col<false>(d, pda, pdb, idesc, 1u);
             }
         }
         if constexpr (STRICT && D > 5) {
