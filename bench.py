@@ -248,16 +248,9 @@ GRAM_TRAFFIC = {
     "k_gram": (436.7e6 + 70.7e6, 60000, 803),      # FP64, ks200k points truncated to N = 60,000
     "k_gram32": (8.661e9 + 0.159e9, 300000, 1848),  # FP32 FFMA, vsa2m points truncated to N = 300,000
 }
-# k_gram_oz (FP64 F, tensor cores): one slab launch of 93,184 rows at rank 1,830 (vsa2m points
-# truncated to N = 300,000); the slabs of a step cover N rows and the tiles grow as rank^2, so the
-# step's traffic scales by N rank^2 (the 6-digit planes written by k_oz_planes not included)
-GRAM_OZ_TRAFFIC = (11.484e9 + 0.027e9, 93184, 1830)
 
 
 def gram_traffic(kernel, N, rank):
-    if kernel == "k_gram_oz":
-        b, n0, r0 = GRAM_OZ_TRAFFIC
-        return b * float(N) * rank * rank / (float(n0) * r0 * r0)
     if kernel not in GRAM_TRAFFIC:
         return None
     b, n0, r0 = GRAM_TRAFFIC[kernel]
@@ -268,10 +261,10 @@ def gram_kernel_name(path, N):
     """The Gram kernel the library runs for this bench's F (contiguous, ld = N)."""
     forced = os.environ.get("KEVD_GRAM", "").startswith("f")
     if path != "bf16x3":
-        return "k_gram" if forced or N % 2 != 0 or N >= (1 << 31) else "k_gram_oz"
+        return "k_gram" if forced or N >= (1 << 31) else "k_gram_oz"
     if forced or N % 4 != 0 or N >= (1 << 31):
         return "k_gram32"
-    return "k_gram_tc"
+    return "k_gram_pl"
 
 
 def stage_table(path, stages, out, cfg, steps, k):
@@ -286,9 +279,9 @@ def stage_table(path, stages, out, cfg, steps, k):
               precision: bytes 4 N (sum_k + d engine_rounds + rank) + 16 N engine_rounds
               (F(:, :k) and X read once per round, new columns written, rho read + written)
       gram    2 N rank (rank + 1) flops (both Grams, unique entries); the tensor-core
-              forms execute 4 BF16 slice products per FP32 product (FP32 F) or 21 BF16
+              forms execute 4 BF16 slice products per FP32 product (FP32 F) or 22 BF16
               digit products per FP64 product (FP64 F, six digits), so their tensor
-              work is 4 x or 21 x that, against the BF16 tensor peak; the FP64 engine
+              work is 4 x or 22 x that, against the BF16 tensor peak; the FP64 engine
               products and lift execute 28 (seven digits)
       lift    2 N rank k flops
       degree  4 passes over F: 4 e N rank bytes
@@ -320,8 +313,8 @@ def stage_table(path, stages, out, cfg, steps, k):
         gk = gram_kernel_name(path, N)
         gflops = 2.0 * N * rank * (rank + 1)
         if gk == "k_gram_oz":
-            # 21 BF16 digit products per FP64 product (pairs of the six digits with s + t <= 5)
-            tab["k_gram_oz (with k_oz_planes)"] = dict(ms=ms["gram"], work=21.0 * gflops, unit="GFLOP/s",
+            # 22 BF16 digit products per FP64 product (pairs of the six digits with s + t <= 5, and (3, 3))
+            tab["k_gram_oz (with k_oz_planes)"] = dict(ms=ms["gram"], work=22.0 * gflops, unit="GFLOP/s",
                                                        peak=pk["bf16"], bound="tensor",
                                                        algorithmic_fp64_gflop=gflops / 1e9)
         else:
@@ -334,11 +327,11 @@ def stage_table(path, stages, out, cfg, steps, k):
                                           peak=pk["bf16"], bound="tensor", algorithmic_fp64_gflop=2.0 * N * rank * k / 1e9)
     else:
         eng_bytes = 4.0 * N * (out["sum_k"] + d * out["engine_rounds"] + rank) + 16.0 * N * out["engine_rounds"]
-        tab["k_engine_tc"] = dict(ms=ms["engine"], work=eng_bytes, unit="GB/s", peak=pk["hbm"], bound="hbm")
+        tab["k_engine_pl (with k_append)"] = dict(ms=ms["engine"], work=eng_bytes, unit="GB/s", peak=pk["hbm"], bound="hbm")
         gk = gram_kernel_name(path, N)
         gflops = 2.0 * N * rank * (rank + 1)
-        if gk == "k_gram_tc":
-            tab[gk] = dict(ms=ms["gram"], work=4.0 * gflops, unit="GFLOP/s", peak=pk["bf16"], bound="tensor",
+        if gk == "k_gram_pl":
+            tab["k_gram_pl (with k_gt_cut)"] = dict(ms=ms["gram"], work=4.0 * gflops, unit="GFLOP/s", peak=pk["bf16"], bound="tensor",
                            algorithmic_fp32_gflop=gflops / 1e9)
         else:
             tab[gk] = dict(ms=ms["gram"], work=gflops, unit="GFLOP/s", peak=FP32_FFMA_GFLOPS, bound="alu")
@@ -371,16 +364,19 @@ def roofline(path, stages, out, cfg, steps, k=None):
         # F_p = K(p,S) W^-T (r^2), Grams (2 r (r+1)).
         eng_fl = N * (2.0 * d * (out["sum_k"] + rank) + float(rank) ** 2)
         p3_fl = N * (2.0 * d * rank + float(rank) ** 2 + 2.0 * rank * (rank + 1))
-        cand = {"factor panel loop (cuBLAS DGEMM/DTRSM + k_lm_kexp + k_lm_rho)": (eng_ms, eng_fl),
-                "normalisation pass 3 (DGEMM + k_lm_kexp + DTRSM + k_gram)": (gram_ms, p3_fl)}
+        cand = {"factor panel loop (cuBLAS DGEMM for K(p,S) Z, k_ozmm, k_lm_kexp, k_lm_rho)": (eng_ms, eng_fl),
+                "normalisation pass 3 (k_ozmm, k_lm_kexp, k_gram_oz)": (gram_ms, p3_fl)}
         dom = max(cand, key=lambda n: cand[n][0])
         ms, fl = cand[dom]
         ach = fl / (ms / 1e3) / 1e9
-        return {"kernel": dom, "bound": "alu", "achieved": ach, "peak": FP64_PEAK_GFLOPS, "unit": "GFLOP/s",
-                "frac": ach / FP64_PEAK_GFLOPS, "traffic": None, "ms_per_step": ms,
-                "peak_source": "nominal FP64 rate of the recipe table (1.25 TFLOP/s); cuBLAS DGEMM measured 1.04",
-                "stages": {n: {"ms": v[0], "gflop": v[1] / 1e9, "frac": v[1] / (v[0] / 1e3) / 1e9 / FP64_PEAK_GFLOPS}
-                           for n, v in cand.items()},
+        # FP64-accurate products cost 28 BF16 digit products on the tensor cores; the
+        # panel loop's K(p,S) Z runs on the FP64 pipe
+        peak = pk["bf16"] / 28.0 if dom.startswith("norm") else FP64_PEAK_GFLOPS
+        return {"kernel": dom, "bound": "tensor" if dom.startswith("norm") else "alu", "achieved": ach, "peak": peak,
+                "unit": "GFLOP/s", "frac": ach / peak, "traffic": None, "ms_per_step": ms,
+                "peak_source": "BF16 tensor peak / 28 digit products" if dom.startswith("norm") else
+                "nominal FP64 rate of the recipe table (1.25 TFLOP/s); cuBLAS DGEMM measured 1.04",
+                "stages": {n: {"ms": v[0], "gflop": v[1] / 1e9} for n, v in cand.items()},
                 "sum_k": out["sum_k"], "sum_m_sq": out["sum_m_sq"]}
     tab = stage_table(path, stages, out, cfg, steps, k)
     own = {n: v for n, v in tab.items() if "achieved" in v}
@@ -403,7 +399,7 @@ def roofline(path, stages, out, cfg, steps, k=None):
            "stages": {n: {kk: vv for kk, vv in t.items() if kk in ("ms", "achieved", "frac", "unit", "bound",
                                                                    "algorithmic_fp32_gflop", "algorithmic_fp64_gflop")}
                       for n, t in tab.items()}}
-    if name == "k_engine_tc":
+    if name == "k_engine_pl":
         res["algorithmic_bytes_per_step"] = v["work"]
     return res
 
@@ -426,7 +422,7 @@ def step_launches(path, mode, out, N, r, b):
     for the tensor-core Gram) + split reduction; eigen stage ~ 9."""
     rounds = out["rounds"]
     factor = 1 + 5 * rounds + 2 + (2 * out["engine_rounds"] if path == "bf16x3" else 0)
-    normalize = 7 + 1 + 1 + 1 + (2 if gram_kernel_name(path, N) in ("k_gram_tc", "k_gram_oz") else 0)
+    normalize = 7 + 1 + 1 + 1 + (2 if gram_kernel_name(path, N) in ("k_gram_pl", "k_gram_oz") else 0)
     return factor + normalize + 9
 
 
