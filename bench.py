@@ -319,11 +319,11 @@ def stage_table(path, stages, out, cfg, steps, k):
                                                        algorithmic_fp64_gflop=gflops / 1e9)
         else:
             tab[gk] = dict(ms=ms["gram"], work=gflops, unit="GFLOP/s", peak=FP64_PEAK_GFLOPS, bound="alu")
-        if os.environ.get("KEVD_LIFT", "").startswith("f") or N % 2 != 0:
+        if os.environ.get("KEVD_LIFT", "").startswith("f"):
             tab["k_dgemm (lift)"] = dict(ms=ms["lift"], work=2.0 * N * rank * k, unit="GFLOP/s",
                                          peak=FP64_PEAK_GFLOPS, bound="alu")
         else:
-            tab["k_ozgemm (lift)"] = dict(ms=ms["lift"], work=28.0 * 2.0 * N * rank * k, unit="GFLOP/s",
+            tab["k_ozmm (lift)"] = dict(ms=ms["lift"], work=28.0 * 2.0 * N * rank * k, unit="GFLOP/s",
                                           peak=pk["bf16"], bound="tensor", algorithmic_fp64_gflop=2.0 * N * rank * k / 1e9)
     else:
         eng_bytes = 4.0 * N * (out["sum_k"] + d * out["engine_rounds"] + rank) + 16.0 * N * out["engine_rounds"]
@@ -335,8 +335,12 @@ def stage_table(path, stages, out, cfg, steps, k):
                            algorithmic_fp32_gflop=gflops / 1e9)
         else:
             tab[gk] = dict(ms=ms["gram"], work=gflops, unit="GFLOP/s", peak=FP32_FFMA_GFLOPS, bound="alu")
-        tab["k_lift32"] = dict(ms=ms["lift"], work=2.0 * N * rank * k, unit="GFLOP/s", peak=FP32_FFMA_GFLOPS,
-                               bound="alu")
+        if os.environ.get("KEVD_LIFT", "").startswith("f"):
+            tab["k_lift32"] = dict(ms=ms["lift"], work=2.0 * N * rank * k, unit="GFLOP/s", peak=FP32_FFMA_GFLOPS,
+                                   bound="alu")
+        else:   # three digits: six BF16 digit products per FP32 product
+            tab["k_ozmm<3> (lift)"] = dict(ms=ms["lift"], work=6.0 * 2.0 * N * rank * k, unit="GFLOP/s",
+                                           peak=pk["bf16"], bound="tensor", algorithmic_fp32_gflop=2.0 * N * rank * k / 1e9)
     tab["degree (k_colsum, k_rowdot)"] = dict(ms=ms["degree"], work=4.0 * e * N * rank, unit="GB/s", peak=pk["hbm"],
                                               bound="hbm")
     for name, v in tab.items():
