@@ -1099,13 +1099,13 @@ static size_t engine_smem() {
 // Greedy rounds of an FP64 factor in one cooperative launch, for N <= 65,536.
 //
 // A greedy round is a step of r dependent ones, and in launches of its own (proposal,
-// gather, H, acceptance, engine) it is mostly their latency: 48 us at N = 2,048, d = 64.
+// gather, H, acceptance, engine) it is mostly their latency: 48 us at N = 2,000, d = 64.
 // Here a CTA owns a 64-row tile for all rounds, a thread a row (its residual in a register),
 // a third warp takes H and its root meanwhile, and a round has one grid barrier, after which
 // every CTA finds the argmax of the tiles' (max, index) pairs by itself.  What bounds it is
 // the chain of d + k dependent FP64 operations of 64 cycles that a row's value is defined by:
 // same operations in the same order as the kernels above, so the same bits: 15 us a round at
-// N = 2,048, k up to 128.  The line at 1,024 tiles: up to there a pair of tile statistics per thread and
+// N = 2,000, k up to 128.  The line at 1,024 tiles: up to there a pair of tile statistics per thread and
 // 16 loads find the argmax, and all CTAs are resident (7 of 64 + 32 threads per SM); above,
 // a round's work on the FP64 pipe outweighs the launches.  Pairs alternate between two
 // buffers, since a CTA may be one round ahead of another's reading.
