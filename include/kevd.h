@@ -367,11 +367,9 @@ int eig_topk_lowmem(const double* X, int64_t N, int32_t d, double eps, const int
 
 /*
  * kevd_kernel_exp -- the table-driven exponential behind the Gaussian kernel values
- * exp(-|x_i - x_s|^2 / eps) of Algorithm 2 in the FP64 engine on the tensor cores (which
- * evaluates the same table and series in fixed point throughout): out[i]
- * = exp(t[i]) for t[i] <= 0 within one ulp, 0 for t[i] <= -708 (a
- * table-driven method with its polynomial in fixed point, so that it runs on
- * the integer pipe).  t, out: device double[n] (out may alias t).  Enqueued on
+ * exp(-|x_i - x_s|^2 / eps) of Algorithm 2 in the FP64 engine on the tensor cores: out[i]
+ * = exp(t[i]) for t[i] <= 0 within one ulp, 0 for t[i] <= -708 (integer arithmetic
+ * throughout).  t, out: device double[n] (out may alias t).  Enqueued on
  * `stream`; the first call on a device uploads an 8 KiB table and waits for it.
  * Returns KEVD_EINVAL for NULL pointers or n < 0.
  */

@@ -913,12 +913,13 @@ __global__ void __launch_bounds__(128) k_linv_planes(FactorWs w, OzWs o, int b) 
 // values exp(-(|x_i|^2 + |x_s|^2 - 2 x_i.x_s) / eps) (1 at the pivot itself)
 // minus Df, as digit planes with one exponent per row (the row maximum over
 // the round's pivots).  Block: 32 rows x ldR / 16 warps, warp g taking the quarter of
-// 16 pivots [16 g, 16 g + 16).  Only the squared distance is formed in FP64 (two
-// operations, 17 cycles per warp and SM each); the scaling by 1 / eps, the exponential
-// (kexp_q62), the difference and the digits are 64-bit fixed point.  Bound: the integer
-// pipe (HBM: 30 bytes per value, 0.5 ms).  N = 1M, b = 128: 2.8 ms per round with nine FP64
-// operations per value, 1.6 ms now.
-__global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, double inv_eps,
+// 16 pivots [16 g, 16 g + 16).  The squared distance (two operations) and the difference
+// are FP64, 17 cycles per warp and SM each; the scaling by 1 / eps, the exponential
+// (kexp_bits) and the digits run on the integer pipe.  R has to be a double here: on a common
+// grid of 2^-62 a row far from every pivot loses its digits, and beyond exp(-43) all of them.
+// Bound: the integer pipe (HBM: 30 bytes per value, 0.5 ms).  N = 1M, b = 128: 2.8 ms per
+// round with nine FP64 operations per value, 1.5 ms now.
+__global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, KexpScale inv_eps,
                                                const unsigned long long* __restrict__ tblg) {
     const FactorState* st = w.st;
     if (st->done || st->m == 0) return;
@@ -940,8 +941,8 @@ __global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, do
         const int64_t row = row0 + lane;
         const bool on = row < N;
         const double xi = on ? w.xn[row] : 0.0;
-        long long R[16];                                       // units of 2^-62
-        unsigned long long mx = 0;
+        long long R[16];                                       // bits of doubles, then their digits
+        unsigned long long mx = 0;                             // max |R|
         // four values at a time, the next four in flight; rolled, R moving down
         double dx[4], df[4];
         auto load = [&](int u) {
@@ -970,10 +971,11 @@ __global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, do
                 const int l = l0 + 4 * u + e;
                 long long v = 0;
                 if (on && l < m) {
-                    const long long kv = s_row[l] == row ? 1ll << 62
-                                                         : kexp_q62(fma(-2.0, cx[e], xi + s_xn[l]), inv_eps, tbl);
-                    v = kv - q62_of(cf[e]);
-                    mx = max(mx, (unsigned long long)(v < 0 ? -v : v));
+                    const double kv = s_row[l] == row ? 1.0
+                                                      : __longlong_as_double((long long)kexp_bits(
+                                                            fma(-2.0, cx[e], xi + s_xn[l]), inv_eps, tbl));
+                    v = __double_as_longlong(kv - cf[e]);
+                    mx = max(mx, (unsigned long long)v & 0x7FFFFFFFFFFFFFFFull);
                 }
                 R[12 + e] = v;
             }
@@ -983,17 +985,10 @@ __global__ void __launch_bounds__(256) k_rprep(FactorWs w, OzWs o, int64_t N, do
         for (int q = 0; q < nq; ++q) mx = max(mx, red[q][lane]);
         __syncthreads();                                       // red is rewritten for the next rows
         if (!on) continue;
-        // max |R| < 2^E, E = bits - 62; T = round(R 2^(54 - E)) of the digits (|T| < 2^54)
-        const int bits = 64 - __clzll((long long)mx);
-        if (g == 0) o.re[row] = mx ? bits - 62 : -900;
-        const int rs = bits - 54;
+        const int E = exp_of(__longlong_as_double((long long)mx));
+        if (g == 0) o.re[row] = E;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) {
-            unsigned long long a = (unsigned long long)(R[e] < 0 ? -R[e] : R[e]);
-            a = rs <= 0 ? a << min(-rs, 63) : ((a >> (rs - 1)) + 1) >> 1;
-            a = min(a, 0x3FFFFFFFFFFFFFull);
-            R[e] = R[e] < 0 ? -(long long)a : (long long)a;
-        }
+        for (int e = 0; e < 16; ++e) R[e] = oz_T_f64<kDigits>(__longlong_as_double(R[e]), E);
         oz_store_quarter<kDigits>(o.Rp, row, g, nq, R);
     }
 }
@@ -1517,8 +1512,8 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
                 }
                 TraceScope tr(kStEngine, s);
                 // R = K(:, T) - F F(T,:)^T; G = R L^-T into F(:, k:k+m), on the tensor cores; rho
-                k_rprep<<<(unsigned)std::min<int64_t>((N + 31) / 32, 152 * 8), 2 * ow.ldR, 0, s>>>(w, ow, N, inv_eps,
-                                                                                                   exp_tbl);
+                k_rprep<<<(unsigned)std::min<int64_t>((N + 31) / 32, 152 * 8), 2 * ow.ldR, 0, s>>>(
+                    w, ow, N, kexp_scale(inv_eps), exp_tbl);
                 KEVD_CUDA_TRY(launch_linv(w, ow, b, s));
                 KEVD_CUDA_TRY(launch_ozmm(oR, oL, N, b, -2, w.st, Fd, ldf, ldf, ow.Fp, ow.ldF / 16, ow.flags, s));
                 k_rho_update<<<(unsigned)((N + 63) / 64), 256, 0, s>>>(w, Fd, ldf, rho, N);

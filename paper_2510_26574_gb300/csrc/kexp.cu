@@ -30,10 +30,13 @@ cudaError_t kexp_table(cudaStream_t s, const unsigned long long** tbl) {
     return e;
 }
 
-__global__ void k_kexp(const double* __restrict__ t, int64_t n, const unsigned long long* __restrict__ tbl,
+// (t > 0 lies outside the engine's use: CUDA's exp; NaN gives 0.)
+__global__ void k_kexp(const double* __restrict__ t, int64_t n, KexpScale one, const unsigned long long* __restrict__ tbl,
                        double* __restrict__ out) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = kexp(t[i], tbl);
+    if (i >= n) return;
+    const double x = t[i];
+    out[i] = x > 0.0 ? exp(x) : x <= 0.0 ? __longlong_as_double((long long)kexp_bits(-x, one, tbl)) : 0.0;
 }
 
 }  // namespace kevd
@@ -46,6 +49,6 @@ extern "C" int kevd_kernel_exp(const double* t, int64_t n, double* out, void* st
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     const unsigned long long* tbl = nullptr;
     if (kexp_table(s, &tbl) != cudaSuccess) return KEVD_ECUDA;
-    k_kexp<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, n, tbl, out);
+    k_kexp<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(t, n, kexp_scale(1.0), tbl, out);
     return cudaGetLastError() == cudaSuccess ? KEVD_OK : KEVD_ECUDA;
 }

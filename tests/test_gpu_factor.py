@@ -269,3 +269,46 @@ def test_greedy_rounds_in_one_launch(kevd, N, d, r):
     assert torch.equal(a["proposals"][:a["rounds"]], b["proposals"][:a["rounds"]])
     assert torch.equal(a["F"][:, :N], b["F"][:, :N])
     assert torch.equal(a["rho"][:N], b["rho"][:N])
+
+
+# Rows far from every pivot: 3,000 points in a box 17 wide with eps = 1, so that most rows lie
+# at t = |x_i - x_s|^2 / eps from 2 to 30 of the nearest of the first round's pivots, and five
+# planted ones outside it, up to t = 500.  A row of F that small keeps its digits (it is
+# divided by its own size in the normalisation): against the FP64-pipe engine the first round's
+# columns agree relative to the row.  Bar: both engines form |x_i|^2 + |x_s|^2 - 2 x_i.x_s with at
+# most d + 4 roundings of (2 max |x|)^2, which is the relative error of K; t's own product and the
+# solve add t and 4 b roundings; the solve amplifies by cond(L).  Later columns (r = 4 b) subtract F's
+# earlier ones, which both engines hold to 2^-53 of 1: 1e-10 as in test_arpc_matches_oracle.
+@pytest.mark.parametrize("r", [32, 128])
+def test_rows_far_from_every_pivot(kevd, monkeypatch, r):
+    b, d, u = 32, 3, 2.0 ** -53
+    rng = np.random.Generator(np.random.PCG64(12))
+    X = 17.0 * (rng.random((3000, d)) - 0.5)
+    far = np.array([10.0, 30.0, 45.0, 200.0, 400.0])
+    X[:5] = 0.0
+    X[:5, 0] = 8.5 + np.sqrt(far) * [1, 1, 1, -1, -1]
+    X[3:5, 0] -= 17.0
+    Xg = _gpu(X)
+    a = kevd.rpchol_factor(Xg, 1.0, r, mode="arpc", b=b, seed=4)
+    monkeypatch.setenv("KEVD_ENGINE", "fp64")
+    c = kevd.rpchol_factor(Xg, 1.0, r, mode="arpc", b=b, seed=4)
+    monkeypatch.delenv("KEVD_ENGINE")
+    rk = a["rank"]
+    S = a["pivots"].cpu().numpy()[:rk]
+    assert rk == c["rank"] and S.tolist() == c["pivots"].cpu().numpy()[:rk].tolist()
+    assert S[:b].min() >= 5                                  # no planted row is a pivot of the first round
+    Fa, Fc = (o["F"].cpu().numpy().T[:, :rk] for o in (a, c))
+    m = len(arpc(X, 1.0, b, b, 4)["pivots"])                 # columns of the first round
+    L = Fc[S[:m], :m]
+    t = ((X[:, None] - X[None, S[:m]]) ** 2).sum(2).min(1)
+    assert (t > 43.7).sum() > 20
+    cond = np.linalg.cond(L)
+    bar = (2 * (d + 4) * u * 4 * (X ** 2).sum(1).max() + 2 * u * t + 4 * b * u) * cond
+    size = np.abs(Fc[:, :m]).max(1)
+    assert size.min() > 0
+    assert np.all(np.abs(Fa[:, :m] - Fc[:, :m]).max(1) <= bar * size)
+    assert np.max(np.abs(Fa - Fc)) < 1e-10
+    if r == b:
+        (da, qa, _, _), (dc, qc, _, _) = (kevd.bistoch_normalize(o["F"], rk) for o in (a, c))
+        s = np.abs(Fc.sum(0))
+        assert np.all(np.abs((da - dc).cpu().numpy()) <= 4 * bar * np.abs(Fc).max(1) * s.sum())
