@@ -570,12 +570,14 @@ __global__ void __launch_bounds__(kGpThreads, 1)
 
 // Row splits per slab for k_gram_pl (0: one split's slices exceed the budget, or F is so large
 // that the card may not hold the slices beside it): the count with the fewest waves of one
-// CTA per SM over all slabs.
+// CTA per SM over all slabs.  A slab has at most kGpStages stages, the y extent of k_gt_cut's
+// grid (4.19 million rows; the budget alone would allow 8.4 million at rank <= 128).
+constexpr int64_t kGpStages = 65535;
 static int gp_slab_splits(int64_t N, int rank, int ngram, int64_t per, int ns, int ntri, int nsm) {
     const int nb = (rank + 127) / 128;
     const size_t one = (size_t)((per + 63) / 64) * nb * (ngram == 2 ? 6 : 4) * kGpTile;
     if ((size_t)N * rank * 4 > ((size_t)128 << 30)) return 0;
-    const int most = (int)std::min<size_t>(ns, kGpBudget / one);
+    const int most = (int)std::min<int64_t>(std::min<int64_t>(ns, kGpBudget / one), kGpStages / ((per + 63) / 64));
     int best = 0;
     int64_t best_waves = INT64_MAX;
     for (int q = 1; q <= most; ++q) {

@@ -199,3 +199,14 @@ def test_fp64_factor_workspace_holds_tensor_core_products(L, monkeypatch):
     monkeypatch.delenv("KEVD_ENGINE")
     assert K.workspace_bytes(K.KEVD_WS_FACTOR, N, d, r, 1, p) == prec     # the precision form has none
     assert K.workspace_bytes(K.KEVD_WS_FACTOR, N, d, r, 1, g) == greedy   # nor greedy (b = 1)
+
+
+@pytest.mark.parametrize("rank", [1, 64, 128, 129, 256, 384])
+@pytest.mark.parametrize("N", [4_194_240, 4_194_304, 8_000_000, 20_000_000, 2**31 - 1])
+def test_fp32_gram_slab_within_grid(L, N, rank):
+    """The slices of one slab of an FP32 factor's Grams: at most 65,535 stages of 64 rows (the
+    extent of a grid in y), of 6 tiles of 16 KB per 128 columns.  The rest of the workspace is 24
+    bytes a row and the partial sums (below 300 MB for three column blocks)."""
+    n = K.workspace_bytes(K.KEVD_WS_NORMALIZE, N, 1, rank, 1, K.make_opts(precision=K.KEVD_PREC_BF16X3))
+    nb = (rank + 127) // 128
+    assert 0 < n - 24 * N < 65535 * nb * 6 * 16384 + 300_000_000

@@ -425,3 +425,22 @@ def test_fp32_grams_from_slices_same_bits(kevd, N, rank):
     assert K.lib().symmetric_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, K._ptr(d), K._ptr(A), K._ptr(ws), small,
                                        K._stream(F.device)) == K.KEVD_OK
     assert torch.equal(sym[0], d) and torch.equal(sym[1], A)
+
+
+# One slab of slices is bounded by the grid that cuts it (65,535 stages of 64 rows): N just past
+# that many rows takes two slabs, and the kernel without slices (a workspace that lacks their
+# last bytes) gives the same bits.
+def test_fp32_grams_more_rows_than_a_grid(kevd):
+    from paper_2510_26574_gb300 import kevd as K
+    N, rank = 65535 * 64 + 68, 8
+    g = torch.Generator(device="cuda").manual_seed(6)
+    F = torch.rand(rank, N, generator=g, device="cuda")
+    ref = kevd.bistoch_normalize(F, rank)
+    sym = kevd.symmetric_normalize(F, rank)
+    full = K.workspace_bytes(K.KEVD_WS_NORMALIZE, N, 1, rank, 1, K.make_opts(precision="bf16x3"))
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    out, d, A = [torch.empty_like(t) for t in ref], torch.empty_like(sym[0]), torch.empty_like(sym[1])
+    tail = [K._ptr(ws), full - 256, K._stream(F.device)]
+    assert K.lib().bistoch_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, *map(K._ptr, out), *tail) == K.KEVD_OK
+    assert K.lib().symmetric_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, K._ptr(d), K._ptr(A), *tail) == K.KEVD_OK
+    assert all(torch.equal(a, b) for a, b in zip(ref + sym, out + [d, A]))
