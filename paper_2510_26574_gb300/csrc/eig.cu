@@ -170,12 +170,14 @@ struct EigWs {
 static inline int lift_ldyp(int r) { return (r + 1) / 2 * 2; }
 
 // Lift from digit planes: F is cut into K-major planes (row-contiguous K = r, padded
-// to 16) one row slab at a time, within kLiftPlaneBudget bytes.
+// to 16) one row slab at a time, within kLiftPlaneBudget bytes and k_lift_planes' grid (65,535
+// blocks of 32 rows in y).
 constexpr size_t kLiftPlaneBudget = (size_t)2 << 30;
+constexpr int64_t kLiftRows = 65535 * 32 / 128 * 128;
 static inline int lift_ldk(int r) { return (r + 15) / 16 * 16; }
 static inline int64_t lift_slab(int64_t N, int r, int D) {
     int64_t S = (int64_t)(kLiftPlaneBudget / ((size_t)2 * D * lift_ldk(r))) / 128 * 128;
-    S = std::max<int64_t>(S, 128);
+    S = std::min<int64_t>(std::max<int64_t>(S, 128), kLiftRows);
     return std::min<int64_t>(S, (N + 127) / 128 * 128);
 }
 

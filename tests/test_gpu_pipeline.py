@@ -183,3 +183,25 @@ def test_fp64_grams_wide_weights(kevd):
     except kevd.KevdError:
         return
     assert not torch.isfinite(A).all()
+
+
+# A slab of the lift is bounded by the grid that cuts its planes (65,535 x 32 rows): at a small rank
+# one more row than that takes two slabs.  The FP64 lift against the FP64-pipe GEMM with the bar of
+# test_tensor_core_lift_matches_fp64_pipe, the FP32 one (three digits, 2^-22 of a row's largest
+# entry in both factors, rank terms) against the same product of its F.
+@pytest.mark.parametrize("dtype", [torch.float64, torch.float32])
+def test_lift_more_rows_than_a_grid(kevd, monkeypatch, dtype):
+    N, r, k = 65535 * 32 + 133, 8, 3
+    g = torch.Generator(device="cuda").manual_seed(3)
+    F = torch.rand(r, N, generator=g, dtype=dtype, device="cuda")
+    d, q, A, C = kevd.bistoch_normalize(F, r)
+    ev, U, kept = kevd.eig_topk(F, r, d, A, C, k)
+    monkeypatch.setenv("KEVD_LIFT", "fp64")
+    ev0, U0, _ = kevd.eig_topk(F.double(), r, d, A, C, k)
+    assert torch.equal(ev, ev0) and kept == r
+    bar = 1e-11 if dtype == torch.float64 else 16 * r * 2.0 ** -22
+    scale = U0.abs().amax(1, keepdim=True)
+    if dtype == torch.float32:      # entries of Y above 1 cancel in U
+        R = torch.linalg.cholesky(A).T
+        scale = torch.linalg.inv(R).abs().max() * F.max().double() / d.min()
+    assert ((U - U0).abs() / scale).max().item() < bar
