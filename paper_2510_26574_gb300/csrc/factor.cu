@@ -1432,9 +1432,10 @@ int rpchol_factor_impl(const void* X, int x_dtype, int64_t N, int32_t d, double 
     size_t need = 0;
     PanelWs pw{};
     OzWs ow{};
-    const bool oz = oz_engine_for(opts, N, b, allow_oz);
-    FactorWs w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b),
-                              pl_engine_for(opts, N, d, r, b, allow_oz));
+    const bool oz = oz_engine_for(opts, N, b, allow_oz), pl = pl_engine_for(opts, N, d, r, b, allow_oz);
+    FactorWs w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b), pl);
+    if (pl && ws_bytes < need)   // no room for the planes: the engine that splits its operands in every round, same bits
+        w = carve_factor(workspace, N, d, r, b, &need, tc, &pw, oz, &ow, factor_rounds(opts, r, b), false);
     if (!workspace || ws_bytes < need || (reinterpret_cast<uintptr_t>(workspace) % kAlign)) return KEVD_EWORKSPACE;
     // the digit planes: X and F (A operands), the pivot panels (B), R and L^-1 of each round
     const unsigned long long* exp_tbl = nullptr;

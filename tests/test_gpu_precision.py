@@ -444,3 +444,35 @@ def test_fp32_grams_more_rows_than_a_grid(kevd):
     assert K.lib().bistoch_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, *map(K._ptr, out), *tail) == K.KEVD_OK
     assert K.lib().symmetric_normalize(K._ptr(F), K.KEVD_F32, N, rank, N, K._ptr(d), K._ptr(A), *tail) == K.KEVD_OK
     assert all(torch.equal(a, b) for a, b in zip(ref + sym, out + [d, A]))
+
+
+# The precision factor without room for the split planes (the last array of its workspace: 16 KB
+# per 128 rows and 32 columns of X and F) runs the engine that splits its operands in every round:
+# the same bits.  A workspace smaller than that is refused.
+@pytest.mark.parametrize("N,d,r,b", [(5000, 64, 256, 64), (3001, 33, 100, 32), (1000, 96, 384, 128)])
+def test_factor_workspace_without_planes_same_bits(kevd, N, d, r, b):
+    import ctypes
+    from paper_2510_26574_gb300 import kevd as K
+    X, eps, _ = make_config("vsa2m", N=N)
+    X = np.concatenate([X, X], 1)[:, :d].astype(np.float32)
+    Xg = torch.from_numpy(np.ascontiguousarray(X)).cuda()
+    ref = kevd.rpchol_factor(Xg, eps, r, b=b, seed=5)
+    o = K.make_opts("arpc", b, 5, precision="bf16x3")
+    full = K.workspace_bytes(K.KEVD_WS_FACTOR, N, d, r, 1, o)
+    small = full - (N + 127) // 128 * ((d + 31) // 32 + (r + 31) // 32) * 16384
+    F = torch.full((r, N), -1.0, device="cuda")
+    piv = torch.zeros(r, dtype=torch.int64, device="cuda")
+    rho = torch.empty(N, dtype=torch.float64, device="cuda")
+    info = K.kevd_factor_info()
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+
+    def call(nbytes):
+        return K.lib().rpchol_factor(K._ptr(Xg), K.KEVD_F32, N, d, eps, r, ctypes.byref(o), K._ptr(F), K.KEVD_F32, N,
+                                     K._ptr(piv), K._ptr(rho), None, ctypes.byref(info), K._ptr(ws), nbytes,
+                                     K._stream(Xg.device))
+    assert call(small - 256) == K.KEVD_EWORKSPACE
+    for nbytes in (small, full - 256, full):
+        F.fill_(-1.0)
+        assert call(nbytes) == K.KEVD_OK
+        assert info.rank == ref["rank"] and torch.equal(piv[:info.rank], ref["pivots"][:info.rank])
+        assert torch.equal(F, ref["F"]) and torch.equal(rho, ref["rho"])
