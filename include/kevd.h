@@ -384,8 +384,8 @@ int kevd_kernel_exp(const double* t, int64_t n, double* out, void* stream);
  * or, with opts->precision = KEVD_PREC_BF16X3, for an FP32 factor, whose Grams keep
  * the slices of one slab (at most 12 GiB; given a workspace without room for them the
  * calls use a slower kernel with the same results).  KEVD_WS_FACTOR with
- * KEVD_PREC_BF16X3 and b >= 32 includes the split operands of X and F (4 bytes per
- * entry, up to 48 GiB); given a workspace that lacks them, rpchol_factor splits both in
+ * KEVD_PREC_BF16X3, b >= 32 and d b <= 3 r^2 includes the split operands of X and F (4 bytes
+ * per entry, up to 48 GiB); given a workspace that lacks them, rpchol_factor splits both in
  * every round, slower and with the same results.
  * Returns 0 for invalid sizes.  The KEVD_WS_EIG and
  * KEVD_WS_LOWMEM_EIG sizes query the eigensolver and therefore need a CUDA

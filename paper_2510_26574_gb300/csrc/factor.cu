@@ -1372,10 +1372,15 @@ static size_t factor_ws_bytes(int64_t N, int d, int r, int b, bool tc, bool oz, 
 // The precision form's engine reads pre-split planes (as large as F) for blocks of b >= 32
 // (a round rewrites the 16-column groups it shares with the last, which smaller blocks would
 // do too often), while they stay within 48 GiB, so that a factor that only just fits the
-// card keeps the engine that needs no copy, and where the caller gives a workspace.
+// card keeps the engine that needs no copy, and where the caller gives a workspace.  The planes of
+// X cost one pass over it, which the rounds have to win back: for d b <= 3 r^2, that is d <= 3 t^2 b
+// with t = r / b rounds.  Whole factor at N = 200,000, planes against splitting in every round (ms):
+// t = 1, b = 64, d = 128 0.51 / 0.54, d = 256 0.72 / 0.67; t = 1, b = 128, d = 256 0.79 / 0.89, d = 512
+// 1.23 / 1.19; t = 2, b = 32, d = 256 0.84 / 0.89, d = 512 1.33 / 1.25; t = 4, b = 64, d = 2,048
+// 5.16 / 6.05.
 static bool pl_engine_for(const kevd_opts* o, int64_t N, int d, int r, int b, bool workspace) {
     int nxh, nH;
-    return workspace && o->precision == KEVD_PREC_BF16X3 && b >= 32 &&
+    return workspace && o->precision == KEVD_PREC_BF16X3 && b >= 32 && (int64_t)d * b <= 3 * (int64_t)r * r &&
            tc_plane_bytes(N, d, r, &nxh, &nH) <= ((size_t)48 << 30);
 }
 

@@ -210,3 +210,16 @@ def test_fp32_gram_slab_within_grid(L, N, rank):
     n = K.workspace_bytes(K.KEVD_WS_NORMALIZE, N, 1, rank, 1, K.make_opts(precision=K.KEVD_PREC_BF16X3))
     nb = (rank + 127) // 128
     assert 0 < n - 24 * N < 65535 * nb * 6 * 16384 + 300_000_000
+
+
+@pytest.mark.parametrize("d,r,b,planes", [(192, 64, 64, True), (193, 64, 64, False), (768, 128, 64, True),
+                                          (769, 128, 64, False), (64, 2048, 31, False)])
+def test_precision_factor_planes_rule(L, d, r, b, planes):
+    """The precision factor's workspace holds the split planes of X and F (16 KB per 128 rows and 32
+    columns of either) for b >= 32 and d b <= 3 r^2: below that the rounds are too few to win back
+    the pass that splits X.  Without them a row takes 8 bytes (|x|^2) and its share of the tile
+    statistics."""
+    n = [K.workspace_bytes(K.KEVD_WS_FACTOR, N, d, r, 1, K.make_opts("arpc", b, 1, precision=K.KEVD_PREC_BF16X3))
+         for N in (128 * 1000, 128 * 2000)]
+    want = 128000 * 8 + 3 * 2000 * 8 + planes * 1000 * ((d + 31) // 32 + (r + 31) // 32) * 16384
+    assert abs(n[1] - n[0] - want) <= 3 * 256                 # the statistics' arrays round up to 256 bytes
