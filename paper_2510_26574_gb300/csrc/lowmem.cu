@@ -209,10 +209,27 @@ __global__ void k_lm_diag(const double* __restrict__ W, int64_t ldw, double* __r
     E[(size_t)c * r + a] = j0 + c <= a ? W[(int64_t)(j0 + c) * ldw + a] : 0.0;
 }
 
+// What the seven digits of the rows of E (r x kLmBlock, exponents ex) leave out, in place: exact.
+__global__ void k_lm_rest(double* __restrict__ E, int r, const int* __restrict__ ex) {
+    const int a = blockIdx.x * blockDim.x + threadIdx.x;
+    if (a >= r) return;
+    const double x = E[(size_t)blockIdx.y * r + a];
+    const int e = ex[a];                                        // -900: no digits
+    E[(size_t)blockIdx.y * r + a] = e <= -900 ? 0.0 : x - ldexp((double)oz_T_f64<kDigits>(x, e), e - 54);
+}
+
 // The unit blocks of the diagonal, kLmBlock columns: E(a, a mod kLmBlock) = 1.
 __global__ void k_lm_unit(double* __restrict__ E, int r) {
     const int a = blockIdx.x * blockDim.x + threadIdx.x;
     if (a < r) E[(size_t)(a % kLmBlock) * r + a] = 1.0;
+}
+
+// C(i, j) = sum_c A(i, c) B(j, c) from seven digit planes, level 7 included: without it rho's error
+// against long double was 5 to 18 % above that of the FP64 library's products, and the rebuilt F's
+// 1.6 to 1.8 times as large; with it 10 to 16 % below and 0.4 to 0.5 times (N = 6,000, r = 256).
+static cudaError_t lm_product(const OzOperand& A, const OzOperand& B, int64_t M, int n, int K, double* C, int64_t ldc,
+                              int* flags, cudaStream_t s) {
+    return launch_ozmm(A, B, M, n, K, nullptr, C, ldc, 0, nullptr, 0, flags, s, kDigits, nullptr, false, true);
 }
 
 // Kp(0:Pc, 0:n) = K(i0:i0+Pc, S_0:S_n) [/ rowdiv]: one DGEMM of the panel's
@@ -225,8 +242,8 @@ static int kernel_panel(cublasHandle_t h, const double* X, int d, int64_t i0, in
         for (int64_t r0 = 0; r0 < Pc; r0 += o->rows) {
             const int64_t rows = std::min(o->rows, Pc - r0);
             KEVD_CUDA_TRY(oz_cut_rowmajor(X + (i0 + r0) * d, rows, d, o->Ap, o->ae, s));
-            KEVD_CUDA_TRY(launch_ozmm(OzOperand{o->Ap, o->nqx, o->ae, 0}, OzOperand{o->XSp, o->nqx, o->xse, 0}, rows, n,
-                                      16 * o->nqx, nullptr, p.Kp + r0, p.P, 0, nullptr, 0, o->flags, s));
+            KEVD_CUDA_TRY(lm_product(OzOperand{o->Ap, o->nqx, o->ae, 0}, OzOperand{o->XSp, o->nqx, o->xse, 0}, rows, n,
+                                     16 * o->nqx, p.Kp + r0, p.P, o->flags, s));
         }
     } else {
         LM_BLAS(cublasDgemm(h, CUBLAS_OP_T, CUBLAS_OP_N, (int)Pc, n, d, &one, X + i0 * d, d, p.XS, d, &zero, p.Kp,
@@ -241,18 +258,24 @@ static int kernel_panel(cublasHandle_t h, const double* X, int d, int64_t i0, in
 // G = R M^-T for nb <= 128 columns of `rows` rows of the panel, in place, from the planes of M
 // and of its explicit inverse: the product with the inverse, corrected once by its residual,
 // without which the error against 64 bits was up to three times that of a triangular solve.
+// The residual takes M whole, `mat` and what its digits leave out (`rest`, 2^-55 of a row's
+// largest entry): that error is the same in every row of F, so the Grams' sums over the rows
+// don't average it out (A's error from the solve alone, emulated for N = 2,000 and ranks 150 and
+// 190: 1.35 and 1.16 times a triangular solve's without the rest, 0.77 and 0.96 times with it).
 static int solve_block(const LmOz& o, double* R, int64_t P, int rows, int nb, const OzOperand& mat,
-                       const OzOperand& inv, cudaStream_t s) {
+                       const OzOperand& rest, const OzOperand& inv, cudaStream_t s) {
     const int nq = (nb + 15) / 16;
     const dim3 grid((rows + 255) / 256, nb);
     const OzOperand A{o.Ap, nq, o.ae, 0};
     KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
-    KEVD_CUDA_TRY(launch_ozmm(A, inv, rows, nb, 16 * nq, nullptr, o.C, o.rows, 0, nullptr, 0, o.flags, s));
+    KEVD_CUDA_TRY(lm_product(A, inv, rows, nb, 16 * nq, o.C, o.rows, o.flags, s));
     KEVD_CUDA_TRY(oz_cut_rows(o.C, o.rows, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
-    KEVD_CUDA_TRY(launch_ozmm(A, mat, rows, nb, 16 * nq, nullptr, o.C2, o.rows, 0, nullptr, 0, o.flags, s));
-    k_lm_sub<<<grid, 256, 0, s>>>(R, P, o.C2, o.rows, rows);
+    for (const OzOperand& m : {mat, rest}) {
+        KEVD_CUDA_TRY(lm_product(A, m, rows, nb, 16 * nq, o.C2, o.rows, o.flags, s));
+        k_lm_sub<<<grid, 256, 0, s>>>(R, P, o.C2, o.rows, rows);
+    }
     KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
-    KEVD_CUDA_TRY(launch_ozmm(A, inv, rows, nb, 16 * nq, nullptr, o.C2, o.rows, 0, nullptr, 0, o.flags, s));
+    KEVD_CUDA_TRY(lm_product(A, inv, rows, nb, 16 * nq, o.C2, o.rows, o.flags, s));
     k_lm_sum<<<grid, 256, 0, s>>>(R, P, o.C, o.C2, o.rows, rows);
     KEVD_LAUNCH_CHECK();
     return KEVD_OK;
@@ -480,8 +503,8 @@ struct LmNormWs {
     // the Grams' planes; o.rows = 0: the library's FP64 products
     LmOz o;
     double* Winv;     // rank x kLmBlock: W's diagonal blocks, then their inverses
-    uint16_t *Wd, *Wp;   // the planes of both
-    int *wde, *we;
+    uint16_t *Wd, *Wr, *Wp;   // the planes of the blocks, of what those leave out, of the inverses
+    int *wde, *wre, *we;
 };
 
 // The products' scratch for `rows` rows, in base (a size with base = NULL).
@@ -529,8 +552,10 @@ static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, bool tc, s
             L.o.xse = c.take<int>(rank);
             L.Winv = c.take<double>((size_t)rank * kLmBlock);
             L.Wd = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
+            L.Wr = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
             L.Wp = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
             L.wde = c.take<int>(rank);
+            L.wre = c.take<int>(rank);
             L.we = c.take<int>(rank);
         }
         L.o.flags = L.flags + 2;
@@ -553,11 +578,13 @@ static int solve_ww(cublasHandle_t h, const double* W, int64_t ldw, int rank, do
     return KEVD_OK;
 }
 
-// The planes of W's diagonal blocks and of their inverses.
+// The planes of W's diagonal blocks, of what those leave out and of the blocks' inverses.
 static int solve_setup(cublasHandle_t h, const double* W, int64_t ldw, int rank, const LmNormWs& L, cudaStream_t s) {
     const double one = 1.0;
     k_lm_diag<<<dim3(grid1(rank), kLmBlock), 256, 0, s>>>(W, ldw, L.Winv, rank);
     KEVD_CUDA_TRY(oz_cut_rows(L.Winv, rank, rank, kLmBlock, kLmBlock / 16, L.Wd, L.wde, L.o.rmax, s));
+    k_lm_rest<<<dim3(grid1(rank), kLmBlock), 256, 0, s>>>(L.Winv, rank, L.wde);
+    KEVD_CUDA_TRY(oz_cut_rows(L.Winv, rank, rank, kLmBlock, kLmBlock / 16, L.Wr, L.wre, L.o.rmax, s));
     KEVD_CUDA_TRY(cudaMemsetAsync(L.Winv, 0, (size_t)rank * kLmBlock * sizeof(double), s));
     k_lm_unit<<<grid1(rank), 256, 0, s>>>(L.Winv, rank);
     KEVD_LAUNCH_CHECK();
@@ -588,15 +615,15 @@ static int solve_panel(const double* W, int64_t ldw, int rank, int64_t Pc, const
             double* R = L.p.Kp + (int64_t)j * P + r0;
             const size_t at = (size_t)(j / kLmBlock) * tile;
             const int st = solve_block(o, R, P, rows, nb, OzOperand{L.Wd + at, nq, L.wde + j, 0},
-                                       OzOperand{L.Wp + at, nq, L.we + j, 0}, s);
+                                       OzOperand{L.Wr + at, nq, L.wre + j, 0}, OzOperand{L.Wp + at, nq, L.we + j, 0}, s);
             if (st != KEVD_OK) return st;
             if (rest == 0) continue;
             KEVD_CUDA_TRY(oz_cut_rows(R, P, rows, nb, nq, o.Ap, o.ae, o.rmax, s));
             for (int c = 0; c < rest; c += kLmBlock) {
                 const int n = std::min(kLmBlock, rest - c);
-                KEVD_CUDA_TRY(launch_ozmm(OzOperand{o.Ap, nq, o.ae, 0},
-                                          OzOperand{o.Bp + (size_t)(c / kLmBlock) * tile, nq, o.be + c, 0}, rows, n,
-                                          kLmBlock, nullptr, o.C, o.rows, 0, nullptr, 0, o.flags, s));
+                KEVD_CUDA_TRY(lm_product(OzOperand{o.Ap, nq, o.ae, 0},
+                                         OzOperand{o.Bp + (size_t)(c / kLmBlock) * tile, nq, o.be + c, 0}, rows, n,
+                                         kLmBlock, o.C, o.rows, o.flags, s));
                 k_lm_sub<<<dim3(grid1(rows), n), 256, 0, s>>>(R + (int64_t)(nb + c) * P, P, o.C, o.rows, rows);
             }
         }
@@ -723,8 +750,8 @@ extern "C" int rpchol_factor_lowmem(const double* X, int64_t N, int32_t d, doubl
                                     R, (int)p.P));
             if (tc) {   // G = R L^-T
                 KEVD_CUDA_TRY(oz_cut_rows(R, p.P, (int)Pc, m, nm, o.Ap, o.ae, o.rmax, s));
-                KEVD_CUDA_TRY(launch_ozmm(OzOperand{o.Ap, nm, o.ae, 0}, OzOperand{q.li.Lp, q.li.ldR / 16, q.li.le, 0},
-                                          Pc, m, 16 * nm, nullptr, R, p.P, 0, nullptr, 0, o.flags, s));
+                KEVD_CUDA_TRY(lm_product(OzOperand{o.Ap, nm, o.ae, 0}, OzOperand{q.li.Lp, q.li.ldR / 16, q.li.le, 0},
+                                         Pc, m, 16 * nm, R, p.P, o.flags, s));
             } else {    // Lc is L row-major (ld b), i.e. L^T column-major
                 LM_BLAS(cublasDtrsm(h, CUBLAS_SIDE_RIGHT, CUBLAS_FILL_MODE_UPPER, CUBLAS_OP_N, CUBLAS_DIAG_NON_UNIT, (int)Pc,
                                     m, &one, w.Lc, b, R, (int)p.P));

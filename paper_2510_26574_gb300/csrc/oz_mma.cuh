@@ -24,6 +24,11 @@
 // for contractions up to 2^15 = kOzNarrowK).  The rest of the kernels' arithmetic is on the
 // integer pipe too: an FP64 operation of any kind costs 17 cycles per warp and SM here.
 //
+// WIDE (seven digits): the six pairs of level 7 that seven digits have join the seventh
+// accumulator.  Without them a product is off by 2^-54 of its operands' largest entries per term,
+// several times what the operands lose in being cut; with them by a third of that.  The low-memory
+// form takes it (lowmem.cu): its products stand where FP64 arithmetic stood.
+//
 // STRICT: levels 5 and 6 in level order, sums in units of 2^-24 with the rest of level 4
 // in the FP32 sum, and one rounding at the end.  It serves contractions beyond
 // kOzNarrowK, and the r x r stage: the subspace iteration stops at a residual of 1e-6,
@@ -69,10 +74,10 @@ constexpr int kOzAccs = D == 3 ? 3 : 7;
 
 // The pairs formed: s + t < D, and (3, 3) beside them for six digits, whose one use is
 // Grams of one operand with itself: of the level 6 terms left out there only d_3 d_3 has
-// a sign on the diagonal (it biased the diagonal of a KS factor's Gram by -1.6e-12).
-template <int D>
+// a sign on the diagonal (it biased the diagonal of a KS factor's Gram by -1.6e-12); WIDE: level 7.
+template <int D, bool WIDE>
 __host__ __device__ constexpr bool oz_pair(int s, int t) {
-    return s + t < D || (D == 6 && s == 3 && t == 3);
+    return s + t < D || (D == 6 && s == 3 && t == 3) || (WIDE && D == 7 && s + t == 7 && s > 0 && t > 0);
 }
 
 // TMEM accumulator of the pair (s, lv - s), and whether it is the accumulator's
@@ -93,7 +98,7 @@ static __device__ __forceinline__ bool mbar_wait_quick(uint32_t bar, uint32_t pa
 
 // Issue state of one CTA (held by the elected lane).  da, db: descriptors of plane 0 of the
 // quarter; pa, pb: plane strides in 16-byte units.
-template <int D, int N, bool STRICT>
+template <int D, int N, bool STRICT, bool WIDE = false>
 struct OzIssuer {
     static constexpr int NA = kOzAccs<D>;
     uint32_t tmem, idesc, pa, pb;
@@ -113,7 +118,7 @@ struct OzIssuer {
                 for (int lv = 0; lv <= D; ++lv)
 #pragma unroll
                     for (int s = 0; s <= lv; ++s)
-                        if (oz_pair<D>(s, lv - s) && oz_acc_of<D>(lv, s) == a)
+                        if (oz_pair<D, WIDE>(s, lv - s) && oz_acc_of<D>(lv, s) == a)
                             umma_bf16(tmem + (uint32_t)(N * a), da + (uint64_t)(s * pa), db + (uint64_t)((lv - s) * pb),
                                       idesc, (start && oz_lead(lv, s)) ? 0u : 1u);
                 if (end) umma_commit(acc_full + 8u * a);
@@ -126,7 +131,7 @@ struct OzIssuer {
         for (int s = 0; s < D; ++s) {
 #pragma unroll
             for (int t = 0; t < D; ++t) {
-                if (!oz_pair<D>(s, t) || (STRICT && s + t > 4)) continue;
+                if (!oz_pair<D, WIDE>(s, t) || (STRICT && s + t > 4)) continue;
                 const uint32_t d = tmem + (uint32_t)(N * oz_acc_of<D>(s + t, s));
                 const uint64_t pda = da + (uint64_t)(s * pa), pdb = db + (uint64_t)(t * pb);
                 if (t == 0) umma_bf16_col<true>(d, pda, pdb, idesc, 1u);

@@ -45,11 +45,12 @@ struct OzOperand {
 // of pout_nq quarters (zeros up to st->kp plus st->m rounded up to 16; pout 32-byte
 // aligned, st->kp a multiple of 16).
 // digits: 7 (FP64 operands) or 3 (FP32 operands: T = round(x 2^(22 - E)), the
-// three pairs of levels 0-2); rowdiv != NULL divides row i of C by rowdiv[i]; strict:
-// see oz_mma.cuh.
+// three pairs of levels 0-2); rowdiv != NULL divides row i of C by rowdiv[i]; strict, wide
+// (seven digits; strict goes before): see oz_mma.cuh.
 cudaError_t launch_ozmm(const OzOperand& A, const OzOperand& B, int64_t M, int n, int K, const FactorState* st,
                         double* C, int64_t ldc, int64_t c_koff, uint16_t* pout, int pout_nq, int* flags,
-                        cudaStream_t s, int digits = 7, const double* rowdiv = nullptr, bool strict = false);
+                        cudaStream_t s, int digits = 7, const double* rowdiv = nullptr, bool strict = false,
+                        bool wide = false);
 
 // Operands of launch_ozmm cut from FP64 matrices, seven digits, one exponent per operand row
 // (ex), zero past the K columns.  The rows of a row-major N x K matrix (factor.cu) ...

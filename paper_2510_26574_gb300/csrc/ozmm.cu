@@ -69,9 +69,9 @@ struct OzCfg {
     static_assert(D * kN <= (int)kCols, "TMEM");
 };
 
-// D digits (levels 0 .. D - 1 of the pairs s + t <= D - 1; D = 3 or 7).  rowdiv:
+// D digits (levels 0 .. D - 1 of the pairs s + t <= D - 1; D = 3 or 7; WIDE: level 7 too).  rowdiv:
 // C(i, :) is divided by rowdiv[i] (one reciprocal per row), when not NULL.
-template <int D, bool STRICT>
+template <int D, bool STRICT, bool WIDE>
 __global__ void __launch_bounds__(kThreads, 1)
     k_ozmm(const OzOperand A, const OzOperand B, int64_t M, int n, int K, const FactorState* __restrict__ st,
            double* __restrict__ Cout, int64_t ldc, int64_t c_koff, uint16_t* __restrict__ pout, int pout_nq,
@@ -185,7 +185,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else if (wid == 1) {
         // ---- MMA issuer: one elected lane ----
         if (elect_one()) {
-            OzIssuer<D, kN, STRICT> is{tmem, kIdesc, kPlaneA >> 4, kPlaneB >> 4, acc_full(0), acc_empty(0), &s_fail};
+            OzIssuer<D, kN, STRICT, WIDE> is{tmem, kIdesc, kPlaneA >> 4, kPlaneB >> 4, acc_full(0), acc_empty(0), &s_fail};
             int st_ = 0, prev = -1;
             uint32_t ph = 0, prev_ph = 0;
             bool ok = true;
@@ -283,23 +283,23 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 }  // namespace
 
-template <int D, bool STRICT>
+template <int D, bool STRICT, bool WIDE = false>
 static cudaError_t launch_ozmm_d(const OzOperand& A, const OzOperand& B, int64_t M, int n, int K,
                                  const FactorState* st, double* C, int64_t ldc, int64_t c_koff, uint16_t* pout,
                                  int pout_nq, const double* rowdiv, int* flags, int sms, cudaStream_t s) {
-    cudaError_t e = cudaFuncSetAttribute(k_ozmm<D, STRICT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(k_ozmm<D, STRICT, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)OzCfg<D>::kSmem);
     if (e != cudaSuccess) return e;
     const int64_t ntile = (M + kM - 1) / kM * ((n + OzCfg<D>::kN - 1) / OzCfg<D>::kN);
     const dim3 grid((unsigned)std::min<int64_t>(ntile, sms));   // persistent: one CTA per SM
-    k_ozmm<D, STRICT><<<grid, kThreads, OzCfg<D>::kSmem, s>>>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv,
-                                                              flags);
+    k_ozmm<D, STRICT, WIDE><<<grid, kThreads, OzCfg<D>::kSmem, s>>>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq,
+                                                                    rowdiv, flags);
     return cudaGetLastError();
 }
 
 cudaError_t launch_ozmm(const OzOperand& A, const OzOperand& B, int64_t M, int n, int K, const FactorState* st,
                         double* C, int64_t ldc, int64_t c_koff, uint16_t* pout, int pout_nq, int* flags,
-                        cudaStream_t s, int digits, const double* rowdiv, bool strict) {
+                        cudaStream_t s, int digits, const double* rowdiv, bool strict, bool wide) {
     if (M < 1 || n < 1 || M >= ((int64_t)1 << 31) || (digits != 3 && digits != kDigits)) return cudaErrorInvalidValue;
     if (!A.p || !B.p || (reinterpret_cast<uintptr_t>(A.p) % 16) || (reinterpret_cast<uintptr_t>(B.p) % 16) ||
         (pout && (digits != kDigits || (reinterpret_cast<uintptr_t>(pout) % 32))))
@@ -317,8 +317,9 @@ cudaError_t launch_ozmm(const OzOperand& A, const OzOperand& B, int64_t M, int n
     if (digits == 3)
         return strict ? launch_ozmm_d<3, true>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s)
                       : launch_ozmm_d<3, false>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s);
-    return strict
-               ? launch_ozmm_d<kDigits, true>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s)
+    if (strict) return launch_ozmm_d<kDigits, true>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s);
+    return wide
+               ? launch_ozmm_d<kDigits, false, true>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s)
                : launch_ozmm_d<kDigits, false>(A, B, M, n, K, st, C, ldc, c_koff, pout, pout_nq, rowdiv, flags, sms, s);
 }
 

@@ -243,3 +243,52 @@ def test_fullsize_ks200k_matches_stored_F_path(kevd):
     ev, U, _ = kevd.eig_topk_lowmem(Xg, eps, out["pivots"], out["W"], rk, dt, A, C, 64)
     assert torch.max(torch.abs(ev - ev_f) / ev_f.abs()).item() < 1e-10
     assert U.shape == (64, N)
+
+
+def _longdouble(X, eps, S, rows):
+    """W (the Cholesky factor of K(S,S)) and F(rows,:) = K(rows,S) W^-T in long double."""
+    X = X.astype(np.longdouble)
+    n = len(S)
+    K = np.stack([np.exp(-((X[np.r_[S, rows]] - X[s]) ** 2).sum(1) / np.longdouble(eps)) for s in S], 1)
+    for j in range(n):
+        K[j + 1:n, j + 1:] -= np.outer(K[j + 1:n, j], K[j + 1:n, j]) / K[j, j]
+        K[j:n, j] /= np.sqrt(K[j, j])
+    W, F = np.tril(K[:n]), K[n:]
+    for j in range(n):
+        F[:, j] /= W[j, j]
+        F[:, j + 1:] -= np.outer(F[:, j], W[j + 1:, j])
+    return W, F
+
+
+# The tensor-core products may not cost digits against the library's FP64 ones (KEVD_ENGINE=fp64):
+# errors against long double, on the same pivots.  rho, which 1 - |F(i,:)|^2 cancels to 1e-3 and below,
+# from 300 rows: no larger.  A and C carry W's own error, which both forms share and which the other roundings
+# move by a few per cent: within 1.05 times, from a factor of two 128-column blocks.
+@pytest.mark.parametrize("seed", [1, 2])
+def test_products_as_accurate_as_fp64(kevd, monkeypatch, seed):
+    def errors(N, r, b, rows):
+        X, eps, _ = make_config("ks200k", N=N)
+        Xg = _gpu(X)
+        o = kevd.rpchol_factor_lowmem(Xg, eps, r, b=b, seed=seed)
+        d, q, A, C = (t.cpu().numpy() for t in kevd.bistoch_normalize_lowmem(Xg, eps, o["pivots"], o["W"], o["rank"]))
+        S = o["pivots"][:o["rank"]].cpu().numpy()
+        if N not in ref:
+            ref[N] = S, _longdouble(X, eps, S, rows)[1]
+        assert np.array_equal(S, ref[N][0])
+        F = ref[N][1]
+        rho = np.linalg.norm((o["rho"].cpu().numpy()[rows] - np.maximum(1 - (F * F).sum(1), 0)).astype(float))
+        if len(rows) < N:
+            return rho
+        dl = F @ F.sum(0)
+        ql = F @ (F / dl[:, None]).sum(0)
+        A0, C0 = (F / dl[:, None]).T @ (F / dl[:, None]), (F / ql[:, None]).T @ F
+        return np.linalg.norm((A - A0).astype(float)), np.linalg.norm((C - C0).astype(float))
+
+    ref = {}
+    big = 8000, 256, 64, np.arange(0, 8000, 27)
+    small = 1100, 200, 100, np.arange(1100)
+    got = errors(*big), *errors(*small)
+    monkeypatch.setenv("KEVD_ENGINE", "fp64")
+    want = errors(*big), *errors(*small)
+    print(got, want)
+    assert got[0] <= want[0] and got[1] <= 1.05 * want[1] and got[2] <= 1.05 * want[2]
