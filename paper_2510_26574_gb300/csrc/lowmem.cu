@@ -550,7 +550,7 @@ static LmNormWs carve_lm_norm(void* base, int64_t N, int d, int rank, bool tc, s
             L.o.rows = rows;
             L.o.XSp = c.take<uint16_t>(oz_tile_elems(rank, L.o.nqx, kDigits));
             L.o.xse = c.take<int>(rank);
-            L.Winv = c.take<double>((size_t)rank * kLmBlock);
+            L.Winv = rows >= rank ? L.o.C : c.take<double>((size_t)rank * kLmBlock);   // (read before the first product)
             L.Wd = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
             L.Wr = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
             L.Wp = c.take<uint16_t>(oz_tile_elems(rank, kLmBlock / 16, kDigits));
