@@ -445,8 +445,13 @@ static LmFactorWs carve_lm_factor(void* base, int64_t N, int d, int r, int b, si
 // max(d, 128) bytes a row beside the panel's 8 r).  K(p,S) Z stays with the library's FP64
 // GEMM: Z's entries reach far above 1, and digits cut by the largest entry of a row left rho
 // with 1.4 times the GEMM's error against 64 bits.  For blocks from 32 on (the FP64 path's line:
-// below, a block leaves most of a 128-row tile of the right operand empty) and from 1,024
-// rows on; otherwise the library's FP64 products and solves serve.
+// below, a block leaves most of a 128-row tile of the right operand empty), from 1,024
+// rows on and for N r >= 7 2^18, where the factor costs more than the launches that a round adds
+// (whole factor, d = 64, b = 32, these products / the library's, ms: N r = 1.0 2^20: N = 16,000
+// 1.05 / 0.83, 8,000 1.84 / 1.65, 4,000 4.42 / 4.04; 1.95 2^20: 30,000 1.18 / 1.30, 16,000 2.01 / 2.21,
+// 8,000 4.61 / 5.27, b = 64 at 4,000 8.12 / 8.23); otherwise the library's FP64 products and
+// solves serve.
+constexpr int64_t kLmOzWork = (int64_t)7 << 18;
 struct LmRound {
     LmPanel p;     // Kp and P of the rows formed at a time
     LmOz o;
@@ -468,7 +473,7 @@ static size_t carve_lm_round(Carver& c, LmRound& q, int64_t rows, int d, int r, 
     return c.off;
 }
 static bool lm_round(const LmPanel& p, int64_t N, int d, int r, int b, LmRound* q) {
-    if (b < 32 || !oz_engine_enabled()) return false;
+    if (b < 32 || N * r < kLmOzWork || !oz_engine_enabled()) return false;
     const size_t bytes = (size_t)p.P * r * sizeof(double);
     q->p = p;
     int64_t lo = 0, hi = std::min<int64_t>(p.P, (N + 127) / 128 * 128) / 128;   // in tiles of 128 rows

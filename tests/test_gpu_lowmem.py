@@ -292,3 +292,20 @@ def test_products_as_accurate_as_fp64(kevd, monkeypatch, seed):
     want = errors(*big), *errors(*small)
     print(got, want)
     assert got[0] <= want[0] and got[1] <= 1.05 * want[1] and got[2] <= 1.05 * want[2]
+
+
+# The factor's products past the line of their rule (N r >= 7 2^18): few wide panels, many pivots in
+# panels of a part of the rows, the largest and a ragged block.  Bars as
+# test_products_tensor_core_and_library.
+@pytest.mark.parametrize("N,r,b", [(57345, 32, 32), (15001, 128, 100), (4000, 480, 128)])
+def test_factor_products_past_their_line(kevd, monkeypatch, N, r, b):
+    X, eps, _ = make_config("ks200k", N=N)
+    Xg = _gpu(X)
+    out = kevd.rpchol_factor_lowmem(Xg, eps, r, b=b, seed=3)
+    monkeypatch.setenv("KEVD_ENGINE", "fp64")
+    ref = kevd.rpchol_factor_lowmem(Xg, eps, r, b=b, seed=3)
+    rk = ref["rank"]
+    assert out["rank"] == rk and torch.equal(out["pivots"][:rk], ref["pivots"][:rk])
+    assert not torch.equal(out["rho"], ref["rho"])            # another route
+    assert torch.max(torch.abs(out["W"] - ref["W"])) < 1e-10
+    assert torch.max(torch.abs(out["rho"] - ref["rho"])) < 1e-10
