@@ -25,6 +25,7 @@
 #include "kexp.cuh"
 #include "oz_digits.cuh"
 #include "ozgemm.cuh"
+#include "rej_root.cuh"
 #include "trace.cuh"
 
 namespace kevd {
@@ -451,24 +452,6 @@ struct RejShared {
     int tpos[128];
     int m;
 };
-
-// s = sqrt(h) and y = 1 / sqrt(h) for normal h: Halley's iteration on a reciprocal-root
-// estimate (relative error below 2^-22, cubed), then one correction of s = h y by its exact
-// residual (P. Markstein, IBM J. Res. Dev. 34(1), 1990).
-__device__ __forceinline__ void rej_root(double h, double& s, double& y) {
-    double y0;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(h));
-    const double e = fma(-(h * y0), y0, 1.0);
-    y = fma(fma(e, 0.375, 0.5), y0 * e, y0);
-    const double s0 = h * y;
-    s = fma(fma(-s0, s0, h), 0.5 * y, s0);
-}
-
-// c / s, y = 1 / s up to rounding: the quotient corrected by its exact residual (as above).
-__device__ __forceinline__ double rej_quot(double c, double s, double y) {
-    const double q = c * y;
-    return fma(fma(-q, s, c), y, q);
-}
 
 // One cluster of kRejCluster CTAs per problem, `cta` the rank in it.  H is overwritten.
 __device__ __forceinline__ void arpc_reject_body(FactorWs w, int b, int r, uint64_t seed, int rnd,
