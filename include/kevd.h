@@ -145,12 +145,14 @@ typedef struct kevd_factor_info {
  * rpchol_factor -- pivoted partial Cholesky of the implicit Gaussian kernel
  * matrix (Section 1.2; Appendix A, Algorithms 2 and 3; kernel of Eq.
  * (data-kernel) with the delay factor J folded into eps).
- * With KEVD_PREC_FP64 the engine's products X X(S,:)^T and F F(S,:)^T run on
- * the tensor cores at FP64 accuracy (six-digit BF16 slices summed exactly),
- * when X's rows have an even length, ldf is even and X, F are 16-byte
- * aligned; otherwise, or with KEVD_ENGINE=fp64 in the environment, on the FP64
- * pipe.  Both agree to rounding (1e-10 in F); kevd_workspace_bytes must be
- * queried under the same environment.
+ * With KEVD_PREC_FP64, KEVD_ARPC, b >= 32 and N < 2^31 the engine's products
+ * X X(S,:)^T and F F(S,:)^T and its solve run on the tensor cores at FP64
+ * accuracy (seven-digit BF16 planes, the leading levels summed exactly),
+ * whatever the layout of X and F; otherwise, or with KEVD_ENGINE=fp64 in the
+ * environment, on the FP64 pipe.  Both agree to rounding (1e-10 in F);
+ * kevd_workspace_bytes must be queried under the same environment.  Greedy FP64
+ * rounds of up to 65,536 rows run in one launch, all of whose time the tracer
+ * counts as KEVD_STAGE_ENGINE.
  *
  *   X         device, N x d row-major, element type x_dtype (KEVD_F64 for
  *             KEVD_PREC_FP64, KEVD_F32 for KEVD_PREC_BF16X3).
@@ -178,7 +180,8 @@ typedef struct kevd_factor_info {
  * (or falls to opts->tol * N).
  * Errors: KEVD_EINVAL (bad argument, or a non-finite coordinate in X, reported
  * after the factorisation ran), KEVD_EWORKSPACE, KEVD_ECUDA, KEVD_ETIMEOUT
- * (precision form: a tensor-core pipeline wait gave up; outputs unspecified).
+ * (a bounded wait of a tensor-core pipeline, or of the barrier between greedy
+ * rounds in one launch, gave up; outputs unspecified).
  */
 int rpchol_factor(const void* X, int x_dtype, int64_t N, int32_t d, double eps, int32_t r,
                   const kevd_opts* opts, void* F, int f_dtype, int64_t ldf,

@@ -332,7 +332,9 @@ __global__ void __launch_bounds__(kGtThreads, 1)
 // N = 2M, rank 1,848, both Grams with the cut and the column maxima: 48.1 ms (k_gram_tc:
 // 79.5 ms).
 // ---------------------------------------------------------------------------
-constexpr size_t kGpBudget = (size_t)12 << 30;      // bytes of slices per slab
+// Bytes of slices per slab: at N = 2M, rank 1,848 one of the five splits takes 8.6 GiB (48 ms;
+// with 6 GiB it would not fit and k_gram_tc's 80 ms return, 24 GiB give nothing more).
+constexpr size_t kGpBudget = (size_t)12 << 30;
 constexpr uint32_t kGpTile = 128 * 128;             // one tile: 128 columns x 64 rows of BF16
 constexpr int kGpChunk = 16;                        // stages per exact chunk: 1,024 rows
 constexpr int kGpThreads = 10 * 32;

@@ -604,7 +604,7 @@ static int solve_setup(cublasHandle_t h, const double* W, int64_t ldw, int rank,
 
 // F_p = K(p,S) W^-T in place on the tensor cores, 128 columns at a time: F_J = R_J W_JJ^-T with
 // the block's explicit inverse, then R(:, > J) -= F_J W(> J, J)^T.  Exponents are per row, so
-// that W may be of any scale.  Measured at N = 60,000, rank 356: 7.0 ms of the Gram
+// that W may be of any scale.  Measured at N = 60,000, rank 356: 7.6 ms of the Gram
 // stage, 18.5 with the library's triangular solve.
 static int solve_panel(const double* W, int64_t ldw, int rank, int64_t Pc, const LmNormWs& L, cudaStream_t s) {
     const LmOz& o = L.o;
